@@ -86,6 +86,24 @@ double norm_quantile(double p) {
     return x;
 }
 
+// The quantiles behind the weight and delay codes, z_c = Phi^-1((c + 1/2) / M):
+// constants of the method, evaluated once per process.  A table build needs
+// 64 x 128 + 8 x 256 of them; evaluating each there (0.04 us and up, erfc and
+// exp per Halley step) took 0.45 ms of every call that makes tables
+// (snn_set_params, snn_step_noalloc, the gradient's base weights).
+struct CodeQuantiles {
+    double w[kWCodes], d[kDCodes];
+    CodeQuantiles() {
+        for (int k = 0; k < kWCodes; ++k) w[k] = norm_quantile(((double)k + 0.5) / (double)kWCodes);
+        for (int k = 0; k < kDCodes; ++k) d[k] = norm_quantile(((double)k + 0.5) / (double)kDCodes);
+    }
+};
+
+const CodeQuantiles& code_quantiles() {
+    static const CodeQuantiles q;       // thread-safe initialisation
+    return q;
+}
+
 void poisson_thresholds(double lam, uint64_t* thr) {
     double term = std::exp(-lam);
     double cdf = term;
@@ -125,21 +143,51 @@ int validate(const snn_config* c) {
     return SNN_OK;
 }
 
+// the constants of the neurons and the background: propagators, DC input,
+// Poisson thresholds, background weight, refractory steps
+void make_constants(snn_net* net) {
+    const snn_config* c = &net->cfg;
+    const int np = c->n_pop;
+    for (int p = 0; p < kMaxPop; ++p) {
+        const double lam = p < np ? c->nu_bg * c->k_ext[p] * (c->dt / 1000.0) : 0.0;
+        poisson_thresholds(lam, net->pois[p]);
+    }
+    const double P22 = std::exp(-c->dt / c->tau_m);
+    const double P11 = std::exp(-c->dt / c->tau_syn);
+    const double P21 = (c->tau_m * c->tau_syn) / (c->c_m * (c->tau_m - c->tau_syn)) * (P22 - P11);
+    const double P20 = c->tau_m / c->c_m * (1.0 - P22);
+    net->prop[0] = (float)P22;
+    net->prop[1] = (float)P21;
+    net->prop[2] = (float)P11;
+    net->prop[3] = (float)P20;
+    for (int p = 0; p < kMaxPop; ++p) net->cdc[p] = p < np ? (float)(P20 * c->i_dc[p]) : 0.f;
+    net->wext_q = (int32_t)std::llround(c->w_ext * 256.0);
+    net->n_ref = (int32_t)std::llround(c->t_ref / c->dt);
+}
+
+// weight of code k of a projection, 1/256 pA, before rounding; false outside
+// the fixed-point range
+bool code_weight(const snn_config* c, int p, int q, double z, double* qv) {
+    double w = c->w_mean[p][q] + c->w_sd[p][q] * z;
+    w = w * c->w_scale;
+    w = w * c->proj_scale[p][q];
+    *qv = w * 256.0;
+    return std::fabs(*qv) < 1073741824.0;
+}
+
+int weight_range_error() { return fail(SNN_ERR_INVALID, "weight outside the fixed-point range"); }
+
 int make_tables(snn_net* net) {
     const snn_config* c = &net->cfg;
     const int np = c->n_pop;
+    const CodeQuantiles& z = code_quantiles();
     for (int p = 0; p < kMaxPop; ++p)
         for (int q = 0; q < kMaxPop; ++q) {
             for (int k = 0; k < kWCodes; ++k) {
                 int32_t v = 0;
                 if (p < np && q < np) {
-                    const double z = norm_quantile(((double)k + 0.5) / (double)kWCodes);
-                    double w = c->w_mean[p][q] + c->w_sd[p][q] * z;
-                    w = w * c->w_scale;
-                    w = w * c->proj_scale[p][q];
-                    const double qv = w * 256.0;
-                    if (!(std::fabs(qv) < 1073741824.0))
-                        return fail(SNN_ERR_INVALID, "weight outside the fixed-point range");
+                    double qv;
+                    if (!code_weight(c, p, q, z.w[k], &qv)) return weight_range_error();
                     v = (int32_t)std::llround(qv);
                 }
                 net->wtab[(p * kMaxPop + q) * kWCodes + k] = v;
@@ -156,29 +204,14 @@ int make_tables(snn_net* net) {
         for (int k = 0; k < kDCodes; ++k) {
             int dl = 1;
             if (q < np) {
-                const double z = norm_quantile(((double)k + 0.5) / (double)kDCodes);
-                const double steps = (c->d_mean[q] + c->d_sd[q] * z) / c->dt;
+                const double steps = (c->d_mean[q] + c->d_sd[q] * z.d[k]) / c->dt;
                 double r = std::round(steps);
                 r = std::min(std::max(r, 1.0), (double)(kRing - 1));
                 dl = (int)r;
             }
             net->dtab[q * kDCodes + k] = (uint8_t)dl;
         }
-    for (int p = 0; p < kMaxPop; ++p) {
-        const double lam = p < np ? c->nu_bg * c->k_ext[p] * (c->dt / 1000.0) : 0.0;
-        poisson_thresholds(lam, net->pois[p]);
-    }
-    const double P22 = std::exp(-c->dt / c->tau_m);
-    const double P11 = std::exp(-c->dt / c->tau_syn);
-    const double P21 = (c->tau_m * c->tau_syn) / (c->c_m * (c->tau_m - c->tau_syn)) * (P22 - P11);
-    const double P20 = c->tau_m / c->c_m * (1.0 - P22);
-    net->prop[0] = (float)P22;
-    net->prop[1] = (float)P21;
-    net->prop[2] = (float)P11;
-    net->prop[3] = (float)P20;
-    for (int p = 0; p < kMaxPop; ++p) net->cdc[p] = p < np ? (float)(P20 * c->i_dc[p]) : 0.f;
-    net->wext_q = (int32_t)std::llround(c->w_ext * 256.0);
-    net->n_ref = (int32_t)std::llround(c->t_ref / c->dt);
+    make_constants(net);
     return SNN_OK;
 }
 
@@ -471,7 +504,16 @@ int host_step_constants(const snn_config* cfg, float prop[4], float cdc[kMaxPop]
     CALL(validate(cfg));
     static thread_local snn_net tmp;   // table workspace reused by this thread
     tmp.cfg = *cfg;
-    CALL(make_tables(&tmp));
+    // the weights themselves come with the caller's rows: only their range is
+    // checked, at the extreme codes, between which the others lie
+    const CodeQuantiles& z = code_quantiles();
+    for (int p = 0; p < cfg->n_pop; ++p)
+        for (int q = 0; q < cfg->n_pop; ++q)
+            for (int k : {0, kWCodes - 1}) {
+                double qv;
+                if (!code_weight(cfg, p, q, z.w[k], &qv)) return weight_range_error();
+            }
+    make_constants(&tmp);
     for (int k = 0; k < 4; ++k) prop[k] = tmp.prop[k];
     for (int p = 0; p < kMaxPop; ++p) {
         cdc[p] = tmp.cdc[p];
@@ -610,14 +652,12 @@ int net_make_tables(snn_net* net) { return make_tables(net); }
 // unrounded weight of every code at projection scale 1, in pA
 void net_base_weights(const snn_net* net, float* wb) {
     const snn_config* c = &net->cfg;
+    const CodeQuantiles& z = code_quantiles();
     for (int p = 0; p < kMaxPop; ++p)
         for (int q = 0; q < kMaxPop; ++q)
             for (int k = 0; k < kWCodes; ++k) {
                 double w = 0.0;
-                if (p < c->n_pop && q < c->n_pop) {
-                    const double z = norm_quantile(((double)k + 0.5) / (double)kWCodes);
-                    w = (c->w_mean[p][q] + c->w_sd[p][q] * z) * c->w_scale;
-                }
+                if (p < c->n_pop && q < c->n_pop) w = (c->w_mean[p][q] + c->w_sd[p][q] * z.w[k]) * c->w_scale;
                 wb[(p * kMaxPop + q) * kWCodes + k] = (float)w;
             }
 }
