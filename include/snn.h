@@ -228,7 +228,7 @@ int snn_sync(snn_net* net);
 /*
  * snn_read_spikes -- drain the recorded spikes (Sec. 3.1.2: output spike
  * times of all neurons are recorded) into steps_host[cap], ids_host[cap];
- * *n receives the count copied.  Order is unspecified (sort if needed).
+ * *n receives the count copied.  The spikes come in ascending (step, id) order.
  * Synchronises the stream.  SNN_ERR_OVERFLOW if spikes were lost on the
  * device or cap is too small (the first cap are returned).
  */
@@ -485,8 +485,8 @@ int snn_batch_step(snn_batch* b, int64_t n_steps);
 int snn_batch_sync(snn_batch* b);
 
 /* snn_batch_read_spikes -- drain the spikes of instance k recorded since the
- * last read of that instance: (step, local neuron id) in device order (not
- * sorted).  Synchronises.  n receives the number written (<= cap). */
+ * last read of that instance: (step, local neuron id), in ascending order.
+ * Synchronises.  n receives the number written (<= cap). */
 int snn_batch_read_spikes(snn_batch* b, int32_t k, uint32_t* steps_host, uint32_t* ids_host,
                           int64_t cap, int64_t* n);
 

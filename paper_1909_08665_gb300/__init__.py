@@ -279,9 +279,7 @@ class Microcircuit:
         n = C.c_int64()
         _check(lib().snn_read_spikes(self._h, _ptr(st, C.c_uint32), _ptr(ids, C.c_uint32),
                                      int(cap), C.byref(n)))
-        st, ids = st[:n.value], ids[:n.value]
-        order = np.lexsort((ids, st))
-        return st[order].astype(np.int64), ids[order].astype(np.int64)
+        return st[:n.value].astype(np.int64), ids[:n.value].astype(np.int64)
 
     def raster_size(self) -> int:
         n = C.c_int64()
@@ -289,7 +287,8 @@ class Microcircuit:
         return n.value
 
     def read_spikes_into(self, steps_buf: np.ndarray, ids_buf: np.ndarray) -> int:
-        """Drain the raster into caller-provided uint32 host buffers (unsorted)."""
+        """Drain the raster into caller-provided uint32 host buffers, in
+        ascending (step, id) order."""
         n = C.c_int64()
         _check(lib().snn_read_spikes(self._h, _ptr(steps_buf, C.c_uint32),
                                      _ptr(ids_buf, C.c_uint32), int(steps_buf.size),
@@ -448,13 +447,11 @@ class MicrocircuitBatch:
         st = np.zeros(cap, np.uint32)
         ids = np.zeros(cap, np.uint32)
         n = self.read_spikes_into(k, st, ids)
-        st, ids = st[:n], ids[:n]
-        order = np.lexsort((ids, st))
-        return st[order].astype(np.int64), ids[order].astype(np.int64)
+        return st[:n].astype(np.int64), ids[:n].astype(np.int64)
 
     def read_spikes_into(self, k: int, steps_buf: np.ndarray, ids_buf: np.ndarray) -> int:
         """Drain instance k's spikes into caller-provided uint32 host buffers
-        (ids relative to the instance, in recording order, not sorted)."""
+        (ids relative to the instance), in ascending (step, id) order."""
         n = C.c_int64()
         _check(lib().snn_batch_read_spikes(self._h, int(k), _ptr(steps_buf, C.c_uint32),
                                            _ptr(ids_buf, C.c_uint32), int(steps_buf.size),

@@ -633,7 +633,9 @@ struct snn_batch {
     bool graph_ok = false;
     long long step = 0;
     std::vector<std::vector<uint32_t>> host_steps, host_ids;   // drained raster per instance
-    std::vector<uint16_t> inst_of;  // instance of every global neuron id (built on the first drain)
+    RasterSort ras_sort;                 // workspace of the raster reads
+    long long ras_lo = 0;                // first step since the last drain
+    bool ras_new = false;                // steps were issued since the last drain
     std::vector<float2> u0_range;        // default initial potentials per instance
     float trial_us = 0.f;                // per-step time of the chosen assignment
 };
@@ -672,6 +674,7 @@ void free_batch(snn_batch* b) {
                     b->d_ras_n, b->d_ic, b->d_step, b->d_sync};
     for (void* x : ptrs)
         if (x) cudaFree(x);
+    raster_sort_free(&b->ras_sort);
     delete b;
 }
 
@@ -835,34 +838,36 @@ int batch_trials(snn_batch* b) {
     return SNN_OK;
 }
 
+// the spikes recorded since the last drain, sorted by (instance, step, id) on
+// the device, appended to each instance's host arrays
 int drain_raster(snn_batch* b) {
     BCK(cudaStreamSynchronize(b->stream));
+    if (!b->ras_new) return SNN_OK;             // no step issued since: nothing recorded
     uint32_t n = 0;
     BCK(cudaMemcpy(&n, b->d_ras_n, sizeof(n), cudaMemcpyDeviceToHost));
     const uint32_t m = std::min(n, b->ras_cap);
     std::vector<uint32_t> st(m), id(m);
     if (m) {
-        BCK(cudaMemcpy(st.data(), b->d_ras_step, sizeof(uint32_t) * m, cudaMemcpyDeviceToHost));
-        BCK(cudaMemcpy(id.data(), b->d_ras_id, sizeof(uint32_t) * m, cudaMemcpyDeviceToHost));
+        const RasterList in = {b->d_ras_n, b->d_ras_step, b->d_ras_id, b->ras_cap, 1, b->n_inst, b->d_goff,
+                               (uint32_t)b->ras_lo, b->step - b->ras_lo, (uint32_t)b->ntot};
+        BCK(raster_sort(&b->ras_sort, in, m, b->stream));
+        BCK(cudaMemcpyAsync(st.data(), b->ras_sort.step, sizeof(uint32_t) * m, cudaMemcpyDeviceToHost, b->stream));
+        BCK(cudaMemcpyAsync(id.data(), b->ras_sort.id, sizeof(uint32_t) * m, cudaMemcpyDeviceToHost, b->stream));
     }
-    BCK(cudaMemset(b->d_ras_n, 0, sizeof(uint32_t)));
-    if (b->inst_of.empty()) {
-        b->inst_of.resize((size_t)b->ntot);
-        for (int k = 0; k < b->n_inst; ++k)
-            std::fill(b->inst_of.begin() + b->goff[k], b->inst_of.begin() + b->goff[k + 1],
-                      (uint16_t)k);
-    }
-    // per-instance counts first, so that each instance's buffers grow once
-    std::vector<uint32_t> cnt((size_t)b->n_inst, 0u);
-    for (uint32_t r = 0; r < m; ++r) ++cnt[b->inst_of[id[r]]];
-    for (int k = 0; k < b->n_inst; ++k) {
-        b->host_steps[k].reserve(b->host_steps[k].size() + cnt[k]);
-        b->host_ids[k].reserve(b->host_ids[k].size() + cnt[k]);
-    }
-    for (uint32_t r = 0; r < m; ++r) {
-        const int k = b->inst_of[id[r]];
-        b->host_steps[k].push_back(st[r]);
-        b->host_ids[k].push_back(id[r] - (uint32_t)b->goff[k]);
+    BCK(cudaMemsetAsync(b->d_ras_n, 0, sizeof(uint32_t), b->stream));
+    BCK(cudaStreamSynchronize(b->stream));
+    b->ras_new = false;
+    b->ras_lo = b->step;
+    for (uint32_t r = 0, k = 0; r < m; ++k) {
+        const uint32_t lo = (uint32_t)b->goff[k], hi = (uint32_t)b->goff[k + 1];
+        const uint32_t e = (uint32_t)(std::partition_point(id.begin() + r, id.end(), [&](uint32_t x) { return x < hi; }) -
+                                      id.begin());
+        b->host_steps[k].insert(b->host_steps[k].end(), st.begin() + r, st.begin() + e);
+        auto& out = b->host_ids[k];
+        const size_t at = out.size();
+        out.insert(out.end(), id.begin() + r, id.begin() + e);
+        for (size_t i = at; i < out.size(); ++i) out[i] -= lo;
+        r = e;
     }
     if (n > b->ras_cap) return set_error(SNN_ERR_OVERFLOW, "batch raster capacity exceeded");
     return SNN_OK;
@@ -1124,6 +1129,7 @@ int snn_batch_create(const snn_config* cfgs, const uint64_t* seeds, int32_t n_in
 int snn_batch_step(snn_batch* b, int64_t n_steps) {
     if (!b || n_steps < 0) return set_error(SNN_ERR_INVALID, "bad arguments");
     int64_t left = n_steps;
+    if (left > 0) b->ras_new = true;
     while (left > 0) {
         if (b->graph_ok && left >= kGraphChunk) {
             BCK(cudaGraphLaunch(b->graph, b->stream));

@@ -219,10 +219,11 @@ void free_net(snn_net* net) {
     if (!net) return;
     void* ptrs[] = {net->d_part_lo, net->d_row_start, net->d_seg, net->d_words, net->d_pre, net->d_wtab,
                     net->d_dtab, net->d_u, net->d_i, net->d_r, net->d_ring, net->d_msg, net->d_wrap,
-                    net->d_ras_step, net->d_ras_id, net->d_ras_n, net->d_rs_step, net->d_rs_id,
-                    net->d_counters, net->d_sync, net->d_pop_spikes, net->d_rt};
+                    net->d_ras_step, net->d_ras_id, net->d_ras_n, net->d_counters,
+                    net->d_sync, net->d_pop_spikes, net->d_rt};
     for (void* p : ptrs)
         if (p) cudaFree(p);
+    raster_sort_free(&net->ras_sort);
     free_grad(net->grad);
     delete net;
 }
@@ -634,6 +635,10 @@ void fill_step_params(const snn_net* net, StepParams* out) {
 cudaError_t net_launch(snn_net* net, StepParams& sp, int64_t t0, int64_t n) {
     const int64_t kMaxLaunch = 1ll << 24;
     int64_t left = n, t = t0;
+    if (n > 0) {
+        net->ras_lo = std::min(net->ras_lo, t0);
+        net->ras_hi = std::max(net->ras_hi, t0 + n);
+    }
     while (left > 0) {
         const int64_t chunk = std::min(left, kMaxLaunch);
         sp.t0 = t;
@@ -842,30 +847,23 @@ int snn_read_spikes(snn_net* net, uint32_t* steps_host, uint32_t* ids_host, int6
         if (cnt[c] > net->ras_cap) lost = true;
         total += std::min<uint32_t>(cnt[c], net->ras_cap);
     }
-    // the first `cap` entries in partition order, packed on the device and
-    // copied back in one transfer per array
+    // sorted on the device, the first `cap` copied back, one transfer per array
     const int64_t got = std::min<int64_t>(total, cap);
     if (got > 0 && (steps_host || ids_host)) {
-        if (net->rs_cap < (size_t)got) {
-            cudaFree(net->d_rs_step);
-            cudaFree(net->d_rs_id);
-            net->d_rs_step = net->d_rs_id = nullptr;
-            net->rs_cap = 0;
-            CALL(dalloc(&net->d_rs_step, (size_t)got, "raster staging"));
-            CALL(dalloc(&net->d_rs_id, (size_t)got, "raster staging"));
-            net->rs_cap = (size_t)got;
-        }
-        CK(launch_pack_raster(net->d_ras_n, net->P, net->ras_cap, got, net->d_ras_step,
-                              net->d_ras_id, net->d_rs_step, net->d_rs_id, net->stream));
+        const RasterList in = {net->d_ras_n, net->d_ras_step, net->d_ras_id, net->ras_cap, net->P, 1, nullptr,
+                               (uint32_t)net->ras_lo, net->ras_hi - net->ras_lo, (uint32_t)net->n};
+        CK(raster_sort(&net->ras_sort, in, (size_t)total, net->stream));
         if (steps_host)
-            CK(cudaMemcpyAsync(steps_host, net->d_rs_step, sizeof(uint32_t) * got,
+            CK(cudaMemcpyAsync(steps_host, net->ras_sort.step, sizeof(uint32_t) * got,
                                cudaMemcpyDeviceToHost, net->stream));
         if (ids_host)
-            CK(cudaMemcpyAsync(ids_host, net->d_rs_id, sizeof(uint32_t) * got,
+            CK(cudaMemcpyAsync(ids_host, net->ras_sort.id, sizeof(uint32_t) * got,
                                cudaMemcpyDeviceToHost, net->stream));
     }
     CK(cudaMemsetAsync(net->d_ras_n, 0, sizeof(uint32_t) * net->P, net->stream));
     CK(cudaStreamSynchronize(net->stream));
+    net->ras_lo = INT64_MAX;
+    net->ras_hi = 0;
     *n = got;
     if (lost) return fail(SNN_ERR_OVERFLOW, "spike raster capacity exceeded; spikes were lost");
     if (got < total) return fail(SNN_ERR_OVERFLOW, "cap smaller than the recorded spikes; the rest were dropped");

@@ -256,11 +256,32 @@ long long input_bound(const uint32_t* indeg, int n, int n_pop, const int32_t* po
 // out[c] = longest (row, partition c) segment, for every partition c
 cudaError_t launch_max_segment(const uint32_t* seg, int n, int n_part, uint32_t* out,
                                cudaStream_t s);
-// the raster entries of every partition (counts clamped to cap_part, then the
-// first `limit` entries in partition order) packed into step_out / id_out
-cudaError_t launch_pack_raster(const uint32_t* counts, int n_part, uint32_t cap_part,
-                               int64_t limit, const uint32_t* ras_step, const uint32_t* ras_id,
-                               uint32_t* step_out, uint32_t* id_out, cudaStream_t s);
+// Recorded spikes of n_part lists (device: counts, which may exceed cap_part,
+// and [n_part][cap_part] steps and ids) sorted into w->step / w->id by
+// (instance, step, id); n is the sum of the counts, clamped.  Every step lies
+// in [t_lo, t_lo + t_span) modulo 2^32, every id below n_ids; goff (device,
+// [n_inst + 1]) gives the instances' id ranges when there are several.
+// The arrays of w grow as needed and are kept (raster_sort_free).
+struct RasterList {
+    const uint32_t* counts;
+    const uint32_t* step;
+    const uint32_t* id;
+    uint32_t cap_part;
+    int32_t n_part, n_inst;
+    const int32_t* goff;
+    uint32_t t_lo;
+    long long t_span;
+    uint32_t n_ids;
+};
+struct RasterSort {
+    uint32_t* step = nullptr;
+    uint32_t* id = nullptr;
+    uint32_t* group = nullptr;
+    unsigned long long* key = nullptr;
+    size_t step_cap = 0, id_cap = 0, group_cap = 0, key_cap = 0;
+};
+cudaError_t raster_sort(RasterSort* w, const RasterList& in, size_t n, cudaStream_t s);
+void raster_sort_free(RasterSort* w);
 cudaError_t launch_init_state(int n, uint32_t key0, uint32_t key1, float lo, float hi,
                               float* u, cudaStream_t s);
 int step_kernel_variant(int npt, bool smem_ring);
