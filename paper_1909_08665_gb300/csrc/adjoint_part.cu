@@ -47,6 +47,8 @@ constexpr uint32_t kApOffMask = (1u << kApWBits) - 1u;
 constexpr uint32_t kApChunk = 32;           // entries per lane before a run is split
 constexpr uint32_t kApMaxChunks = 4;         // lanes one source's run is split over
 constexpr int kApPre = 4;                    // neurons per thread in the membrane phase (ncmax <= 2048)
+constexpr int kApPart = 16;                  // partials of a neuron in flight
+constexpr int kApFlags = 2;                  // spike flags per thread in flight
 constexpr int kApHeader = 8;                 // n_lg, nc, p_lo, span, e_off, 0, 0, 0
 // header, then for the entries of delay >= 2 ("far") lenmax[n_lg] and
 // ebase[n_lg], for those of delay 1 ("near") lenmax[n_lg] and ebase[n_lg],
@@ -80,6 +82,10 @@ k_adjoint_part(const __grid_constant__ AdjPartParams p) {
     double* s_gN = reinterpret_cast<double*>(
         (reinterpret_cast<uintptr_t>(s_far + (size_t)p.max_lg * 32) + 7) & ~uintptr_t(7));
     uint8_t* s_mn = reinterpret_cast<uint8_t*>(s_gN + ncmax);
+    // spike flags of the lanes' sources, of two steps: loaded a step ahead, so
+    // that no walk waits for them
+    uint8_t* s_spk = s_mn + ncmax;               // [2][max_lg * 32]
+    const uint32_t spk_row = (uint32_t)p.max_lg * 32u;
 
     if (tid == 0) s_abort = 0u;
     {
@@ -131,14 +137,15 @@ k_adjoint_part(const __grid_constant__ AdjPartParams p) {
     // source's chunks and writes its partial.  Spiking sources' weight
     // partials go to gAc after each walk.
     auto walk = [&](int64_t tt, uint32_t tDt, bool far) {
-        const uint8_t* flt = p.tr_f + (size_t)(tt - p.t_first) * n;
+        const uint8_t* spk_t = s_spk + (size_t)(tt & 1) * spk_row;
         const uint32_t base_t = tDt * ws;
         for (uint32_t wl = warp_first[warp]; wl < warp_first[warp + 1]; ++wl) {
             const uint32_t L = lg_order[wl];
             const uint32_t j = srcs[L * 32 + lane];
             const uint32_t lm = far ? lenmax[L] : lenmax_n[L];
             const uint32_t eb = far ? ebase[L] : ebase_n[L];
-            const bool spk = j != kApNone && (flt[j] & 1u) != 0u;
+            const bool spk = spk_t[L * 32 + lane] != 0u;
+            const bool any_spk = __any_sync(0xffffffffu, spk);
             float acc = 0.f;
             float pa[kMaxPop];
 #pragma unroll
@@ -146,19 +153,29 @@ k_adjoint_part(const __grid_constant__ AdjPartParams p) {
             const uint32_t* ep = ent + eb + lane;
             // entry: weight index << 19 | delay * ws + target; the window
             // cell of step tt + delay is that offset plus tt's row, wrapped
+            // (a - RW is huge where a < RW).  Few lane groups hold a spiking
+            // source: the others walk without the test.
+            if (!any_spk) {
+#pragma unroll 8
+                for (uint32_t k = 0; k < lm; ++k) {
+                    const uint32_t e = ep[k * 32];
+                    const uint32_t a = base_t + (e & kApOffMask);
+                    acc = __fadd_rn(acc, __fmul_rn(wf[e >> kApWBits], win[min(a, a - RW)]));
+                }
+            } else {
 #pragma unroll 4
-            for (uint32_t k = 0; k < lm; ++k) {
-                const uint32_t e = ep[k * 32];
-                const uint32_t wi = e >> kApWBits;
-                uint32_t a = base_t + (e & kApOffMask);
-                a -= a >= RW ? RW : 0u;
-                const float lv = win[a];
-                acc = __fadd_rn(acc, __fmul_rn(wf[wi], lv));
-                if (spk) {
-                    const float v = __fmul_rn(wb[wi], lv);
-                    const uint32_t pr = wi / (kMaxPop * kWCodes);
+                for (uint32_t k = 0; k < lm; ++k) {
+                    const uint32_t e = ep[k * 32];
+                    const uint32_t wi = e >> kApWBits;
+                    const uint32_t a = base_t + (e & kApOffMask);
+                    const float lv = win[min(a, a - RW)];
+                    acc = __fadd_rn(acc, __fmul_rn(wf[wi], lv));
+                    if (spk) {
+                        const float v = __fmul_rn(wb[wi], lv);
+                        const uint32_t pr = wi / (kMaxPop * kWCodes);
 #pragma unroll
-                    for (int kk = 0; kk < kMaxPop; ++kk) pa[kk] = __fadd_rn(pa[kk], kk == (int)pr ? v : 0.f);
+                        for (int kk = 0; kk < kMaxPop; ++kk) pa[kk] = __fadd_rn(pa[kk], kk == (int)pr ? v : 0.f);
+                    }
                 }
             }
             // the chunks of a source sit in consecutive lanes; its first lane
@@ -179,7 +196,7 @@ k_adjoint_part(const __grid_constant__ AdjPartParams p) {
                     __stcg(&pds[(size_t)c * n + j], tot);
                 }
             }
-            if (__any_sync(0xffffffffu, spk)) {
+            if (any_spk) {
 #pragma unroll
                 for (int kk = 0; kk < kMaxPop; ++kk) {
                     float t2 = pa[kk];
@@ -194,7 +211,7 @@ k_adjoint_part(const __grid_constant__ AdjPartParams p) {
                     double* ga = p.gAc + ((size_t)c * n + j) * kMaxPop;
 #pragma unroll
                     for (int kk = 0; kk < kMaxPop; ++kk)
-                        if ((uint32_t)kk < span) ga[kk] += (double)pa[kk];
+                        if ((uint32_t)kk < span) atomicAdd(&ga[kk], (double)pa[kk]);   // nothing waits for it
                 }
             }
         }
@@ -228,6 +245,16 @@ k_adjoint_part(const __grid_constant__ AdjPartParams p) {
         return s_abort == 0u;
     };
 
+    // spike flag of lane slot k (lane group k / 32) in trace row `row`
+    auto flag_of = [&](uint32_t k, int row) -> uint8_t {
+        const uint32_t j = srcs[k];
+        return j != kApNone ? (uint8_t)(__ldg(p.tr_f + (size_t)row * n + j) & 1u) : (uint8_t)0;
+    };
+    for (uint32_t k = tid; k < 32u * n_lg; k += kApThreads) {
+        s_spk[(size_t)(t_top & 1) * spk_row + k] = flag_of(k, p.len - 1);
+        if (p.len > 1) s_spk[(size_t)((t_top - 1) & 1) * spk_row + k] = flag_of(k, p.len - 2);
+    }
+    __syncthreads();
     uint32_t tD = (uint32_t)(t_top % R);      // window slot of step t
     // step t_top's gather, both parts, before the first barrier
     walk(t_top, tD, true);
@@ -248,8 +275,27 @@ k_adjoint_part(const __grid_constant__ AdjPartParams p) {
             u_pre[k] = i < nc ? ut[lo + i] : 0.f;
             f_pre[k] = i < nc ? fl[lo + i] : (uint8_t)0;
         }
+        // the spike flags of step t - 2, into step t's place: its walks are done
+        uint8_t nf[kApFlags];
+        if (s > 1) {
+#pragma unroll
+            for (int k = 0; k < kApFlags; ++k) {
+                const uint32_t i = (uint32_t)tid + (uint32_t)k * kApThreads;
+                nf[k] = i < 32u * n_lg ? flag_of(i, s - 2) : (uint8_t)0;
+            }
+        }
         // the far part of step t - 1's gather while the other CTAs arrive
         if (s > 0) walk(t - 1, tD1, true);
+        if (s > 1) {
+            uint8_t* row = s_spk + (size_t)(t & 1) * spk_row;
+#pragma unroll
+            for (int k = 0; k < kApFlags; ++k) {
+                const uint32_t i = (uint32_t)tid + (uint32_t)k * kApThreads;
+                if (i < 32u * n_lg) row[i] = nf[k];
+            }
+            for (uint32_t i = (uint32_t)tid + kApFlags * kApThreads; i < 32u * n_lg; i += kApThreads)
+                row[i] = flag_of(i, s - 2);
+        }
         if (!wait()) break;
         // ---- membrane and current adjoints of partition c's neurons ----
         float* pds_all = p.pds + (size_t)(t & 1) * p.n_part * n;
@@ -258,8 +304,17 @@ k_adjoint_part(const __grid_constant__ AdjPartParams p) {
             const uint32_t i = (uint32_t)tid + (uint32_t)kp * kApThreads;
             if (i >= nc) break;
             const int32_t gi = lo + (int32_t)i;
+            // the partials of the partitions, kApPart in flight, added in order
             float acc = 0.f;
-            for (int cc = 0; cc < p.n_part; ++cc) acc = __fadd_rn(acc, __ldcg(&pds_all[(size_t)cc * n + gi]));
+            for (int c0 = 0; c0 < p.n_part; c0 += kApPart) {
+                float v[kApPart];
+#pragma unroll
+                for (int r = 0; r < kApPart; ++r)
+                    v[r] = c0 + r < p.n_part ? __ldcg(&pds_all[(size_t)(c0 + r) * n + gi]) : 0.f;
+#pragma unroll
+                for (int r = 0; r < kApPart; ++r)
+                    if (c0 + r < p.n_part) acc = __fadd_rn(acc, v[r]);
+            }
             const float ds = __fadd_rn(p.gs[pop_index(p.pop_start, p.n_pop, gi)], acc);
             const uint8_t f = f_pre[kp];
             const bool mn = s_mn[i] != 0u;
@@ -515,7 +570,8 @@ int adjoint_part_plan(int n, int n_pop, const int32_t* pop_start, int n_part, co
     }
     const size_t ws = ((size_t)ncmax + 31) / 32 * 32;
     const size_t smem = img_max * 4 + (size_t)R * ws * 4 + (size_t)2 * (span_max * kMaxPop * kWCodes + 4) * 4 +
-                        (size_t)ncmax * 8 + (size_t)max_lg * 32 * 4 + 8 + (size_t)ncmax * 8 + (size_t)ncmax;
+                        (size_t)ncmax * 8 + (size_t)max_lg * 32 * 4 + 8 + (size_t)ncmax * 8 + (size_t)ncmax +
+                        (size_t)max_lg * 64;
     if (smem > (size_t)optin) return 1;
     plan->grid = n_part * G;
     plan->groups = G;
@@ -549,6 +605,10 @@ void adjoint_part_free(AdjPartPlan* plan) {
 }
 
 cudaError_t launch_adjoint_part(const AdjPartPlan& plan, AdjPartParams& ap, cudaStream_t s) {
+    // the attribute is the kernel's, not the plan's: another network's plan may
+    // have set it lower
+    cudaError_t e = cudaFuncSetAttribute(k_adjoint_part, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)plan.smem);
+    if (e != cudaSuccess) return e;
     ap.groups = plan.groups;
     ap.ring_r = plan.ring_r;
     ap.span_max = plan.span_max;
