@@ -2,10 +2,21 @@
 // Sec. 2.1 Eq. 1 run backwards) with its row gather done partition by
 // partition, for networks whose rows fit in the SMs' shared memory.
 //
-// The gather of step t is ds_j = gs + sum over row j of (w / 256) lI_{i,t+d}.
-// Only its delay-1 entries need step t + 1's lI; the rest ("far", delay >= 2)
-// is computed while the grid barrier of step t + 1 completes (a split
-// barrier: arrive, far gather of step t, wait), the near part after it.
+// The gather of step t is ds_j = gs + sum over row j of (w / 256) lI_{i,t+d},
+// d >= 1, and lI_t = P11 lI_{t+1} + m_{t+1} P21 lu_{t+1}: the gather of step
+// t - 1 needs lu_{t+1} and so the partials of step t + 1, but not those of
+// step t.  A CTA therefore gathers step t - 1 while the grid barrier of step
+// t's partials completes, watched by a warp of its own, and only then adds
+// them up into lu_t.  It writes step t - 1's partials over step t + 1's after
+// that barrier, which every CTA reached after it had read the latter.  The
+// entries of delay 1 ("near") are walked after the others ("far") and
+// cover the round trip of the partials.  Measured on the 10 % network, us per
+// step (backward of 2000 recorded steps): 7.5 with the wait before the
+// membrane adjoint and all it needs, 6.4 with the spike flags and partials
+// fetched ahead, 5.8 in this order.  What bounds it now: the shared-memory
+// wavefronts of the far walk (2.3 us: entry 1, weight and window 2.3 each on
+// random banks), then the round trip of freshly written partials (1 us).
+//
 // Gathered from a global lI ring, it costs one L2 request per synapse and
 // step.  Here the targets are split into the network's partitions and the
 // sources of each partition into G groups: CTA (c, g) keeps, for the whole
@@ -41,6 +52,7 @@ namespace {
 
 constexpr int kApThreads = 512;
 constexpr int kApWarps = kApThreads / 32;
+constexpr int kApLaunch = kApThreads + 32;   // and the warp that watches the grid barrier
 constexpr uint32_t kApNone = 0xffffffffu;
 constexpr uint32_t kApWBits = 19;            // weight index << 19 | window cell offset
 constexpr uint32_t kApOffMask = (1u << kApWBits) - 1u;
@@ -55,7 +67,50 @@ constexpr int kApHeader = 8;                 // n_lg, nc, p_lo, span, e_off, 0, 
 // src[32 n_lg], chunks[32 n_lg] (m on a source's first lane, else 0),
 // warp_first[kApWarps + 1], lg_order[n_lg], then the entries at e_off
 
-__global__ void __launch_bounds__(kApThreads, 1)
+// the chunks of a source added in order, on its first lane (m chunks, else 0)
+__device__ __forceinline__ float add_chunks(float v, uint32_t m) {
+    float tot = v;
+#pragma unroll
+    for (uint32_t r = 1; r < kApMaxChunks; ++r) {
+        const float w = __shfl_down_sync(0xffffffffu, v, r);
+        if (r < m) tot = __fadd_rn(tot, w);
+    }
+    return tot;
+}
+
+// The walk of a lane group with a spiking source: its sum as in the plain
+// walk, and the spiking lanes' weight partials, one per target population of
+// the partition, added into ga.  A CTA with such a group is the last to
+// arrive, and nearly every step has some: with PW = 8 sums an entry costs 35
+// instructions, with the 2 that a partition usually spans 17, without 9.
+template <int PW>
+__device__ __forceinline__ void walk_spiking(const uint32_t* ep, uint32_t lm, uint32_t base_t, uint32_t RW,
+                                             const float* win, const float* wf, const float* wb, bool spk,
+                                             uint32_t m, double* ga, uint32_t span, float& acc) {
+    float pa[PW];
+#pragma unroll
+    for (int k = 0; k < PW; ++k) pa[k] = 0.f;
+#pragma unroll 4
+    for (uint32_t k = 0; k < lm; ++k) {
+        const uint32_t e = ep[k * 32];
+        const uint32_t wi = e >> kApWBits;
+        const uint32_t a = base_t + (e & kApOffMask);
+        const float lv = win[min(a, a - RW)];
+        acc = __fadd_rn(acc, __fmul_rn(wf[wi], lv));
+        // (lanes without a spike drop their sums)
+        const float v = __fmul_rn(wb[wi], lv);
+        const uint32_t pr = wi / (kMaxPop * kWCodes);
+#pragma unroll
+        for (int kk = 0; kk < PW; ++kk) pa[kk] = __fadd_rn(pa[kk], kk == (int)pr ? v : 0.f);
+    }
+#pragma unroll
+    for (int kk = 0; kk < PW; ++kk) {
+        const float t2 = add_chunks(pa[kk], m);
+        if (m > 0u && spk && (uint32_t)kk < span) atomicAdd(&ga[kk], (double)t2);   // nothing waits for it
+    }
+}
+
+__global__ void __launch_bounds__(kApLaunch, 1)
 k_adjoint_part(const __grid_constant__ AdjPartParams p) {
     extern __shared__ __align__(16) uint32_t s_img[];
     __shared__ volatile uint32_t s_abort;
@@ -92,7 +147,7 @@ k_adjoint_part(const __grid_constant__ AdjPartParams p) {
         const uint32_t o0 = p.img_off[blockIdx.x], words = p.img_off[blockIdx.x + 1] - o0;
         const uint4* src = reinterpret_cast<const uint4*>(p.img + o0);   // offsets are multiples of 4
         uint4* dst = reinterpret_cast<uint4*>(s_img);
-        for (uint32_t k = tid; k < words / 4; k += kApThreads) dst[k] = __ldg(&src[k]);
+        for (uint32_t k = tid; k < words / 4; k += kApLaunch) dst[k] = __ldg(&src[k]);
     }
     __syncthreads();
     const uint32_t n_lg = s_img[0], nc = s_img[1], p_lo = s_img[2], span = s_img[3];
@@ -106,7 +161,7 @@ k_adjoint_part(const __grid_constant__ AdjPartParams p) {
     const uint32_t* lg_order = warp_first + kApWarps + 1;
     const uint32_t* ent = s_img + s_img[4];
     const int32_t lo = p.part_lo[c];
-    for (uint32_t k = tid; k < span * kMaxPop * kWCodes; k += kApThreads) {
+    for (uint32_t k = tid; k < span * kMaxPop * kWCodes; k += kApLaunch) {
         const uint32_t gk = p_lo * kMaxPop * kWCodes + k;
         wf[k] = __fmul_rn(__int2float_rn(__ldg(&p.wtab[gk])), 0.00390625f);
         wb[k] = __ldg(&p.wbase[gk]);
@@ -115,7 +170,7 @@ k_adjoint_part(const __grid_constant__ AdjPartParams p) {
         wf[w_zero + tid] = 0.f;
         wb[w_zero + tid] = 0.f;
     }
-    for (uint32_t i = tid; i < nc; i += kApThreads) {
+    for (uint32_t i = tid; i < nc; i += kApLaunch) {
         s_lu[i] = p.lu[lo + i];
         s_lI[i] = p.lI[lo + i];
         s_mn[i] = p.mnext[lo + i];
@@ -123,7 +178,7 @@ k_adjoint_part(const __grid_constant__ AdjPartParams p) {
     }
     // the window of the first step processed, t_top: lI of steps t_top + d
     const int64_t t_top = p.t_first + p.len - 1;
-    for (uint32_t k = tid; k < (R - 1) * nc; k += kApThreads) {
+    for (uint32_t k = tid; k < (R - 1) * nc; k += kApLaunch) {
         const uint32_t d = 1 + k / nc, i = k - (d - 1) * nc;
         const int64_t tt = t_top + d;
         win[(uint32_t)(tt % R) * ws + i] = __ldcg(&p.lring[(size_t)(tt & (kRing - 1)) * n + lo + i]);
@@ -131,9 +186,8 @@ k_adjoint_part(const __grid_constant__ AdjPartParams p) {
     __syncthreads();
 
     const uint32_t RW = R * ws;               // window words
-    // The gather of step tt, far (delay >= 2: window steps tt + 2 .. , all
-    // final before step tt + 1's membrane phase) or near (delay 1: step tt +
-    // 1).  The far sums wait in s_far; the near walk adds them, combines a
+    // The gather of step tt, far (delay >= 2) or near (delay 1: window step
+    // tt + 1).  The far sums wait in s_far; the near walk adds them, combines a
     // source's chunks and writes its partial.  Spiking sources' weight
     // partials go to gAc after each walk.
     auto walk = [&](int64_t tt, uint32_t tDt, bool far) {
@@ -144,147 +198,158 @@ k_adjoint_part(const __grid_constant__ AdjPartParams p) {
             const uint32_t j = srcs[L * 32 + lane];
             const uint32_t lm = far ? lenmax[L] : lenmax_n[L];
             const uint32_t eb = far ? ebase[L] : ebase_n[L];
-            const bool spk = spk_t[L * 32 + lane] != 0u;
-            const bool any_spk = __any_sync(0xffffffffu, spk);
-            float acc = 0.f;
-            float pa[kMaxPop];
-#pragma unroll
-            for (int k = 0; k < kMaxPop; ++k) pa[k] = 0.f;
+            const bool spk = (spk_t[L * 32 + lane] & 1u) != 0u;
+            const uint32_t m = lens[L * 32 + lane];
             const uint32_t* ep = ent + eb + lane;
+            float acc = 0.f;
             // entry: weight index << 19 | delay * ws + target; the window
             // cell of step tt + delay is that offset plus tt's row, wrapped
             // (a - RW is huge where a < RW).  Few lane groups hold a spiking
-            // source: the others walk without the test.
-            if (!any_spk) {
+            // source: the others walk without its weight partials.
+            if (!__any_sync(0xffffffffu, spk)) {
 #pragma unroll 8
                 for (uint32_t k = 0; k < lm; ++k) {
                     const uint32_t e = ep[k * 32];
                     const uint32_t a = base_t + (e & kApOffMask);
                     acc = __fadd_rn(acc, __fmul_rn(wf[e >> kApWBits], win[min(a, a - RW)]));
                 }
+            } else if (span <= 2u) {
+                walk_spiking<2>(ep, lm, base_t, RW, win, wf, wb, spk, m,
+                                p.gAc + ((size_t)c * n + (spk ? j : 0u)) * kMaxPop, span, acc);
             } else {
-#pragma unroll 4
-                for (uint32_t k = 0; k < lm; ++k) {
-                    const uint32_t e = ep[k * 32];
-                    const uint32_t wi = e >> kApWBits;
-                    const uint32_t a = base_t + (e & kApOffMask);
-                    const float lv = win[min(a, a - RW)];
-                    acc = __fadd_rn(acc, __fmul_rn(wf[wi], lv));
-                    if (spk) {
-                        const float v = __fmul_rn(wb[wi], lv);
-                        const uint32_t pr = wi / (kMaxPop * kWCodes);
-#pragma unroll
-                        for (int kk = 0; kk < kMaxPop; ++kk) pa[kk] = __fadd_rn(pa[kk], kk == (int)pr ? v : 0.f);
-                    }
-                }
+                walk_spiking<kMaxPop>(ep, lm, base_t, RW, win, wf, wb, spk, m,
+                                      p.gAc + ((size_t)c * n + (spk ? j : 0u)) * kMaxPop, span, acc);
             }
             // the chunks of a source sit in consecutive lanes; its first lane
             // (m > 0) adds them in chunk order
-            const uint32_t m = lens[L * 32 + lane];
             if (far) {
                 s_far[L * 32 + lane] = acc;
             } else {
                 acc = __fadd_rn(s_far[L * 32 + lane], acc);
-                float tot = acc;
-#pragma unroll
-                for (uint32_t r = 1; r < kApMaxChunks; ++r) {
-                    const float v = __shfl_down_sync(0xffffffffu, acc, r);
-                    if (r < m) tot = __fadd_rn(tot, v);
-                }
+                const float tot = add_chunks(acc, m);
                 if (m > 0u) {
                     float* pds = p.pds + (size_t)(tt & 1) * p.n_part * n;
                     __stcg(&pds[(size_t)c * n + j], tot);
                 }
             }
-            if (any_spk) {
-#pragma unroll
-                for (int kk = 0; kk < kMaxPop; ++kk) {
-                    float t2 = pa[kk];
-#pragma unroll
-                    for (uint32_t r = 1; r < kApMaxChunks; ++r) {
-                        const float v = __shfl_down_sync(0xffffffffu, pa[kk], r);
-                        if (r < m) t2 = __fadd_rn(t2, v);
-                    }
-                    pa[kk] = t2;
-                }
-                if (m > 0u && spk) {
-                    double* ga = p.gAc + ((size_t)c * n + j) * kMaxPop;
-#pragma unroll
-                    for (int kk = 0; kk < kMaxPop; ++kk)
-                        if ((uint32_t)kk < span) atomicAdd(&ga[kk], (double)pa[kk]);   // nothing waits for it
-                }
-            }
         }
     };
-    // split grid barrier: every CTA arrives once its partials are written,
-    // does the next step's far gather, then waits
-    uint32_t gen = 0;
+    // Grid barrier k: the partials of step t_top - k are written.  The last
+    // warp watches it while the others gather.
     auto arrive = [&]() {
         __syncthreads();
-        if (tid == 0) red_release_gpu_add(p.barrier, 1u);
+        // the watching warp waits for the partials' writes, no gathering one
+        if (tid == kApThreads) red_release_gpu_add(p.barrier, 1u);
     };
-    auto wait = [&]() -> bool {
-        if (tid == 0) {
-            const uint32_t target = (gen + 1u) * gridDim.x;
-            const uint64_t t_start = globaltimer_ns();
-            uint32_t iter = 0;
-            while (ld_acquire_gpu(p.barrier) < target) {
-                if ((++iter & 255u) == 0u) {
-                    if (ld_relaxed_gpu(p.abort_flag) != 0u) { s_abort = 1u; break; }
-                    if (globaltimer_ns() - t_start > p.timeout_ns) {
-                        atomicOr(p.status, kStatusTimeout);
-                        atomicExch(p.abort_flag, 1u);
-                        s_abort = 1u;
-                        break;
-                    }
+    auto watch = [&](int k) {
+        const uint32_t target = ((uint32_t)k + 1u) * gridDim.x;
+        const uint64_t t_start = globaltimer_ns();
+        uint32_t iter = 0;
+        while (ld_acquire_gpu(p.barrier) < target) {
+            if ((++iter & 255u) == 0u) {
+                if (ld_relaxed_gpu(p.abort_flag) != 0u) { s_abort = 1u; break; }
+                if (globaltimer_ns() - t_start > p.timeout_ns) {
+                    atomicOr(p.status, kStatusTimeout);
+                    atomicExch(p.abort_flag, 1u);
+                    s_abort = 1u;
+                    break;
                 }
             }
         }
-        __syncthreads();
-        ++gen;
-        return s_abort == 0u;
     };
 
     // spike flag of lane slot k (lane group k / 32) in trace row `row`
+    uint32_t my_src[kApFlags];
+#pragma unroll
+    for (int k = 0; k < kApFlags; ++k) {
+        const uint32_t i = (uint32_t)tid + (uint32_t)k * kApThreads;
+        my_src[k] = i < 32u * n_lg ? srcs[i] : kApNone;
+    }
     auto flag_of = [&](uint32_t k, int row) -> uint8_t {
         const uint32_t j = srcs[k];
-        return j != kApNone ? (uint8_t)(__ldg(p.tr_f + (size_t)row * n + j) & 1u) : (uint8_t)0;
+        uint8_t f = 0;
+        if (j != kApNone) f = __ldg(p.tr_f + (size_t)row * n + j);
+        return f;
     };
-    for (uint32_t k = tid; k < 32u * n_lg; k += kApThreads) {
+    // the trace of the partition's neurons in row `row`
+    float u_pre[kApPre];
+    uint8_t f_pre[kApPre];
+    auto load_trace = [&](int row) {
+#pragma unroll
+        for (int k = 0; k < kApPre; ++k) {
+            const uint32_t i = (uint32_t)tid + (uint32_t)k * kApThreads;
+            u_pre[k] = 0.f;
+            f_pre[k] = 0;
+            if (tid < kApThreads && i < nc) {
+                u_pre[k] = __ldg(p.tr_u + (size_t)row * n + lo + i);
+                f_pre[k] = __ldg(p.tr_f + (size_t)row * n + lo + i);
+            }
+        }
+    };
+    load_trace(p.len - 1);
+    for (uint32_t k = tid; k < 32u * n_lg; k += kApLaunch) {
         s_spk[(size_t)(t_top & 1) * spk_row + k] = flag_of(k, p.len - 1);
         if (p.len > 1) s_spk[(size_t)((t_top - 1) & 1) * spk_row + k] = flag_of(k, p.len - 2);
     }
     __syncthreads();
     uint32_t tD = (uint32_t)(t_top % R);      // window slot of step t
     // step t_top's gather, both parts, before the first barrier
-    walk(t_top, tD, true);
-    __syncwarp();
-    walk(t_top, tD, false);
+    if (warp < kApWarps) {
+        walk(t_top, tD, true);
+        __syncwarp();
+        walk(t_top, tD, false);
+    }
     arrive();
+    // Step t: lI_t follows from lu_{t+1}; with it the gather of step t - 1 is
+    // done while the partials of step t come in, and lu_t last of all.
     for (int s = p.len - 1; s >= 0; --s) {
         const int64_t t = p.t_first + s;
-        const uint32_t tD1 = tD == 0u ? R - 1u : tD - 1u;     // window slot of step t - 1
-        // this step's trace of the partition's neurons, loaded before the wait
-        const uint8_t* fl = p.tr_f + (size_t)s * n;
-        const float* ut = p.tr_u + (size_t)s * n;
-        float u_pre[kApPre];
-        uint8_t f_pre[kApPre];
-#pragma unroll
-        for (int k = 0; k < kApPre; ++k) {
-            const uint32_t i = (uint32_t)tid + (uint32_t)k * kApThreads;
-            u_pre[k] = i < nc ? ut[lo + i] : 0.f;
-            f_pre[k] = i < nc ? fl[lo + i] : (uint8_t)0;
+        const int k_bar = p.len - 1 - s;
+        if (warp == kApWarps) {                       // the watching warp
+            __syncthreads();
+            if (lane == 0) watch(k_bar);
+            __syncthreads();
+            if (s_abort != 0u) break;
+            if (s > 0) arrive();
+            continue;
         }
-        // the spike flags of step t - 2, into step t's place: its walks are done
-        uint8_t nf[kApFlags];
-        if (s > 1) {
+        const uint32_t tD1 = tD == 0u ? R - 1u : tD - 1u;     // window slot of step t - 1
+        // ---- lI_t and what else of step t needs no partials ----
+        float slope[kApPre], keep[kApPre];            // s'(u_t); (1 - s_t) m_{t+1} P22 lu_{t+1}
 #pragma unroll
-            for (int k = 0; k < kApFlags; ++k) {
-                const uint32_t i = (uint32_t)tid + (uint32_t)k * kApThreads;
-                nf[k] = i < 32u * n_lg ? flag_of(i, s - 2) : (uint8_t)0;
+        for (int kp = 0; kp < kApPre; ++kp) {
+            const uint32_t i = (uint32_t)tid + (uint32_t)kp * kApThreads;
+            slope[kp] = keep[kp] = 0.f;
+            if (i < nc) {
+                const uint8_t f = f_pre[kp];
+                const bool mn = s_mn[i] != 0u;
+                const float lu1 = s_lu[i];
+                const float lub = mn ? __fmul_rn(p.P22, lu1) : 0.f;
+                const float lIt = __fadd_rn(__fmul_rn(p.P11, s_lI[i]), mn ? __fmul_rn(p.P21, lu1) : 0.f);
+                const float sv = (f & 1u) ? 1.f : 0.f;
+                const float x = __fsub_rn(u_pre[kp], p.theta);
+                const float a = __fadd_rn(1.0f, __fmul_rn(10.0f, fabsf(x)));
+                slope[kp] = __fdiv_rn(1.0f, __fmul_rn(a, a));
+                keep[kp] = __fmul_rn(__fsub_rn(1.f, sv), lub);
+                s_lI[i] = lIt;
+                s_mn[i] = (uint8_t)((f >> 1) & 1u);
+                win[tD * ws + i] = lIt;
+                if (g == 0) s_gN[i] += (double)lIt;
             }
         }
-        // the far part of step t - 1's gather while the other CTAs arrive
+        __syncthreads();
+        // the trace of step t - 1 and the spike flags of step t - 2 (into step
+        // t's place: its walks are done), in flight during the gather
+        uint8_t nf[kApFlags];
+        if (s > 0) load_trace(s - 1);
+        if (s > 1) {
+            const uint8_t* fl = p.tr_f + (size_t)(s - 2) * n;
+#pragma unroll
+            for (int k = 0; k < kApFlags; ++k) {
+                nf[k] = 0;
+                if (my_src[k] != kApNone) nf[k] = __ldg(fl + my_src[k]);
+            }
+        }
         if (s > 0) walk(t - 1, tD1, true);
         if (s > 1) {
             uint8_t* row = s_spk + (size_t)(t & 1) * spk_row;
@@ -296,51 +361,40 @@ k_adjoint_part(const __grid_constant__ AdjPartParams p) {
             for (uint32_t i = (uint32_t)tid + kApFlags * kApThreads; i < 32u * n_lg; i += kApThreads)
                 row[i] = flag_of(i, s - 2);
         }
-        if (!wait()) break;
-        // ---- membrane and current adjoints of partition c's neurons ----
-        float* pds_all = p.pds + (size_t)(t & 1) * p.n_part * n;
+        __syncthreads();                              // the partials of step t are there
+        if (s_abort != 0u) break;
+        const float* pds_t = p.pds + (size_t)(t & 1) * p.n_part * n + lo;
+        // a neuron's first kApPart partials, in flight during the near walk
+        float v[kApPart];
+#pragma unroll
+        for (int r = 0; r < kApPart; ++r)
+            v[r] = (uint32_t)tid < nc && r < p.n_part ? __ldcg(&pds_t[(size_t)r * n + tid]) : 0.f;
+        if (s > 0) walk(t - 1, tD1, false);
+        // ---- lu_t: the partials added in the partitions' order ----
 #pragma unroll
         for (int kp = 0; kp < kApPre; ++kp) {
             const uint32_t i = (uint32_t)tid + (uint32_t)kp * kApThreads;
             if (i >= nc) break;
-            const int32_t gi = lo + (int32_t)i;
-            // the partials of the partitions, kApPart in flight, added in order
             float acc = 0.f;
             for (int c0 = 0; c0 < p.n_part; c0 += kApPart) {
-                float v[kApPart];
+                if (kp > 0 || c0 > 0) {
 #pragma unroll
-                for (int r = 0; r < kApPart; ++r)
-                    v[r] = c0 + r < p.n_part ? __ldcg(&pds_all[(size_t)(c0 + r) * n + gi]) : 0.f;
+                    for (int r = 0; r < kApPart; ++r)
+                        v[r] = c0 + r < p.n_part ? __ldcg(&pds_t[(size_t)(c0 + r) * n + i]) : 0.f;
+                }
 #pragma unroll
                 for (int r = 0; r < kApPart; ++r)
                     if (c0 + r < p.n_part) acc = __fadd_rn(acc, v[r]);
             }
-            const float ds = __fadd_rn(p.gs[pop_index(p.pop_start, p.n_pop, gi)], acc);
-            const uint8_t f = f_pre[kp];
-            const bool mn = s_mn[i] != 0u;
-            const float lu1 = s_lu[i];
-            const float lub = mn ? __fmul_rn(p.P22, lu1) : 0.f;
-            const float lIt = __fadd_rn(__fmul_rn(p.P11, s_lI[i]), mn ? __fmul_rn(p.P21, lu1) : 0.f);
-            const float sv = (f & 1u) ? 1.f : 0.f;
-            const float x = __fsub_rn(u_pre[kp], p.theta);
-            const float a = __fadd_rn(1.0f, __fmul_rn(10.0f, fabsf(x)));
-            const float slope = __fdiv_rn(1.0f, __fmul_rn(a, a));
-            s_lu[i] = __fadd_rn(__fmul_rn(ds, slope), __fmul_rn(__fsub_rn(1.f, sv), lub));
-            s_lI[i] = lIt;
-            s_mn[i] = (uint8_t)((f >> 1) & 1u);
-            win[tD * ws + i] = lIt;
-            if (g == 0) s_gN[i] += (double)lIt;
+            const float ds = __fadd_rn(p.gs[pop_index(p.pop_start, p.n_pop, lo + (int32_t)i)], acc);
+            s_lu[i] = __fadd_rn(__fmul_rn(ds, slope[kp]), keep[kp]);
         }
-        __syncthreads();
-        // the near part of step t - 1's gather (it reads step t), its partials
-        if (s > 0) {
-            walk(t - 1, tD1, false);
-            arrive();
-        }
+        if (s > 0) arrive();
         tD = tD1;
     }
+    __syncthreads();
     if (g == 0 && s_abort == 0u) {
-        for (uint32_t i = tid; i < nc; i += kApThreads) {
+        for (uint32_t i = tid; i < nc; i += kApLaunch) {
             p.lu[lo + i] = s_lu[i];
             p.lI[lo + i] = s_lI[i];
             p.mnext[lo + i] = s_mn[i];
@@ -348,7 +402,7 @@ k_adjoint_part(const __grid_constant__ AdjPartParams p) {
         }
         // the lI ring of the next launch (the segment before): steps t_first
         // .. t_first + R - 2, which the window holds now
-        for (uint32_t k = tid; k < (R - 1) * nc; k += kApThreads) {
+        for (uint32_t k = tid; k < (R - 1) * nc; k += kApLaunch) {
             const uint32_t d = k / nc, i = k - d * nc;
             const int64_t tt = p.t_first + d;
             p.lring[(size_t)(tt & (kRing - 1)) * n + lo + i] = win[(uint32_t)(tt % R) * ws + i];
@@ -589,7 +643,7 @@ int adjoint_part_plan(int n, int n_pop, const int32_t* pop_start, int n_part, co
         e = cudaFuncSetAttribute(k_adjoint_part, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     int per_sm = 0;
     if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_adjoint_part, kApThreads, smem);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_adjoint_part, kApLaunch, smem);
     if (e != cudaSuccess || per_sm * sms < plan->grid) {
         adjoint_part_free(plan);
         cudaGetLastError();
@@ -618,7 +672,7 @@ cudaError_t launch_adjoint_part(const AdjPartPlan& plan, AdjPartParams& ap, cuda
     ap.img_off = plan.d_img_off;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(plan.grid);
-    cfg.blockDim = dim3(kApThreads);
+    cfg.blockDim = dim3(kApLaunch);
     cfg.dynamicSmemBytes = plan.smem;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
