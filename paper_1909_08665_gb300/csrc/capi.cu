@@ -218,7 +218,7 @@ int make_tables(snn_net* net) {
 void free_net(snn_net* net) {
     if (!net) return;
     void* ptrs[] = {net->d_part_lo, net->d_row_start, net->d_seg, net->d_words, net->d_pre, net->d_wtab,
-                    net->d_dtab, net->d_u, net->d_i, net->d_r, net->d_ring, net->d_msg, net->d_wrap,
+                    net->d_dtab, net->d_u, net->d_i, net->d_r, net->d_ring, net->d_ring_io, net->d_msg, net->d_wrap,
                     net->d_ras_step, net->d_ras_id, net->d_ras_n, net->d_counters,
                     net->d_sync, net->d_pop_spikes, net->d_rt};
     for (void* p : ptrs)
@@ -709,6 +709,26 @@ int net_update_saturation(snn_net* net) {
     return SNN_OK;
 }
 
+int net_ring_to_host(snn_net* net, int32_t* host) {
+    const size_t words = (size_t)kRing * net->n;
+    if (!net->d_ring_io) CALL(dalloc(&net->d_ring_io, words, "ring staging"));
+    CK(launch_ring_layout(net->d_part_lo, net->P, net->ncmax, net->n, net->d_ring, net->d_ring_io, true,
+                          net->stream));
+    CK(cudaMemcpyAsync(host, net->d_ring_io, sizeof(int32_t) * words, cudaMemcpyDeviceToHost, net->stream));
+    CK(cudaStreamSynchronize(net->stream));
+    return SNN_OK;
+}
+
+int net_ring_from_host(snn_net* net, const int32_t* host) {
+    const size_t words = (size_t)kRing * net->n;
+    if (!net->d_ring_io) CALL(dalloc(&net->d_ring_io, words, "ring staging"));
+    CK(cudaMemcpyAsync(net->d_ring_io, host, sizeof(int32_t) * words, cudaMemcpyHostToDevice, net->stream));
+    CK(launch_ring_layout(net->d_part_lo, net->P, net->ncmax, net->n, net->d_ring, net->d_ring_io, false,
+                          net->stream));
+    CK(cudaStreamSynchronize(net->stream));
+    return SNN_OK;
+}
+
 cudaError_t net_clear_wraps(snn_net* net) {
     if (!net->d_wrap) return cudaSuccess;
     return cudaMemsetAsync(net->d_wrap, 0, sizeof(int32_t) * (size_t)net->P * kRing * net->ncmax,
@@ -892,17 +912,7 @@ int snn_read_state(snn_net* net, float* u_host, float* i_syn_host, int32_t* refr
 
 int snn_read_ring(snn_net* net, int32_t* ring_host) {
     if (!net || !ring_host) return fail(SNN_ERR_INVALID, "bad arguments");
-    CK(cudaStreamSynchronize(net->stream));
-    std::vector<int32_t> tmp((size_t)net->P * kRing * net->ncmax);
-    CK(cudaMemcpy(tmp.data(), net->d_ring, sizeof(int32_t) * tmp.size(), cudaMemcpyDeviceToHost));
-    for (int c = 0; c < net->P; ++c) {
-        const int lo = net->part_lo[c], nc = net->part_lo[c + 1] - lo;
-        for (int slot = 0; slot < kRing; ++slot)
-            for (int k = 0; k < nc; ++k)
-                ring_host[(size_t)slot * net->n + lo + k] =
-                    tmp[((size_t)c * kRing + slot) * net->ncmax + k];
-    }
-    return SNN_OK;
+    return net_ring_to_host(net, ring_host);
 }
 
 int snn_counters(snn_net* net, int64_t* step, uint64_t* spikes, uint64_t* events) {

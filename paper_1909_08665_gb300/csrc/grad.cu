@@ -779,16 +779,7 @@ int snn_save_state(snn_net* net, void* buf_host, int64_t cap, int64_t* n_bytes) 
     GCK(cudaMemcpy(b + 32, net->d_u, n * 4, cudaMemcpyDeviceToHost));
     GCK(cudaMemcpy(b + 32 + n * 4, net->d_i, n * 4, cudaMemcpyDeviceToHost));
     GCK(cudaMemcpy(b + 32 + n * 8, net->d_r, n * 4, cudaMemcpyDeviceToHost));
-    std::vector<int32_t> tmp(ring_words(net));
-    GCK(cudaMemcpy(tmp.data(), net->d_ring, tmp.size() * 4, cudaMemcpyDeviceToHost));
-    int32_t* ring = reinterpret_cast<int32_t*>(b + 32 + n * 12);
-    for (int c = 0; c < net->P; ++c) {
-        const int lo = net->part_lo[c], nc = net->part_lo[c + 1] - lo;
-        for (int slot = 0; slot < kRing; ++slot)
-            std::memcpy(ring + (size_t)slot * n + lo, tmp.data() + ((size_t)c * kRing + slot) * net->ncmax,
-                        sizeof(int32_t) * nc);
-    }
-    return SNN_OK;
+    return net_ring_to_host(net, reinterpret_cast<int32_t*>(b + 32 + n * 12));
 }
 
 int snn_load_state(snn_net* net, const void* buf_host, int64_t n_bytes) {
@@ -801,19 +792,11 @@ int snn_load_state(snn_net* net, const void* buf_host, int64_t n_bytes) {
     std::memcpy(hdr, b, 32);
     if (hdr[0] != kStateMagic || hdr[1] != (uint64_t)n || hdr[3] != (uint64_t)kRing)
         return set_error(SNN_ERR_INVALID, "not a state of this network");
-    std::vector<int32_t> tmp(ring_words(net), 0);
-    const int32_t* ring = reinterpret_cast<const int32_t*>(b + 32 + n * 12);
-    for (int c = 0; c < net->P; ++c) {
-        const int lo = net->part_lo[c], nc = net->part_lo[c + 1] - lo;
-        for (int slot = 0; slot < kRing; ++slot)
-            std::memcpy(tmp.data() + ((size_t)c * kRing + slot) * net->ncmax, ring + (size_t)slot * n + lo,
-                        sizeof(int32_t) * nc);
-    }
     GCK(cudaStreamSynchronize(net->stream));
     GCK(cudaMemcpy(net->d_u, b + 32, n * 4, cudaMemcpyHostToDevice));
     GCK(cudaMemcpy(net->d_i, b + 32 + n * 4, n * 4, cudaMemcpyHostToDevice));
     GCK(cudaMemcpy(net->d_r, b + 32 + n * 8, n * 4, cudaMemcpyHostToDevice));
-    GCK(cudaMemcpy(net->d_ring, tmp.data(), tmp.size() * 4, cudaMemcpyHostToDevice));
+    GCALL(net_ring_from_host(net, reinterpret_cast<const int32_t*>(b + 32 + n * 12)));
     GCK(clear_messages(net));
     GCK(net_clear_wraps(net));
     GCK(cudaStreamSynchronize(net->stream));

@@ -61,6 +61,7 @@ struct snn_net {
     uint32_t* d_ras_step = nullptr;
     uint32_t* d_ras_id = nullptr;
     uint32_t* d_ras_n = nullptr;
+    int32_t* d_ring_io = nullptr;           // [64][n] the ring in the ABI's layout (host copies)
     snn::RasterSort ras_sort;               // workspace of the raster reads
     int64_t ras_lo = INT64_MAX, ras_hi = 0; // steps launched since the last raster read
     unsigned long long* d_counters = nullptr;
@@ -86,6 +87,9 @@ int net_upload_weights(snn_net* net);
 // recompute the input bound from the weights; the first time it reaches 2^31
 // the wrap-count array is allocated, and the step kernel counts wrap-arounds
 int net_update_saturation(snn_net* net);
+// the ring buffers to / from host memory, slot-major [64][n] (synchronises)
+int net_ring_to_host(snn_net* net, int32_t* host);
+int net_ring_from_host(snn_net* net, const int32_t* host);
 // zero the wrap counts (after the ring was replaced: load, restore)
 cudaError_t net_clear_wraps(snn_net* net);
 // launch the step kernel for n steps from step t0 with the given parameters

@@ -282,6 +282,9 @@ struct RasterSort {
 };
 cudaError_t raster_sort(RasterSort* w, const RasterList& in, size_t n, cudaStream_t s);
 void raster_sort_free(RasterSort* w);
+// the ring [n_part][kRing][ncmax] into slot-major abi [kRing][n], or back
+cudaError_t launch_ring_layout(const int32_t* part_lo, int n_part, int ncmax, int n, int32_t* ring,
+                               int32_t* abi, bool to_abi, cudaStream_t s);
 cudaError_t launch_init_state(int n, uint32_t key0, uint32_t key1, float lo, float hi,
                               float* u, cudaStream_t s);
 int step_kernel_variant(int npt, bool smem_ring);
