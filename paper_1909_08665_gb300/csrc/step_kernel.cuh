@@ -21,6 +21,12 @@
 //         spikes of step t are compacted with warp ballots and published as
 //         a message of 64-bit words (tag = t+1, value) -- the count and the
 //         neuron ids; the Poisson background count of step t is drawn.
+//         The warps only arrive at the barrier that completes the count, and
+//         go on; the last warp waits at it and publishes the count.  (With a
+//         CTA barrier there, the count waited for the warps that had to have
+//         the other partitions' message heads first: us per step at scale
+//         0.02 1.72, 0.1 1.78, 4 14.6; now 1.64, 1.73 and 12.7; at scale 1
+//         2.57 either way.)
 //   D     wait for every partition's message of step t-1 (each word carries
 //         its own tag, so a matching tag is both the grid-wide barrier and
 //         the data; no fence, no counter), look up each spike's run for this
@@ -337,7 +343,7 @@ __device__ __forceinline__ void early_runs(const StepParams& sp, int c, const ul
 template <bool SAT, int BATCH, int WAVE>
 __device__ __forceinline__ bool deliver_list(const StepParams& sp, unsigned char* smem,
                                              const SmemLayout& L, int c, uint32_t wbase,
-                                             int64_t tb, int32_t* ring, int32_t* wrap,
+                                             int64_t tb, int par, int32_t* ring, int32_t* wrap,
                                              unsigned long long& events,
                                              const ulonglong2 (&pre)[4],
                                              const EarlyRuns& early) {
@@ -347,6 +353,9 @@ __device__ __forceinline__ bool deliver_list(const StepParams& sp, unsigned char
     const uint32_t tag = (uint32_t)(tb + 1);
     uint32_t* s_warp = reinterpret_cast<uint32_t*>(smem + L.warp);
     volatile uint32_t* s_misc = reinterpret_cast<uint32_t*>(smem + L.misc);
+    // listed spikes, in the counter of this list's parity; the other one is
+    // cleared after the barrier below, when its last readers are done
+    volatile uint32_t* s_list = s_misc + 6 + par;
     unsigned long long* s_inl = reinterpret_cast<unsigned long long*>(smem + L.inl);
     uint32_t* s_rb = reinterpret_cast<uint32_t*>(smem + L.rb);
     uint32_t* s_rl = reinterpret_cast<uint32_t*>(smem + L.rl);
@@ -408,7 +417,7 @@ __device__ __forceinline__ bool deliver_list(const StepParams& sp, unsigned char
     //     ids beyond the inline ones are loaded 8 at a time, all in flight,
     //     and the run bounds of a group of ids are looked up together
     if (tid < P && my_cnt > 0u) {
-        const uint32_t at = atomicAdd(const_cast<uint32_t*>(&s_misc[3]), my_cnt);
+        const uint32_t at = atomicAdd(const_cast<uint32_t*>(s_list), my_cnt);
         if (at + my_cnt <= (uint32_t)kChunk) {
             if (early.ok) {                          // bounds looked up during A(tb + 1)
 #pragma unroll
@@ -454,19 +463,18 @@ __device__ __forceinline__ bool deliver_list(const StepParams& sp, unsigned char
         }
     }
     __syncthreads();
-    const uint32_t S_fast = s_misc[3];
+    const uint32_t S_fast = *s_list;
+    if (tid == 0) s_misc[6 + (par ^ 1)] = 0u;
     if (s_misc[2]) return false;
     if (S_fast <= (uint32_t)kChunk) {
         deliver_batches<SAT, BATCH, WAVE>(sp, s_rb, s_rl, s_w, wbase, S_fast, tb, ring, wrap, events,
                                           s_cnt);
         __syncthreads();
-        if (tid == 0) s_misc[3] = 0u;
         flush_counts(S_fast);
         return s_misc[2] == 0u;
     }
     // 2b. more than kChunk spikes: offsets by a block-wide scan, in chunks
     const uint32_t S = block_scan<1>(cnt, s_warp);   // cnt[0] <- my offset
-    if (tid == 0) s_misc[3] = 0u;
     const uint32_t my_off = cnt[0];
 
     for (uint32_t base = 0; base < S; base += kChunk) {
@@ -528,6 +536,15 @@ __device__ __forceinline__ void span16(const uint32_t* base, unsigned long long 
 // only in its own instantiation, so the plain step loop is unchanged.
 constexpr int kModePaced = 1;
 constexpr int kModeSat = 2;
+
+constexpr int kPublisher = kStepThreads - 32;   // first thread of the warp that publishes a step's count
+// barrier `id` of the CTA: arrive without waiting, or wait for all n threads
+__device__ __forceinline__ void barrier_arrive(int id, int n) {
+    asm volatile("barrier.cta.arrive %0, %1;" ::"r"(id), "r"(n) : "memory");
+}
+__device__ __forceinline__ void barrier_wait(int id, int n) {
+    asm volatile("barrier.cta.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
+}
 
 template <int NPT, bool SMEM_RING, int MODE>
 __global__ void __launch_bounds__(kStepThreads, 1)
@@ -672,6 +689,29 @@ k_step(const __grid_constant__ StepParams sp) {
                     }
                 }
             }
+        }
+        // every warp has counted its spikes: the last one waits for that and
+        // publishes the count; the others only arrive and go on
+        if (tid < kPublisher) {
+            barrier_arrive(1, kStepThreads);
+        } else {
+            barrier_wait(1, kStepThreads);
+            if (tid == kPublisher) {
+                const uint32_t nsp = *my_cnt;
+                // counter of step s+1 (last read in step s-1, before this barrier)
+                s_misc[(s + 1) & 1] = 0u;
+                if (!(sp.inject_fault == 1 && c == 0)) __stcg(&my_msg[0], tag | nsp);
+                spikes += nsp;
+                if (ras_base + nsp > sp.ras_cap) atomicOr(sp.status, kStatusRasterOverflow);
+                if (sp.st_counts != nullptr && nsp > 0u) {
+                    const int64_t r = t - sp.sc_t0;
+                    if (r >= 0 && r < sp.sc_cap) atomicAdd(&sp.st_counts[4 * r], nsp);
+                }
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < NPT; ++k) {
+            const int li = tid + k * kStepThreads;
             // background count of step t (independent of the network): drawn
             // here, added to the ring input in C(t)
             if (sp.mode == 0 && li < nc) {
@@ -698,30 +738,17 @@ k_step(const __grid_constant__ StepParams sp) {
         EarlyRuns early;
         early.ok = false;
         if (EARLY && s > 0 && tid < P) early_runs(sp, c, pre, (uint32_t)t, early);
-        __syncthreads();
-        const uint32_t nsp = *my_cnt;
-        if (tid == 0) {
-            // counter of step s+1 (last used in step s-1): its readers are all
-            // past a barrier; in step 0 it is still zero from the start and is
-            // left alone (no barrier separates it from step 1's adds)
-            if (s > 0) s_misc[(s + 1) & 1] = 0u;
-            if (!(sp.inject_fault == 1 && c == 0)) __stcg(&my_msg[0], tag | nsp);
-            spikes += nsp;
-            if (ras_base + nsp > sp.ras_cap) atomicOr(sp.status, kStatusRasterOverflow);
-            if (sp.st_counts != nullptr && nsp > 0u) {
-                const int64_t r = t - sp.sc_t0;
-                if (r >= 0 && r < sp.sc_cap) atomicAdd(&sp.st_counts[4 * r], nsp);
-            }
-        }
-        ras_base += nsp;
         // ---- D: spikes of step t-1 ----
         if (s > 0) {
             if (!deliver_list<SAT, BatchShape<NPT>::kSpikes, BatchShape<NPT>::kWave>(
-                    sp, smem, L, c, wt_base, t - 1, ring, wrap, events, pre, early)) {
+                    sp, smem, L, c, wt_base, t - 1, s & 1, ring, wrap, events, pre, early)) {
                 aborted = true;
                 break;
             }
+        } else {
+            __syncthreads();                     // the counts of step 0, as after a delivery
         }
+        ras_base += *my_cnt;
         // ---- C(t): ring slot t, Poisson background, synaptic current ----
         const uint32_t slot = (uint32_t)t & (kRing - 1);
 #pragma unroll
@@ -777,7 +804,7 @@ k_step(const __grid_constant__ StepParams sp) {
         EarlyRuns none;
         none.ok = false;
         deliver_list<SAT, BatchShape<NPT>::kSpikes, BatchShape<NPT>::kWave>(
-            sp, smem, L, c, wt_base, tl, ring, wrap, events, pre, none);
+            sp, smem, L, c, wt_base, tl, sp.n_steps & 1, ring, wrap, events, pre, none);
     }
     __syncthreads();
 #pragma unroll
@@ -791,7 +818,7 @@ k_step(const __grid_constant__ StepParams sp) {
     }
     if (SMEM_RING)
         for (int k = tid; k < kRing * sp.ncmax; k += kStepThreads) ring_g[k] = ring[k];
-    if (tid == 0) {
+    if (tid == kPublisher) {
         sp.ras_n[c] = ras_base;
         atomicAdd(&sp.counters[0], spikes);
     }
