@@ -751,12 +751,21 @@ k_step(const __grid_constant__ StepParams sp) {
         ras_base += *my_cnt;
         // ---- C(t): ring slot t, Poisson background, synaptic current ----
         const uint32_t slot = (uint32_t)t & (kRing - 1);
+        // all of the thread's cells are in flight before the first is cleared
+        // (one after the other, their L2 round trips made C(t) 3 us of the 4x
+        // network's step: 12.7 us per step, now 9.0; 2x 8.4, now 5.3)
+        int32_t cells[NPT];
+#pragma unroll
+        for (int k = 0; k < NPT; ++k) {
+            const int li = tid + k * kStepThreads;
+            cells[k] = li < nc ? ring[slot * (uint32_t)sp.ncmax + (uint32_t)li] : 0;
+        }
 #pragma unroll
         for (int k = 0; k < NPT; ++k) {
             const int li = tid + k * kStepThreads;
             if (li < nc) {
                 const uint32_t cell = slot * (uint32_t)sp.ncmax + (uint32_t)li;
-                const int32_t r = ring[cell];
+                const int32_t r = cells[k];
                 ring[cell] = 0;
                 // the input wraps modulo 2^32, as the int32 accumulation of
                 // the method does; SAT: its true value r + 2^32 wraps + pacc
