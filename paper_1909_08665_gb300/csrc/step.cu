@@ -153,7 +153,7 @@ k_deliver_part(const __grid_constant__ StepParams sp, const uint32_t* __restrict
             s_rl[k] = __ldg(sg + 1) - b;
         }
         __syncthreads();
-        deliver_batches<false, BatchShape<1>::kSpikes, BatchShape<1>::kWave>(
+        deliver_batches<false>(
             sp, s_rb, s_rl, s_w, wbase, (uint32_t)m, t, ring, nullptr, events, nullptr);
         __syncthreads();
     }

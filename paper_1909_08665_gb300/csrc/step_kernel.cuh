@@ -57,24 +57,16 @@ namespace snn {
 constexpr int kWarps = kStepThreads / 32;
 constexpr uint32_t kStatusRasterOverflow = 2u;
 constexpr int kInline = 7;              // ids read together with a message header (64 B)
-// A warp takes BATCH spikes at once and loads the first 32 WAVE entries of
-// each of their runs in one wave (runs: mean 26 entries at scale 1 and 4,
-// rarely above 96).  At full size (one neuron per thread) the spikes are
-// dealt round-robin over the warps and each warp loads its next batch before
-// the adds of the current one; measured that way, 2 x 3 is fastest (2.566 us
-// per step; 3 x 3: 2.618, 2 x 2: 2.658, 4 x 3: 2.695, 4 x 2: 2.725, 1 x 3:
-// 2.754; two batches ahead, 2 x 3: 2.657, 1 x 3: 2.779), against 2.711 for
-// 3 x 3 in contiguous batches without the early load, the fastest shape of
-// those (earlier in the kernel's history 3.00 us; 4 x 4: 3.14, 2 x 3: 3.08,
-// 3 x 2: 3.24, 2 x 2: 3.21).  At 4x
-// (4 neurons per thread, 177 spikes per step; contiguous batches, loaded one
-// at a time: the registers of that variant are spent) 8 x 3 is fastest
-// (14.3 us; 4 x 4: 14.5, 3 x 3: 15.9, 6 x 4: 16.0, 8 x 4: 16.4).
-template <int NPT>
-struct BatchShape {
-    static constexpr int kSpikes = NPT == 1 ? 2 : 8;
-    static constexpr int kWave = 3;
-};
+// A warp takes kBatchSpikes spikes at once and loads the first 32 kRunWave
+// entries of each of their runs in one wave (runs: mean 26 entries at scale 1
+// and 4, rarely above 96).  The spikes are dealt round-robin over the warps,
+// and each warp loads its next batch before the adds of the current one.  us
+// per step by shape (spikes x waves), full size: 2 x 3 2.57, 3 x 3 2.62, 2 x 2
+// 2.66, 4 x 3 2.70, 1 x 3 2.75, two batches ahead 2.66; 4x (4 neurons per
+// thread): 2 x 3 8.23, 3 x 3 8.26, and in contiguous batches without the early
+// load 4 x 3 8.53, 6 x 3 8.66, 8 x 3 9.01, 8 x 2 9.74.
+constexpr int kBatchSpikes = 2;
+constexpr int kRunWave = 3;
 constexpr uint32_t kPopWords = kMaxPop * kWCodes;   // weight-table entries per target population
 
 // ---------------------------------------------------------------------------
@@ -170,17 +162,16 @@ __device__ inline bool poll_word(const StepParams& sp, const unsigned long long*
 
 // ---------------------------------------------------------------------------
 // the runs s_rb/s_rl[0, m) of the spikes of step tb into this CTA's ring:
-// batches of kBatchSpikes spikes per warp (BatchShape).  Entry x of a run (a pre-decoded synapse) is
+// batches of kBatchSpikes spikes per warp.  Entry x of a run (a pre-decoded synapse) is
 // the weight-table index x >> kPreOffBits and the ring offset
 // x & kPreOffMask = delay * ncmax + local target; its weight, looked up in
 // s_w (table rows from population p_lo on, wbase = p_lo * kPopWords), is
 // added at ((tb mod 64) * ncmax + offset) wrapped into the 64-slot ring.  Each
-// lane loads entries lane + 32 h (h < kRunWave) of all the batch's runs before the
-// first add (all loads in flight at once); longer runs finish in a loop.  In
-// the pipelined shape (PIPE) warp w's batch of round r holds the list's
-// spikes r kStride + w + k kWarps (k < kBatchSpikes), so a short list spreads
-// over all warps, and the next round's batch is loaded before this one's
-// adds; otherwise a batch is kBatchSpikes consecutive spikes.
+// lane loads entries lane + 32 h (h < kRunWave) of all the batch's runs before
+// the first add (all loads in flight at once); longer runs finish in a loop.
+// Warp w's batch of round r holds the list's spikes r kStride + w + k kWarps
+// (k < kBatchSpikes), so a short list spreads over all warps, and the next
+// round's batch is loaded before this one's adds.
 // ---------------------------------------------------------------------------
 // SAT: the networks whose input can leave the int32 range also count, per
 // ring cell, the net number of times its int32 sum wrapped around (+1 past
@@ -205,7 +196,7 @@ __device__ __forceinline__ void add_entry(uint32_t x, const int32_t* s_w, uint32
 
 // s_cnt (non-null while per-step counts are recorded): the list's synaptic
 // events and its non-empty runs are added into s_cnt[0], s_cnt[1]
-template <bool SAT, int kBatchSpikes, int kRunWave>
+template <bool SAT>
 __device__ __forceinline__ void deliver_batches(const StepParams& sp, const uint32_t* s_rb,
                                                 const uint32_t* s_rl, const int32_t* s_w,
                                                 uint32_t wbase, uint32_t m, int64_t tb,
@@ -215,17 +206,13 @@ __device__ __forceinline__ void deliver_batches(const StepParams& sp, const uint
     const int32_t R = kRing * sp.ncmax;                  // ring words of this CTA
     const int32_t base_t = (int32_t)(((uint32_t)tb & (kRing - 1)) * (uint32_t)sp.ncmax);
     const uint32_t* pre = sp.pre;
-    // PIPE: the warp's next batch is loaded before this one's adds, so its
-    // round trip overlaps them (steps with more than kStride spikes); only
-    // where the registers allow it (the one-neuron-per-thread shape)
-    constexpr bool PIPE = kBatchSpikes * kRunWave <= 9;
     // run bounds and first-wave entries of the batch whose first spike is
     // list position g0 (nothing past m is read)
     auto load = [&](uint32_t g0, uint32_t (&rb)[kBatchSpikes], uint32_t (&rl)[kBatchSpikes],
                     uint32_t (&ev)[kBatchSpikes][kRunWave]) {
 #pragma unroll
         for (int k = 0; k < kBatchSpikes; ++k) {
-            const uint32_t i = g0 + (uint32_t)k * (PIPE ? (uint32_t)kWarps : 1u);
+            const uint32_t i = g0 + (uint32_t)(k * kWarps);
             const bool ok = i < m;
             rb[k] = ok ? s_rb[i] : 0u;
             rl[k] = ok ? s_rl[i] : 0u;
@@ -237,15 +224,14 @@ __device__ __forceinline__ void deliver_batches(const StepParams& sp, const uint
         }
     };
     constexpr uint32_t kStride = (uint32_t)kWarps * kBatchSpikes;
-    uint32_t g0 = (uint32_t)warp * (PIPE ? 1u : (uint32_t)kBatchSpikes);
+    uint32_t g0 = (uint32_t)warp;
     uint32_t rb[kBatchSpikes], rl[kBatchSpikes];
     uint32_t ev[kBatchSpikes][kRunWave];
-    if (PIPE) load(g0, rb, rl, ev);
+    load(g0, rb, rl, ev);
     for (; g0 < m; g0 += kStride) {
         uint32_t nrb[kBatchSpikes], nrl[kBatchSpikes];
         uint32_t nev[kBatchSpikes][kRunWave];
-        if (PIPE) load(g0 + kStride, nrb, nrl, nev);
-        else load(g0, rb, rl, ev);
+        load(g0 + kStride, nrb, nrl, nev);
 #pragma unroll
         for (int k = 0; k < kBatchSpikes; ++k) {
 #pragma unroll
@@ -267,14 +253,12 @@ __device__ __forceinline__ void deliver_batches(const StepParams& sp, const uint
             atomicAdd(&s_cnt[0], ev_sum);
             atomicAdd(&s_cnt[1], busy);
         }
-        if (PIPE) {
 #pragma unroll
-            for (int k = 0; k < kBatchSpikes; ++k) {
-                rb[k] = nrb[k];
-                rl[k] = nrl[k];
+        for (int k = 0; k < kBatchSpikes; ++k) {
+            rb[k] = nrb[k];
+            rl[k] = nrl[k];
 #pragma unroll
-                for (int h = 0; h < kRunWave; ++h) ev[k][h] = nev[k][h];
-            }
+            for (int h = 0; h < kRunWave; ++h) ev[k][h] = nev[k][h];
         }
     }
 }
@@ -340,7 +324,7 @@ __device__ __forceinline__ void early_runs(const StepParams& sp, int c, const ul
 // delivery of the spikes of step tb (message tag tb+1) into this CTA's ring;
 // returns false if a wait timed out or another CTA aborted
 // ---------------------------------------------------------------------------
-template <bool SAT, int BATCH, int WAVE>
+template <bool SAT>
 __device__ __forceinline__ bool deliver_list(const StepParams& sp, unsigned char* smem,
                                              const SmemLayout& L, int c, uint32_t wbase,
                                              int64_t tb, int par, int32_t* ring, int32_t* wrap,
@@ -467,7 +451,7 @@ __device__ __forceinline__ bool deliver_list(const StepParams& sp, unsigned char
     if (tid == 0) s_misc[6 + (par ^ 1)] = 0u;
     if (s_misc[2]) return false;
     if (S_fast <= (uint32_t)kChunk) {
-        deliver_batches<SAT, BATCH, WAVE>(sp, s_rb, s_rl, s_w, wbase, S_fast, tb, ring, wrap, events,
+        deliver_batches<SAT>(sp, s_rb, s_rl, s_w, wbase, S_fast, tb, ring, wrap, events,
                                           s_cnt);
         __syncthreads();
         flush_counts(S_fast);
@@ -503,7 +487,7 @@ __device__ __forceinline__ bool deliver_list(const StepParams& sp, unsigned char
             }
         }
         __syncthreads();
-        deliver_batches<SAT, BATCH, WAVE>(sp, s_rb, s_rl, s_w, wbase, m, tb, ring, wrap, events,
+        deliver_batches<SAT>(sp, s_rb, s_rl, s_w, wbase, m, tb, ring, wrap, events,
                                           s_cnt);
         __syncthreads();
     }
@@ -740,7 +724,7 @@ k_step(const __grid_constant__ StepParams sp) {
         if (EARLY && s > 0 && tid < P) early_runs(sp, c, pre, (uint32_t)t, early);
         // ---- D: spikes of step t-1 ----
         if (s > 0) {
-            if (!deliver_list<SAT, BatchShape<NPT>::kSpikes, BatchShape<NPT>::kWave>(
+            if (!deliver_list<SAT>(
                     sp, smem, L, c, wt_base, t - 1, s & 1, ring, wrap, events, pre, early)) {
                 aborted = true;
                 break;
@@ -812,7 +796,7 @@ k_step(const __grid_constant__ StepParams sp) {
         }
         EarlyRuns none;
         none.ok = false;
-        deliver_list<SAT, BatchShape<NPT>::kSpikes, BatchShape<NPT>::kWave>(
+        deliver_list<SAT>(
             sp, smem, L, c, wt_base, tl, sp.n_steps & 1, ring, wrap, events, pre, none);
     }
     __syncthreads();
