@@ -535,9 +535,10 @@ __global__ void __launch_bounds__(kStepThreads, 1)
 k_step(const __grid_constant__ StepParams sp) {
     constexpr bool PACED = (MODE & kModePaced) != 0;
     constexpr bool SAT = (MODE & kModeSat) != 0;
-    // early run lookups keep 2 x kInline more registers live across the
-    // background draw: only in the one-neuron-per-thread variant
-    constexpr bool EARLY = NPT == 1;
+    // early run lookups keep 2 x kInline more registers live until the delivery:
+    // not in the widest variant (us per step without / with: 1.3x 3.44 / 3.12,
+    // 2x 4.78 / 4.46, 4x 8.23 / 8.15)
+    constexpr bool EARLY = NPT <= 4;
     extern __shared__ __align__(16) unsigned char smem[];
     const int tid = threadIdx.x;
     const int lane = tid & 31;
