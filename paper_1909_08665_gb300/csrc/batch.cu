@@ -634,6 +634,7 @@ struct snn_batch {
     long long step = 0;
     std::vector<std::vector<uint32_t>> host_steps, host_ids;   // drained raster per instance
     RasterSort ras_sort;                 // workspace of the raster reads
+    HostStage stage;                     // small reads
     long long ras_lo = 0;                // first step since the last drain
     bool ras_new = false;                // steps were issued since the last drain
     std::vector<float2> u0_range;        // default initial potentials per instance
@@ -675,6 +676,7 @@ void free_batch(snn_batch* b) {
     for (void* x : ptrs)
         if (x) cudaFree(x);
     raster_sort_free(&b->ras_sort);
+    host_stage_free(&b->stage);
     delete b;
 }
 
@@ -841,21 +843,26 @@ int batch_trials(snn_batch* b) {
 // the spikes recorded since the last drain, sorted by (instance, step, id) on
 // the device, appended to each instance's host arrays
 int drain_raster(snn_batch* b) {
-    BCK(cudaStreamSynchronize(b->stream));
-    if (!b->ras_new) return SNN_OK;             // no step issued since: nothing recorded
-    uint32_t n = 0;
-    BCK(cudaMemcpy(&n, b->d_ras_n, sizeof(n), cudaMemcpyDeviceToHost));
-    const uint32_t m = std::min(n, b->ras_cap);
+    if (!b->ras_new) {                          // no step issued since: nothing recorded
+        BCK(cudaStreamSynchronize(b->stream));
+        return SNN_OK;
+    }
+    const RasterList in = {b->d_ras_n, b->d_ras_step, b->d_ras_id, b->ras_cap, 1, b->n_inst, b->d_goff,
+                           (uint32_t)b->ras_lo, b->step - b->ras_lo, (uint32_t)b->ntot};
+    RasterSmall small;
+    BCK(raster_read_small(in, b->d_ras_n, &b->stage, b->stream, &small));
+    const uint32_t m = small.n;
     std::vector<uint32_t> st(m), id(m);
-    if (m) {
-        const RasterList in = {b->d_ras_n, b->d_ras_step, b->d_ras_id, b->ras_cap, 1, b->n_inst, b->d_goff,
-                               (uint32_t)b->ras_lo, b->step - b->ras_lo, (uint32_t)b->ntot};
+    if (small.done) {
+        std::memcpy(st.data(), small.step, sizeof(uint32_t) * m);
+        std::memcpy(id.data(), small.id, sizeof(uint32_t) * m);
+    } else {
         BCK(raster_sort(&b->ras_sort, in, m, b->stream));
         BCK(cudaMemcpyAsync(st.data(), b->ras_sort.step, sizeof(uint32_t) * m, cudaMemcpyDeviceToHost, b->stream));
         BCK(cudaMemcpyAsync(id.data(), b->ras_sort.id, sizeof(uint32_t) * m, cudaMemcpyDeviceToHost, b->stream));
+        BCK(cudaMemsetAsync(b->d_ras_n, 0, sizeof(uint32_t), b->stream));
+        BCK(cudaStreamSynchronize(b->stream));
     }
-    BCK(cudaMemsetAsync(b->d_ras_n, 0, sizeof(uint32_t), b->stream));
-    BCK(cudaStreamSynchronize(b->stream));
     b->ras_new = false;
     b->ras_lo = b->step;
     for (uint32_t r = 0, k = 0; r < m; ++k) {
@@ -869,7 +876,7 @@ int drain_raster(snn_batch* b) {
         for (size_t i = at; i < out.size(); ++i) out[i] -= lo;
         r = e;
     }
-    if (n > b->ras_cap) return set_error(SNN_ERR_OVERFLOW, "batch raster capacity exceeded");
+    if (small.lost) return set_error(SNN_ERR_OVERFLOW, "batch raster capacity exceeded");
     return SNN_OK;
 }
 
@@ -1179,8 +1186,17 @@ int snn_batch_read_spikes(snn_batch* b, int32_t k, uint32_t* steps_host, uint32_
 int snn_batch_read_state(snn_batch* b, int32_t k, float* u_host, float* i_syn_host,
                          int32_t* refr_host) {
     if (!b || k < 0 || k >= b->n_inst) return set_error(SNN_ERR_INVALID, "bad arguments");
-    BCK(cudaStreamSynchronize(b->stream));
     const InstCold& C = b->cold_h[k];
+    if (C.n <= kStageNeurons) {
+        const uint32_t* const src[3] = {reinterpret_cast<const uint32_t*>(b->d_u) + C.goff,
+                                        reinterpret_cast<const uint32_t*>(b->d_i) + C.goff,
+                                        reinterpret_cast<const uint32_t*>(b->d_r) + C.goff};
+        uint32_t* const dst[3] = {reinterpret_cast<uint32_t*>(u_host), reinterpret_cast<uint32_t*>(i_syn_host),
+                                  reinterpret_cast<uint32_t*>(refr_host)};
+        BCK(read_arrays(3, src, dst, C.n, &b->stage, b->stream));
+        return SNN_OK;
+    }
+    BCK(cudaStreamSynchronize(b->stream));
     if (u_host) BCK(cudaMemcpy(u_host, b->d_u + C.goff, sizeof(float) * C.n, cudaMemcpyDeviceToHost));
     if (i_syn_host)
         BCK(cudaMemcpy(i_syn_host, b->d_i + C.goff, sizeof(float) * C.n, cudaMemcpyDeviceToHost));
@@ -1191,9 +1207,10 @@ int snn_batch_read_state(snn_batch* b, int32_t k, float* u_host, float* i_syn_ho
 
 int snn_batch_counters(snn_batch* b, int32_t k, int64_t* step, uint64_t* spikes, uint64_t* events) {
     if (!b || k < 0 || k >= b->n_inst) return set_error(SNN_ERR_INVALID, "bad arguments");
-    BCK(cudaStreamSynchronize(b->stream));
     unsigned long long c[2];
-    BCK(cudaMemcpy(c, b->d_ic + 2 * k, sizeof(c), cudaMemcpyDeviceToHost));
+    const uint32_t* const src[1] = {reinterpret_cast<const uint32_t*>(b->d_ic + 2 * k)};
+    uint32_t* const dst[1] = {reinterpret_cast<uint32_t*>(c)};
+    BCK(read_arrays(1, src, dst, 4, &b->stage, b->stream));
     if (step) *step = b->step;
     if (spikes) *spikes = c[0];
     if (events) *events = c[1];

@@ -224,6 +224,7 @@ void free_net(snn_net* net) {
     for (void* p : ptrs)
         if (p) cudaFree(p);
     raster_sort_free(&net->ras_sort);
+    host_stage_free(&net->stage);
     free_grad(net->grad);
     delete net;
 }
@@ -482,6 +483,12 @@ int build_from_rows(snn_net* net, const uint64_t* row_ptr, const uint32_t* words
     CK(launch_seg_from_rows(net->d_row_start, net->d_words, n, net->d_part_lo, P, net->d_seg, s));
     CK(cudaStreamSynchronize(s));
     return finish_network(net);
+}
+
+int raster_overflow(bool lost, bool short_cap) {
+    if (lost) return fail(SNN_ERR_OVERFLOW, "spike raster capacity exceeded; spikes were lost");
+    if (short_cap) return fail(SNN_ERR_OVERFLOW, "cap smaller than the recorded spikes; the rest were dropped");
+    return SNN_OK;
 }
 
 int check_status(snn_net* net) {
@@ -858,20 +865,36 @@ int snn_sync(snn_net* net) {
 int snn_read_spikes(snn_net* net, uint32_t* steps_host, uint32_t* ids_host, int64_t cap,
                     int64_t* n) {
     if (!net || !n || cap < 0) return fail(SNN_ERR_INVALID, "bad arguments");
-    CK(cudaStreamSynchronize(net->stream));
-    std::vector<uint32_t> cnt(net->P);
-    CK(cudaMemcpy(cnt.data(), net->d_ras_n, sizeof(uint32_t) * net->P, cudaMemcpyDeviceToHost));
+    const RasterList in = {net->d_ras_n, net->d_ras_step, net->d_ras_id, net->ras_cap, net->P, 1, nullptr,
+                           (uint32_t)net->ras_lo, net->ras_hi - net->ras_lo, (uint32_t)net->n};
     int64_t total = 0;
     bool lost = false;
-    for (int c = 0; c < net->P; ++c) {
-        if (cnt[c] > net->ras_cap) lost = true;
-        total += std::min<uint32_t>(cnt[c], net->ras_cap);
+    if (net->P < kStepThreads) {
+        RasterSmall r;
+        CK(raster_read_small(in, net->d_ras_n, &net->stage, net->stream, &r));
+        total = r.n;
+        lost = r.lost;
+        if (r.done) {
+            const int64_t got = std::min<int64_t>(total, cap);
+            if (steps_host) std::memcpy(steps_host, r.step, sizeof(uint32_t) * got);
+            if (ids_host) std::memcpy(ids_host, r.id, sizeof(uint32_t) * got);
+            net->ras_lo = INT64_MAX;
+            net->ras_hi = 0;
+            *n = got;
+            return raster_overflow(lost, got < total);
+        }
+    } else {
+        CK(cudaStreamSynchronize(net->stream));
+        std::vector<uint32_t> cnt(net->P);
+        CK(cudaMemcpy(cnt.data(), net->d_ras_n, sizeof(uint32_t) * net->P, cudaMemcpyDeviceToHost));
+        for (int c = 0; c < net->P; ++c) {
+            if (cnt[c] > net->ras_cap) lost = true;
+            total += std::min<uint32_t>(cnt[c], net->ras_cap);
+        }
     }
     // sorted on the device, the first `cap` copied back, one transfer per array
     const int64_t got = std::min<int64_t>(total, cap);
     if (got > 0 && (steps_host || ids_host)) {
-        const RasterList in = {net->d_ras_n, net->d_ras_step, net->d_ras_id, net->ras_cap, net->P, 1, nullptr,
-                               (uint32_t)net->ras_lo, net->ras_hi - net->ras_lo, (uint32_t)net->n};
         CK(raster_sort(&net->ras_sort, in, (size_t)total, net->stream));
         if (steps_host)
             CK(cudaMemcpyAsync(steps_host, net->ras_sort.step, sizeof(uint32_t) * got,
@@ -885,16 +908,15 @@ int snn_read_spikes(snn_net* net, uint32_t* steps_host, uint32_t* ids_host, int6
     net->ras_lo = INT64_MAX;
     net->ras_hi = 0;
     *n = got;
-    if (lost) return fail(SNN_ERR_OVERFLOW, "spike raster capacity exceeded; spikes were lost");
-    if (got < total) return fail(SNN_ERR_OVERFLOW, "cap smaller than the recorded spikes; the rest were dropped");
-    return SNN_OK;
+    return raster_overflow(lost, got < total);
 }
 
 int snn_raster_size(snn_net* net, int64_t* n) {
     if (!net || !n) return fail(SNN_ERR_INVALID, "bad arguments");
-    CK(cudaStreamSynchronize(net->stream));
-    std::vector<uint32_t> cnt(net->P);
-    CK(cudaMemcpy(cnt.data(), net->d_ras_n, sizeof(uint32_t) * net->P, cudaMemcpyDeviceToHost));
+    uint32_t cnt[kStepThreads];
+    const uint32_t* const src[1] = {net->d_ras_n};
+    uint32_t* const dst[1] = {cnt};
+    CK(read_arrays(1, src, dst, net->P, &net->stage, net->stream));
     int64_t total = 0;
     for (int c = 0; c < net->P; ++c) total += std::min<uint32_t>(cnt[c], net->ras_cap);
     *n = total;
@@ -903,6 +925,15 @@ int snn_raster_size(snn_net* net, int64_t* n) {
 
 int snn_read_state(snn_net* net, float* u_host, float* i_syn_host, int32_t* refr_host) {
     if (!net) return fail(SNN_ERR_INVALID, "net is NULL");
+    if (net->n <= kStageNeurons) {
+        const uint32_t* const src[3] = {reinterpret_cast<const uint32_t*>(net->d_u),
+                                        reinterpret_cast<const uint32_t*>(net->d_i),
+                                        reinterpret_cast<const uint32_t*>(net->d_r)};
+        uint32_t* const dst[3] = {reinterpret_cast<uint32_t*>(u_host), reinterpret_cast<uint32_t*>(i_syn_host),
+                                  reinterpret_cast<uint32_t*>(refr_host)};
+        CK(read_arrays(3, src, dst, net->n, &net->stage, net->stream));
+        return SNN_OK;
+    }
     CK(cudaStreamSynchronize(net->stream));
     if (u_host) CK(cudaMemcpy(u_host, net->d_u, sizeof(float) * net->n, cudaMemcpyDeviceToHost));
     if (i_syn_host) CK(cudaMemcpy(i_syn_host, net->d_i, sizeof(float) * net->n, cudaMemcpyDeviceToHost));
@@ -917,9 +948,10 @@ int snn_read_ring(snn_net* net, int32_t* ring_host) {
 
 int snn_counters(snn_net* net, int64_t* step, uint64_t* spikes, uint64_t* events) {
     if (!net) return fail(SNN_ERR_INVALID, "net is NULL");
-    CK(cudaStreamSynchronize(net->stream));
     unsigned long long c[2];
-    CK(cudaMemcpy(c, net->d_counters, sizeof(c), cudaMemcpyDeviceToHost));
+    const uint32_t* const src[1] = {reinterpret_cast<const uint32_t*>(net->d_counters)};
+    uint32_t* const dst[1] = {reinterpret_cast<uint32_t*>(c)};
+    CK(read_arrays(1, src, dst, 4, &net->stage, net->stream));
     if (step) *step = net->step;
     if (spikes) *spikes = c[0];
     if (events) *events = c[1];

@@ -62,6 +62,7 @@ struct snn_net {
     uint32_t* d_ras_id = nullptr;
     uint32_t* d_ras_n = nullptr;
     int32_t* d_ring_io = nullptr;           // [64][n] the ring in the ABI's layout (host copies)
+    snn::HostStage stage;                   // small reads
     snn::RasterSort ras_sort;               // workspace of the raster reads
     int64_t ras_lo = INT64_MAX, ras_hi = 0; // steps launched since the last raster read
     unsigned long long* d_counters = nullptr;

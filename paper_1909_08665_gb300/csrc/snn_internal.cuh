@@ -281,6 +281,32 @@ struct RasterSort {
     size_t step_cap = 0, id_cap = 0, group_cap = 0, key_cap = 0;
 };
 cudaError_t raster_sort(RasterSort* w, const RasterList& in, size_t n, cudaStream_t s);
+// Pinned host memory that kernels write small results into (grows, is kept).
+struct HostStage {
+    void* host = nullptr;
+    void* dev = nullptr;
+    size_t bytes = 0;
+};
+cudaError_t host_stage(HostStage* st, size_t bytes, uint32_t** host, uint32_t** dev);
+void host_stage_free(HostStage* st);
+// Counts the recorded spikes and, when they are few, reads them: done = they
+// are in step / id (host memory of the stage), sorted, and the lists cleared.
+// n_part must be below kStepThreads.  Waits for the stream.
+struct RasterSmall {
+    uint32_t n;
+    bool lost, done;
+    const uint32_t* step;
+    const uint32_t* id;
+};
+cudaError_t raster_read_small(const RasterList& in, uint32_t* counts, HostStage* stage, cudaStream_t s,
+                              RasterSmall* out);
+// `count` (1..3) device arrays of n words to the host (a null destination is
+// skipped): one launch and one wait, instead of a wait and a copy call of 13
+// us for each; used up to kStageNeurons words, where the transfer itself takes
+// less than that.  Waits for the stream.
+constexpr int kStageNeurons = 32768;
+cudaError_t read_arrays(int count, const uint32_t* const* dev_src, uint32_t* const* host_dst, int n,
+                        HostStage* stage, cudaStream_t s);
 void raster_sort_free(RasterSort* w);
 // the ring [n_part][kRing][ncmax] into slot-major abi [kRing][n], or back
 cudaError_t launch_ring_layout(const int32_t* part_lo, int n_part, int ncmax, int n, int32_t* ring,
