@@ -433,6 +433,13 @@ int snn_grad_set_trace_budget(snn_net* net, int64_t bytes);
  * the fastest, and resets every instance to its initial state.
  * snn_batch_get_info reports the probe times and the chosen per-step time.
  *
+ * Where every instance's partitions fit on the GPU at once (up to 4096 neurons
+ * per SM), the instances run as networks of their own side by side in one
+ * launch, each waiting only for itself; with up to 512 neurons per SM that
+ * form is taken without further trials, with more it is one more candidate.
+ * snn_batch_set_tiling ends it for the batch: the steps issued after the call
+ * use the tilings.
+ *
  * Steps are issued as replays of one captured CUDA graph of 1000 steps; the
  * kernel reads its first step index from device memory and advances it, so
  * replays need no parameter update.  Remainders (n_steps mod 1000) use a
@@ -462,9 +469,11 @@ typedef struct snn_batch_info {
  *   cfgs[n_inst], seeds[n_inst]   host arrays, read during the call
  *   opt                           may be NULL; raster_capacity is the total
  *                                 raster capacity of the batch (default
- *                                 64 Mi spikes), timeout_s the barrier limit,
- *                                 inject_fault = 1 makes CTA 0 skip its
- *                                 barrier arrivals (tests the bounded wait:
+ *                                 64 Mi spikes; side by side, a partition
+ *                                 takes up to four times its share),
+ *                                 timeout_s the barrier limit,
+ *                                 inject_fault = 1 makes CTA 0 withhold its
+ *                                 arrivals (tests the bounded wait:
  *                                 snn_batch_sync then reports
  *                                 SNN_ERR_TIMEOUT); n_part is ignored
  *   stream                        cudaStream_t of all the batch's work

@@ -14,7 +14,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libsnn_gb300.so")
 SOURCES = ["capi.cu", "build_net.cu", "step.cu", "step_mode_plain.cu", "step_mode_paced.cu",
-           "step_mode_sat.cu", "step_mode_sat_paced.cu", "noalloc.cu", "batch.cu", "grad.cu",
+           "step_mode_sat.cu", "step_mode_sat_paced.cu", "step_multi.cu", "noalloc.cu", "batch.cu", "grad.cu",
            "adjoint_part.cu", "deliver_cluster.cu", "deliver_words.cu", "deliver_stream.cu",
            "raster_sort.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

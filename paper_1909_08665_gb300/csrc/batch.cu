@@ -3,6 +3,11 @@
 // Sec. 3.1.2 ring buffers, Sec. 3.1.3 per-step processing), replayed from a
 // captured CUDA graph.
 //
+// Two forms.  Where all instances' partitions are co-resident they run side by
+// side through the step kernel (step_multi.cu; plan_parts, setup_parts below).
+// Larger batches, and batches for which a tiling was asked, run through
+// k_batch:
+//
 // The neurons of all instances are concatenated: instance k owns the global
 // range [goff_k, goff_k + n_k).  CTA b owns the contiguous range
 // [b * chunk, (b + 1) * chunk), chunk = ceil(total / CTAs) <= 512 NPT, and keeps u, I and the refractory
@@ -41,6 +46,7 @@
 #include <vector>
 
 #include "../../include/snn.h"
+#include "net.h"
 #include "snn_internal.cuh"
 
 namespace snn {
@@ -566,6 +572,16 @@ __global__ void __launch_bounds__(kBThreads) k_probe_deliver(const __grid_consta
     }
 }
 
+// ring buffers of one instance, from the partitioned form's slot-major copy
+// [64][n] (slot = step mod 64) to the batch's [depth][ntot] (slot = step mod
+// depth); no input lies beyond the longest delay
+__global__ void __launch_bounds__(256) k_ring_to_batch(const int32_t* src, int n, long long t, int depth,
+                                                       int32_t* dst, size_t ntot) {
+    for (int d = blockIdx.y; d < depth; d += gridDim.y)
+        for (int i = blockIdx.x * 256 + threadIdx.x; i < n; i += gridDim.x * 256)
+            dst[(size_t)((t + d) % depth) * ntot + i] = src[(size_t)((t + d) & (kRing - 1)) * n + i];
+}
+
 constexpr int kNptVariants[] = {1, 2, 4, 6, 8, 12, 16};
 
 template <int NPT>
@@ -639,6 +655,21 @@ struct snn_batch {
     bool ras_new = false;                // steps were issued since the last drain
     std::vector<float2> u0_range;        // default initial potentials per instance
     float trial_us = 0.f;                // per-step time of the chosen assignment
+    // the partitioned form (step_multi.cu): every instance a network of its own
+    // partitions, all of them co-resident; d_u, d_i, d_r, the raster and the
+    // counters are the batch's
+    std::vector<snn_net*> nets;          // empty: does not fit
+    bool part = false;                   // steps run in this form
+    int part_npt = 0, part_grid = 0;
+    bool part_smem_ring = false;
+    size_t part_smem = 0, part_ring_words = 0, part_msg_words = 0;
+    uint32_t part_cap = 0;               // raster capacity of a partition
+    std::vector<size_t> part_ring_off;   // of each instance, words
+    StepParams* d_part = nullptr;        // [n_inst]
+    int32_t* d_part_first = nullptr;     // [n_inst + 1] first CTA of each instance
+    int32_t* d_part_ring = nullptr;      // [partition][64][ncmax of its instance]
+    unsigned long long* d_part_msg = nullptr;
+    uint32_t* d_part_n = nullptr;        // [part_grid] recorded spikes
 };
 
 namespace {
@@ -668,9 +699,12 @@ int balloc(T** p, size_t n, const char* what) {
 void free_batch(snn_batch* b) {
     if (!b) return;
     if (b->graph) cudaGraphExecDestroy(b->graph);
-    for (auto* x : b->row_start) cudaFree(x);
-    for (auto* x : b->words) cudaFree(x);
-    void* ptrs[] = {b->d_wtab_all, b->d_ps_all, b->d_hot, b->d_cold, b->d_pois, b->d_cdc, b->d_goff, b->d_u, b->d_i,
+    for (snn_net* net : b->nets) snn_destroy(net);      // they own the rows
+    if (b->nets.empty()) {
+        for (auto* x : b->row_start) cudaFree(x);
+        for (auto* x : b->words) cudaFree(x);
+    }
+    void* ptrs[] = {b->d_part, b->d_part_first, b->d_part_ring, b->d_part_msg, b->d_part_n, b->d_wtab_all, b->d_ps_all, b->d_hot, b->d_cold, b->d_pois, b->d_cdc, b->d_goff, b->d_u, b->d_i,
                     b->d_r, b->d_ring, b->d_list, b->d_cnt, b->d_ras_step, b->d_ras_id,
                     b->d_ras_n, b->d_ic, b->d_step, b->d_sync};
     for (void* x : ptrs)
@@ -696,6 +730,11 @@ cudaError_t launch_batch(snn_batch* b, int n_steps) {
     void* args[] = {&p};
     cudaError_t e = cudaMemsetAsync(b->d_sync, 0, sizeof(uint32_t), b->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(b->d_sync + 2, 0, sizeof(uint32_t), b->stream);
+    if (b->part)
+        return e != cudaSuccess ? e
+                                : launch_step_multi(b->part_npt, b->part_smem_ring, b->part_smem, b->part_grid,
+                                                    b->d_part, b->d_part_first, b->n_inst, b->d_step, n_steps,
+                                                    b->stream);
     if (e == cudaSuccess) e = cudaLaunchKernelExC(&cfg, select_batch(b->npt), args);
     return e;
 }
@@ -769,6 +808,12 @@ cudaError_t reset_state(snn_batch* b) {
     if (e == cudaSuccess) e = cudaMemsetAsync(b->d_ic, 0, sizeof(unsigned long long) * 2 * b->n_inst, s);
     if (e == cudaSuccess) e = cudaMemsetAsync(b->d_step, 0, sizeof(long long), s);
     if (e == cudaSuccess) e = cudaMemsetAsync(b->d_sync, 0, sizeof(uint32_t) * 4, s);
+    if (e == cudaSuccess && !b->nets.empty()) {
+        // (message tags count steps: the rewound run must not meet old ones)
+        e = cudaMemsetAsync(b->d_part_ring, 0, sizeof(int32_t) * b->part_ring_words, s);
+        if (e == cudaSuccess) e = cudaMemsetAsync(b->d_part_msg, 0, sizeof(unsigned long long) * b->part_msg_words, s);
+        if (e == cudaSuccess) e = cudaMemsetAsync(b->d_part_n, 0, sizeof(uint32_t) * b->part_grid, s);
+    }
     for (int k = 0; k < b->n_inst && e == cudaSuccess; ++k) {
         const InstHot& H = b->hot_h[k];
         e = launch_init_state((int)H.key.w, H.key.x, H.key.y, b->u0_range[k].x, b->u0_range[k].y,
@@ -805,13 +850,20 @@ int batch_trials(snn_batch* b) {
                 cand.push_back(a);
             }
     }
+    // The partitioned form, where the instances fit, is one more candidate;
+    // with one neuron per thread the only one (it takes 1.7 to 2.6 us per step
+    // there, a step of the other form never below 5).
+    const size_t n_cand = b->nets.empty() ? cand.size() : b->part_npt == 1 ? 1 : cand.size() + 1;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     BCK(cudaEventCreate(&e0));
     BCK(cudaEventCreate(&e1));
     float best = 1e30f;
     size_t best_c = 0;
+    bool best_part = false;
     cudaError_t e = cudaSuccess;
-    for (size_t c = 0; c < cand.size() && e == cudaSuccess; ++c) {
+    for (size_t x = 0; x < n_cand && e == cudaSuccess; ++x) {
+        b->part = !b->nets.empty() && x == 0;
+        const size_t c = b->nets.empty() || x == 0 ? x : x - 1;
         for (int k = 0; k < K; ++k) b->hot_h[k].key.z = cand[c][k];
         e = cudaMemcpyAsync(b->d_hot, b->hot_h.data(), sizeof(InstHot) * K, cudaMemcpyHostToDevice, s);
         if (e == cudaSuccess) e = reset_state(b);
@@ -825,8 +877,10 @@ int batch_trials(snn_batch* b) {
         if (e == cudaSuccess && ms < best) {
             best = ms;
             best_c = c;
+            best_part = b->part;
         }
     }
+    b->part = best_part;
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     if (e != cudaSuccess) return set_cuda_error(e, "batch autotune trials");
@@ -840,6 +894,165 @@ int batch_trials(snn_batch* b) {
     return SNN_OK;
 }
 
+// capture one launch of kGraphChunk steps; replays advance the device step
+// counter, so no parameter changes between replays (captured on a private
+// stream: the legacy default stream cannot be captured; the graph is then
+// launched on the batch's own stream)
+int capture_graph(snn_batch* b) {
+    if (b->graph) cudaGraphExecDestroy(b->graph);
+    b->graph = nullptr;
+    b->graph_ok = false;
+    cudaStream_t s = b->stream;
+    cudaGraph_t g = nullptr;
+    cudaStream_t cs = nullptr;
+    if (cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking) == cudaSuccess) {
+        if (cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
+            b->stream = cs;
+            const cudaError_t le = launch_batch(b, kGraphChunk);
+            b->stream = s;
+            const cudaError_t ce = cudaStreamEndCapture(cs, &g);
+            if (le == cudaSuccess && ce == cudaSuccess && g &&
+                cudaGraphInstantiate(&b->graph, g, 0) == cudaSuccess)
+                b->graph_ok = true;
+            if (g) cudaGraphDestroy(g);
+        }
+        cudaStreamDestroy(cs);
+    }
+    cudaGetLastError();
+    return SNN_OK;
+}
+
+int saturation_error() {
+    return set_error(SNN_ERR_SATURATED,
+                     "a batch instance's input of one step can exceed the int32 "
+                     "fixed-point range; step it as a single network (snn_create), "
+                     "which checks for saturation");
+}
+
+// Partitions of every instance for the partitioned form, as few neurons each
+// as let all of them be co-resident (one CTA per SM; below kFewest a step is
+// no faster); false when that takes more than a partition may hold, or when
+// the configurations are not valid (reported where they are built).
+constexpr int kFewest = 160, kMostPart = 8 * kStepThreads;
+bool plan_parts(const snn_config* cfgs, int n_inst, int sms, std::vector<int>* n_part) {
+    std::vector<long long> n(n_inst, 0);
+    for (int k = 0; k < n_inst; ++k) {
+        if (cfgs[k].n_pop < 1 || cfgs[k].n_pop > kMaxPop) return false;
+        for (int p = 0; p < cfgs[k].n_pop; ++p) n[k] += cfgs[k].pop_size[p];
+        if (n[k] < 1 || n[k] > SNN_MAX_NEURONS) return false;
+    }
+    auto ctas = [&](long long size) {
+        long long c = 0;
+        for (long long x : n) c += (x + size - 1) / size;
+        return c;
+    };
+    long long lo = kFewest, hi = kMostPart;
+    if (ctas(hi) > std::min(sms, kStepThreads - 1)) return false;
+    while (lo < hi) {
+        const long long m = (lo + hi) / 2;
+        if (ctas(m) <= std::min(sms, kStepThreads - 1)) hi = m;
+        else lo = m + 1;
+    }
+    n_part->resize(n_inst);
+    for (int k = 0; k < n_inst; ++k) (*n_part)[k] = (int)((n[k] + lo - 1) / lo);
+    return true;
+}
+
+// state, messages and parameters of the partitioned form; the form is dropped
+// (b->nets stay: they own the rows) when its kernel does not fit
+int setup_parts(snn_batch* b) {
+    const int K = b->n_inst;
+    int dev = 0, optin = 0, sms = 0, ncmax = 0;
+    BCK(cudaGetDevice(&dev));
+    BCK(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+    BCK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    std::vector<int32_t> first(K + 1, 0);
+    std::vector<size_t> msg_off(K + 1, 0);
+    std::vector<int> stride(K);
+    b->part_ring_off.assign(K + 1, 0);
+    size_t with_ring = 0, bare = 0;
+    for (int k = 0; k < K; ++k) {
+        const snn_net* net = b->nets[k];
+        ncmax = std::max(ncmax, net->ncmax);
+        first[k + 1] = first[k] + net->P;
+        stride[k] = (net->ncmax + 2 + 7) / 8 * 8;
+        msg_off[k + 1] = msg_off[k] + (size_t)4 * net->P * stride[k];
+        b->part_ring_off[k + 1] = b->part_ring_off[k] + (size_t)net->P * kRing * net->ncmax;
+        with_ring = std::max(with_ring, step_shared_bytes(net->ncmax, net->P, net->w_span, true));
+        bare = std::max(bare, step_shared_bytes(net->ncmax, net->P, net->w_span, false));
+    }
+    b->part_npt = ncmax <= kStepThreads ? 1 : ncmax <= 2 * kStepThreads ? 2 : ncmax <= 4 * kStepThreads ? 4 : 8;
+    // (the kernel's parameters take static shared memory)
+    const size_t room = (size_t)optin - sizeof(StepParams) - 64;
+    b->part_smem_ring = with_ring <= room && b->part_npt <= 2;
+    b->part_smem = b->part_smem_ring ? with_ring : bare;
+    b->part_ring_words = b->part_ring_off[K];
+    b->part_msg_words = msg_off[K];
+    BCALL(balloc(&b->d_part, K, "batch partitions"));
+    BCALL(balloc(&b->d_part_first, K + 1, "batch partitions"));
+    BCALL(balloc(&b->d_part_ring, b->part_ring_words, "batch ring buffers"));
+    BCALL(balloc(&b->d_part_msg, b->part_msg_words, "batch spike messages"));
+    BCALL(balloc(&b->d_part_n, b->part_grid, "batch raster counts"));
+    std::vector<StepParams> sp(K);
+    for (int k = 0; k < K; ++k) {
+        StepParams& x = sp[k];
+        fill_step_params(b->nets[k], &x);
+        const size_t at = (size_t)b->goff[k];
+        x.u = b->d_u + at;
+        x.i_syn = b->d_i + at;
+        x.refr = b->d_r + at;
+        x.ring = b->d_part_ring + b->part_ring_off[k];
+        x.msg = b->d_part_msg + msg_off[k];
+        x.msg_stride = stride[k];
+        x.ras_step = b->d_ras_step + (size_t)first[k] * b->part_cap;
+        x.ras_id = b->d_ras_id + (size_t)first[k] * b->part_cap;
+        x.ras_n = b->d_part_n + first[k];
+        x.ras_cap = b->part_cap;
+        x.ras_id0 = (uint32_t)at;
+        x.counters = b->d_ic + 2 * k;
+        x.pop_spikes = nullptr;
+        x.status = b->d_sync + 1;
+        x.abort_flag = b->d_sync + 2;
+        x.timeout_ns = b->p.timeout_ns;
+        x.inject_fault = k == 0 ? b->p.inject_fault : 0;
+    }
+    BCK(cudaMemcpy(b->d_part, sp.data(), sizeof(StepParams) * K, cudaMemcpyHostToDevice));
+    BCK(cudaMemcpy(b->d_part_first, first.data(), sizeof(int32_t) * (K + 1), cudaMemcpyHostToDevice));
+    int per_sm = 0;
+    BCK(step_multi_configure(b->part_npt, b->part_smem_ring, b->part_smem, &per_sm));
+    if (per_sm * sms < b->part_grid) return set_error(SNN_ERR_UNSUPPORTED, "batch partitions exceed co-resident CTAs");
+    b->part = true;
+    BCK(reset_state(b));
+    return SNN_OK;
+}
+
+int drain_raster(snn_batch* b);
+
+// on to the tiled form, which steps a batch once a tiling was asked for
+int leave_parts(snn_batch* b) {
+    BCALL(drain_raster(b));
+    cudaStream_t s = b->stream;
+    int32_t* tmp = nullptr;
+    int n_most = 1;
+    for (const snn_net* net : b->nets) n_most = std::max(n_most, net->n);
+    BCALL(balloc(&tmp, (size_t)kRing * n_most, "ring staging"));
+    cudaError_t e = cudaSuccess;
+    for (int k = 0; k < b->n_inst && e == cudaSuccess; ++k) {
+        const snn_net* net = b->nets[k];
+        e = launch_ring_layout(net->d_part_lo, net->P, net->ncmax, net->n, b->d_part_ring + b->part_ring_off[k], tmp,
+                               true, s);
+        if (e != cudaSuccess) break;
+        k_ring_to_batch<<<dim3((net->n + 255) / 256, 16), 256, 0, s>>>(tmp, net->n, b->step, b->ring_depth,
+                                                                     b->d_ring + b->goff[k], (size_t)b->ntot);
+        e = cudaGetLastError();
+    }
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    cudaFree(tmp);
+    if (e != cudaSuccess) return set_cuda_error(e, "ring layout of the tiled form");
+    b->part = false;
+    return capture_graph(b);
+}
+
 // the spikes recorded since the last drain, sorted by (instance, step, id) on
 // the device, appended to each instance's host arrays
 int drain_raster(snn_batch* b) {
@@ -847,10 +1060,12 @@ int drain_raster(snn_batch* b) {
         BCK(cudaStreamSynchronize(b->stream));
         return SNN_OK;
     }
-    const RasterList in = {b->d_ras_n, b->d_ras_step, b->d_ras_id, b->ras_cap, 1, b->n_inst, b->d_goff,
-                           (uint32_t)b->ras_lo, b->step - b->ras_lo, (uint32_t)b->ntot};
+    uint32_t* counts = b->part ? b->d_part_n : b->d_ras_n;
+    const int lists = b->part ? b->part_grid : 1;
+    const RasterList in = {counts, b->d_ras_step, b->d_ras_id, b->part ? b->part_cap : b->ras_cap, lists,
+                           b->n_inst, b->d_goff, (uint32_t)b->ras_lo, b->step - b->ras_lo, (uint32_t)b->ntot};
     RasterSmall small;
-    BCK(raster_read_small(in, b->d_ras_n, &b->stage, b->stream, &small));
+    BCK(raster_read_small(in, counts, &b->stage, b->stream, &small));
     const uint32_t m = small.n;
     std::vector<uint32_t> st(m), id(m);
     if (small.done) {
@@ -860,7 +1075,7 @@ int drain_raster(snn_batch* b) {
         BCK(raster_sort(&b->ras_sort, in, m, b->stream));
         BCK(cudaMemcpyAsync(st.data(), b->ras_sort.step, sizeof(uint32_t) * m, cudaMemcpyDeviceToHost, b->stream));
         BCK(cudaMemcpyAsync(id.data(), b->ras_sort.id, sizeof(uint32_t) * m, cudaMemcpyDeviceToHost, b->stream));
-        BCK(cudaMemsetAsync(b->d_ras_n, 0, sizeof(uint32_t), b->stream));
+        BCK(cudaMemsetAsync(counts, 0, sizeof(uint32_t) * lists, b->stream));
         BCK(cudaStreamSynchronize(b->stream));
     }
     b->ras_new = false;
@@ -911,6 +1126,8 @@ int snn_batch_create(const snn_config* cfgs, const uint64_t* seeds, int32_t n_in
     std::vector<int32_t> ps_all((size_t)n_inst * 8);
     int rc = SNN_OK;
     long long ntot = 0;
+    std::vector<int> n_part;
+    const bool parts = plan_parts(cfgs, n_inst, prop.multiProcessorCount, &n_part);
     for (int k = 0; k < n_inst && rc == SNN_OK; ++k) {
         HostTables ht;
         rc = host_tables(&cfgs[k], &ht);
@@ -936,15 +1153,29 @@ int snn_batch_create(const snn_config* cfgs, const uint64_t* seeds, int32_t n_in
         unsigned long long* rs = nullptr;
         uint32_t* wd = nullptr;
         uint64_t nnz = 0;
-        rc = build_rows_device(&cfgs[k], seeds[k], s, &rs, &wd, &nnz);
-        if (rc != SNN_OK) break;
+        if (parts) {
+            snn_net* net = nullptr;
+            rc = net_build_rows(&cfgs[k], seeds[k], s, n_part[k], &net);
+            if (rc != SNN_OK) break;
+            b->nets.push_back(net);
+            rs = net->d_row_start;
+            wd = net->d_words;
+            nnz = net->nnz;
+        } else {
+            rc = build_rows_device(&cfgs[k], seeds[k], s, &rs, &wd, &nnz);
+            if (rc != SNN_OK) break;
+        }
         b->row_start.push_back(rs);
         b->words.push_back(wd);
         b->nnz[k] = nnz;
         // the batch kernel adds in plain int32: refuse an instance whose input
         // of one step could leave that range (snn_create counts wrap-arounds
         // for such networks instead)
-        {
+        if (parts && b->nets.back()->sat_check) {
+            rc = saturation_error();
+            break;
+        }
+        if (!parts) {
             uint32_t* d_in = nullptr;
             std::vector<uint32_t> indeg((size_t)ht.n * kMaxPop);
             cudaError_t e = cudaMalloc(&d_in, sizeof(uint32_t) * std::max<size_t>(indeg.size(), 1));
@@ -960,10 +1191,7 @@ int snn_batch_create(const snn_config* cfgs, const uint64_t* seeds, int32_t n_in
             }
             if (input_bound(indeg.data(), ht.n, ht.n_pop, ht.pop_start, ht.wtab, ht.wext_q,
                             ht.mode) > 2147483647ll) {
-                rc = set_error(SNN_ERR_SATURATED,
-                               "a batch instance's input of one step can exceed the int32 "
-                               "fixed-point range; step it as a single network (snn_create), "
-                               "which checks for saturation");
+                rc = saturation_error();
                 break;
             }
         }
@@ -1018,6 +1246,14 @@ int snn_batch_create(const snn_config* cfgs, const uint64_t* seeds, int32_t n_in
     }
     const long long cap = (opt && opt->raster_capacity > 0) ? opt->raster_capacity : (64ll << 20);
     b->ras_cap = (uint32_t)std::min<long long>(cap, 0x7fffffff);
+    long long ras_words = b->ras_cap;
+    if (parts) {
+        // a list per partition; four times its share of the capacity each, as
+        // the populations' rates differ
+        for (int P : n_part) b->part_grid += P;
+        b->part_cap = (uint32_t)std::min<long long>(std::max<long long>(4 * (long long)b->ras_cap / b->part_grid, 1), b->ras_cap);
+        ras_words = std::max<long long>(ras_words, (long long)b->part_cap * b->part_grid);
+    }
     if (rc == SNN_OK) rc = balloc(&b->d_hot, n_inst, "batch instance constants");
     if (rc == SNN_OK) rc = balloc(&b->d_cold, n_inst, "batch instance rows");
     if (rc == SNN_OK) rc = balloc(&b->d_pois, pois.size(), "batch background tables");
@@ -1029,8 +1265,8 @@ int snn_batch_create(const snn_config* cfgs, const uint64_t* seeds, int32_t n_in
     if (rc == SNN_OK) rc = balloc(&b->d_ring, (size_t)b->ring_depth * ntot, "batch ring buffers");
     if (rc == SNN_OK) rc = balloc(&b->d_list, (size_t)2 * kTilings * ntot, "batch spike lists");
     if (rc == SNN_OK) rc = balloc(&b->d_cnt, 4 * kTilings, "batch list counters");
-    if (rc == SNN_OK) rc = balloc(&b->d_ras_step, b->ras_cap, "batch raster");
-    if (rc == SNN_OK) rc = balloc(&b->d_ras_id, b->ras_cap, "batch raster");
+    if (rc == SNN_OK) rc = balloc(&b->d_ras_step, ras_words, "batch raster");
+    if (rc == SNN_OK) rc = balloc(&b->d_ras_id, ras_words, "batch raster");
     if (rc == SNN_OK) rc = balloc(&b->d_ras_n, 1, "batch raster count");
     if (rc == SNN_OK) rc = balloc(&b->d_ic, (size_t)2 * n_inst, "batch counters");
     if (rc == SNN_OK) rc = balloc(&b->d_step, 1, "batch step");
@@ -1102,33 +1338,14 @@ int snn_batch_create(const snn_config* cfgs, const uint64_t* seeds, int32_t n_in
         free_batch(b);
         return set_error(SNN_ERR_CUDA, "probe kernel shared memory");
     }
-    rc = autotune(b);
+    if (parts) rc = setup_parts(b);
+    if (rc == SNN_OK) rc = autotune(b);
     if (rc == SNN_OK && !(opt && opt->inject_fault)) rc = batch_trials(b);
     if (rc != SNN_OK) {
         free_batch(b);
         return rc;
     }
-    // capture one launch of kGraphChunk steps; replays advance the device
-    // step counter, so no parameter changes between replays
-    // (captured on a private stream: the legacy default stream cannot be
-    // captured; the graph is then launched on the batch's own stream)
-    cudaGraph_t g = nullptr;
-    cudaStream_t cs = nullptr;
-    b->graph_ok = false;
-    if (cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking) == cudaSuccess) {
-        if (cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
-            b->stream = cs;
-            const cudaError_t le = launch_batch(b, kGraphChunk);
-            b->stream = s;
-            const cudaError_t ce = cudaStreamEndCapture(cs, &g);
-            if (le == cudaSuccess && ce == cudaSuccess && g &&
-                cudaGraphInstantiate(&b->graph, g, 0) == cudaSuccess)
-                b->graph_ok = true;
-            if (g) cudaGraphDestroy(g);
-        }
-        cudaStreamDestroy(cs);
-    }
-    cudaGetLastError();
+    BCALL(capture_graph(b));
     *out = b;
     return SNN_OK;
 }
@@ -1228,9 +1445,9 @@ int snn_batch_get_info(snn_batch* b, int32_t k, snn_batch_info* info) {
     info->tune_us_block = b->tune_us[1][k];
     info->tune_us_flat = b->tune_us[2][k];
     info->trial_us_per_step = b->trial_us;
-    info->blocks = b->blocks;
+    info->blocks = b->part ? b->part_grid : b->blocks;
     info->threads = kBThreads;
-    info->neurons_per_thread = b->npt;
+    info->neurons_per_thread = b->part ? b->part_npt : b->npt;
     info->graph = b->graph_ok ? 1 : 0;
     info->graph_steps = kGraphChunk;
     return SNN_OK;
@@ -1240,6 +1457,7 @@ int snn_batch_set_tiling(snn_batch* b, int32_t k, int32_t tiling) {
     if (!b || k < 0 || k >= b->n_inst || tiling < 0 || tiling >= kTilings)
         return set_error(SNN_ERR_INVALID, "bad arguments");
     b->hot_h[k].key.z = (uint32_t)tiling;
+    if (b->part) BCALL(leave_parts(b));
     BCK(cudaMemcpyAsync(b->d_hot + k, &b->hot_h[k], sizeof(InstHot), cudaMemcpyHostToDevice,
                         b->stream));
     BCK(cudaStreamSynchronize(b->stream));

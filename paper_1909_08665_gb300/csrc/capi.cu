@@ -557,6 +557,35 @@ int host_tables(const snn_config* cfg, HostTables* out) {
     return SNN_OK;
 }
 
+int net_build_rows(const snn_config* cfg, uint64_t seed, cudaStream_t stream, int n_part, snn_net** out) {
+    CALL(validate(cfg));
+    snn_net* net = new snn_net();
+    net->cfg = *cfg;
+    net->seed = seed;
+    net->stream = stream;
+    net->n_pop = cfg->n_pop;
+    net->pop_start[0] = 0;
+    for (int p = 0; p < kMaxPop; ++p)
+        net->pop_start[p + 1] = net->pop_start[p] + (p < cfg->n_pop ? cfg->pop_size[p] : 0);
+    net->n = net->pop_start[cfg->n_pop];
+    net->P = n_part;
+    net->part_lo.resize(n_part + 1);
+    net->ncmax = 0;
+    for (int c = 0; c <= n_part; ++c) {
+        net->part_lo[c] = (int32_t)(((long long)c * net->n) / n_part);
+        if (c) net->ncmax = std::max(net->ncmax, net->part_lo[c] - net->part_lo[c - 1]);
+    }
+    net->w_span = partition_pop_span(net->part_lo.data(), n_part, net->pop_start, net->n_pop);
+    int rc = make_tables(net);
+    if (rc == SNN_OK) rc = build_generated(net);
+    if (rc != SNN_OK) {
+        free_net(net);
+        return rc;
+    }
+    *out = net;
+    return SNN_OK;
+}
+
 int build_rows_device(const snn_config* cfg, uint64_t seed, cudaStream_t stream,
                       unsigned long long** row_start, uint32_t** words, uint64_t* nnz) {
     CALL(validate(cfg));

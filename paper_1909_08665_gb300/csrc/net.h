@@ -93,6 +93,9 @@ int net_ring_to_host(snn_net* net, int32_t* host);
 int net_ring_from_host(snn_net* net, const int32_t* host);
 // zero the wrap counts (after the ring was replaced: load, restore)
 cudaError_t net_clear_wraps(snn_net* net);
+// a network's rows in `n_part` partitions and what the step kernel reads of
+// them, without state, messages or raster (a member of a batch)
+int net_build_rows(const snn_config* cfg, uint64_t seed, cudaStream_t stream, int n_part, snn_net** out);
 // launch the step kernel for n steps from step t0 with the given parameters
 cudaError_t net_launch(snn_net* net, StepParams& sp, int64_t t0, int64_t n);
 void free_grad(snn_grad* g);

@@ -177,6 +177,7 @@ struct StepParams {
     uint32_t* ras_step;                 // [n_part][ras_cap]
     uint32_t* ras_id;
     uint32_t* ras_n;                    // [n_part] spikes recorded (may exceed cap)
+    uint32_t ras_id0;                   // added to the recorded ids
     unsigned long long* counters;       // [0] spikes, [1] synaptic events
     unsigned long long* pop_spikes;     // [8] spikes per population
     uint32_t* status;
@@ -388,6 +389,12 @@ cudaError_t launch_adjoint_part(const AdjPartPlan& plan, AdjPartParams& ap, cuda
 cudaError_t launch_adjoint_part_fold(int n, int n_part, int n_pop, const int32_t* part_lo,
                                      const int32_t* pop_start, const double* gAc, double* gA,
                                      cudaStream_t s);
+// The step kernel over several networks in one launch (step_multi.cu): CTA b
+// runs partition b - first[k] of network k, first[k] <= b < first[k + 1], from
+// step *step on; *step is advanced afterwards.
+cudaError_t step_multi_configure(int npt, bool smem_ring, size_t smem, int* blocks_per_sm);
+cudaError_t launch_step_multi(int npt, bool smem_ring, size_t smem, int grid, const StepParams* params,
+                              const int32_t* first, int n_net, long long* step, int n_steps, cudaStream_t s);
 // stand-alone delivery through the step kernel's runs (one CTA per partition)
 cudaError_t launch_deliver_part(const StepParams& sp, const uint32_t* spikes, int n, int64_t t,
                                 bool smem_ring, cudaStream_t s);

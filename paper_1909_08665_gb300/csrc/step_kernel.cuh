@@ -530,19 +530,17 @@ __device__ __forceinline__ void barrier_wait(int id, int n) {
     asm volatile("barrier.cta.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
 }
 
+// One CTA's steps: partition c of the network sp describes.
 template <int NPT, bool SMEM_RING, int MODE>
-__global__ void __launch_bounds__(kStepThreads, 1)
-k_step(const __grid_constant__ StepParams sp) {
+__device__ __forceinline__ void step_body(const StepParams& sp, const int c, unsigned char* smem) {
     constexpr bool PACED = (MODE & kModePaced) != 0;
     constexpr bool SAT = (MODE & kModeSat) != 0;
     // early run lookups keep 2 x kInline more registers live until the delivery:
     // not in the widest variant (us per step without / with: 1.3x 3.44 / 3.12,
     // 2x 4.78 / 4.46, 4x 8.23 / 8.15)
     constexpr bool EARLY = NPT <= 4;
-    extern __shared__ __align__(16) unsigned char smem[];
     const int tid = threadIdx.x;
     const int lane = tid & 31;
-    const int c = blockIdx.x;
     const int P = sp.n_part;
     const SmemLayout L = smem_layout(sp.ncmax, P, sp.w_span, SMEM_RING);
     uint32_t* s_pois = reinterpret_cast<uint32_t*>(smem + L.pois);
@@ -670,7 +668,7 @@ k_step(const __grid_constant__ StepParams sp) {
                     const uint32_t rp = ras_base + pos;
                     if (rp < sp.ras_cap) {
                         sp.ras_step[(size_t)c * sp.ras_cap + rp] = (uint32_t)t;
-                        sp.ras_id[(size_t)c * sp.ras_cap + rp] = id;
+                        sp.ras_id[(size_t)c * sp.ras_cap + rp] = sp.ras_id0 + id;
                     }
                 }
             }
@@ -818,6 +816,13 @@ k_step(const __grid_constant__ StepParams sp) {
     }
     if (SAT && saturated) atomicOr(sp.status, kStatusSaturated);
     if (lane == 0 && events) atomicAdd(&sp.counters[1], events);   // per-warp counts
+}
+
+template <int NPT, bool SMEM_RING, int MODE>
+__global__ void __launch_bounds__(kStepThreads, 1)
+k_step(const __grid_constant__ StepParams sp) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    step_body<NPT, SMEM_RING, MODE>(sp, (int)blockIdx.x, smem);
 }
 
 // the kernel of one MODE for a launch shape (neurons per thread, ring in
