@@ -75,6 +75,8 @@ struct snn_grad {
     uint32_t* pre = nullptr;        // pre-decoded rows of the adjoint gather (small networks)
     bool part_planned = false;      // the partition-local adjoint was considered
     snn::AdjPartPlan* part = nullptr;   // its plan, when the network fits
+    int32_t part_ncmax = 0;         // most neurons of one of its partitions
+    int32_t* part_lo = nullptr;     // [adj_part + 1] their bounds
     float* pds = nullptr;           // [2][P][n] its partial spike adjoints
     double* gAc = nullptr;          // [P][n][8] its partial weight gradients
 };
@@ -85,7 +87,7 @@ void free_grad(snn_grad* g) {
     if (!g) return;
     void* ptrs[] = {g->ckpt, g->tr_u, g->tr_f, g->lu, g->lI, g->lring, g->mnext, g->gA, g->gN,
                     g->wbase, g->out, g->sync, g->saved, g->saved_ras, g->saved_status,
-                    g->pop_start, g->blk, g->order, g->pre};
+                    g->pop_start, g->blk, g->order, g->pre, g->part_lo};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     if (g->part) {
@@ -537,7 +539,7 @@ int snn_grad_backward(snn_net* net, const double* g_rate, double* g_alpha, doubl
     if (!g || !g->ready) return set_error(SNN_ERR_INVALID, "no gradient forward to differentiate");
     if (net->step != g->t_start + g->n_steps)
         return set_error(SNN_ERR_INVALID, "the network was stepped after the gradient forward");
-    const int n = net->n, P = net->P;
+    const int n = net->n, P = net->P, PA = net->adj_part;
     cudaStream_t s = net->stream;
     GCALL(galloc(&g->lu, n, "adjoint"));
     GCALL(galloc(&g->lI, n, "adjoint"));
@@ -591,17 +593,55 @@ int snn_grad_backward(snn_net* net, const double* g_rate, double* g_alpha, doubl
         // the partition-local gather when every CTA's share of the rows fits
         // in shared memory
         AdjPartPlan plan;
-        const int rc = adjoint_part_plan(n, net->n_pop, net->pop_start, P, net->part_lo.data(), net->ncmax,
-                                         net->nnz, net->d_row_start, net->d_pre, net->d_seg, &plan);
+        std::vector<int32_t> lo(PA + 1);
+        for (int c = 0; c <= PA; ++c) {
+            lo[c] = (int32_t)(((long long)c * n) / PA);
+            if (c) g->part_ncmax = std::max(g->part_ncmax, lo[c] - lo[c - 1]);
+        }
+        GCALL(galloc(&g->part_lo, PA + 1, "adjoint partitions"));
+        GCK(cudaMemcpy(g->part_lo, lo.data(), sizeof(int32_t) * (PA + 1), cudaMemcpyHostToDevice));
+        // the rows cut and decoded for these partitions, where they are not
+        // the step kernel's
+        uint32_t *seg = net->d_seg, *pre = net->d_pre;
+        if (PA != P) {
+            seg = pre = nullptr;
+            DeliverParams dp;
+            std::memset(&dp, 0, sizeof(dp));
+            dp.n = n;
+            dp.n_pop = net->n_pop;
+            dp.n_part = PA;
+            dp.ncmax = g->part_ncmax;
+            for (int p = 0; p <= kMaxPop; ++p) dp.pop_start[p] = net->pop_start[p];
+            dp.part_lo = g->part_lo;
+            dp.words = net->d_words;
+            int rc = galloc(&seg, (size_t)n * (PA + 1) + 4, "adjoint row segments");
+            if (rc == SNN_OK) rc = galloc(&pre, (size_t)net->nnz + 4, "adjoint rows");
+            cudaError_t e = cudaSuccess;
+            if (rc == SNN_OK) e = launch_seg_from_rows(net->d_row_start, net->d_words, n, g->part_lo, PA, seg, s);
+            if (rc == SNN_OK && e == cudaSuccess) e = launch_predecode(dp, net->d_row_start, pre, s);
+            if (rc == SNN_OK && e == cudaSuccess) e = cudaStreamSynchronize(s);
+            if (rc == SNN_OK && e != cudaSuccess) rc = set_cuda_error(e, "adjoint rows");
+            if (rc != SNN_OK) {
+                cudaFree(seg);
+                cudaFree(pre);
+                return rc;
+            }
+        }
+        const int rc = adjoint_part_plan(n, net->n_pop, net->pop_start, PA, lo.data(), g->part_ncmax,
+                                         net->nnz, net->d_row_start, pre, seg, &plan);
+        if (PA != P) {
+            cudaFree(seg);
+            cudaFree(pre);
+        }
         if (rc < 0) return set_error(SNN_ERR_CUDA, "partition-local adjoint plan");
         if (rc == 0) {
             g->part = new AdjPartPlan(plan);
-            GCALL(galloc(&g->pds, (size_t)2 * P * n, "adjoint partials"));
-            GCALL(galloc(&g->gAc, (size_t)P * n * kMaxPop, "gradient partials"));
+            GCALL(galloc(&g->pds, (size_t)2 * PA * n, "adjoint partials"));
+            GCALL(galloc(&g->gAc, (size_t)PA * n * kMaxPop, "gradient partials"));
         }
         g->part_planned = true;
     }
-    if (g->part) GCK(cudaMemsetAsync(g->gAc, 0, sizeof(double) * (size_t)P * n * kMaxPop, s));
+    if (g->part) GCK(cudaMemsetAsync(g->gAc, 0, sizeof(double) * (size_t)PA * n * kMaxPop, s));
     if (!g->blk) {
         // CTA row ranges with equal total row length, rows longest first
         int dev = 0, sms = 0;
@@ -696,8 +736,8 @@ int snn_grad_backward(snn_net* net, const double* g_rate, double* g_alpha, doubl
             std::memset(&pp, 0, sizeof(pp));
             pp.n = n;
             pp.n_pop = net->n_pop;
-            pp.n_part = P;
-            pp.ncmax = net->ncmax;
+            pp.n_part = PA;
+            pp.ncmax = g->part_ncmax;
             pp.len = len;
             pp.t_first = t0;
             pp.P22 = ap.P22;
@@ -707,7 +747,7 @@ int snn_grad_backward(snn_net* net, const double* g_rate, double* g_alpha, doubl
             for (int k = 0; k < kMaxPop; ++k) pp.gs[k] = ap.gs[k];
             for (int k = 0; k <= kMaxPop; ++k) pp.pop_start[k] = net->pop_start[k];
             pp.timeout_ns = ap.timeout_ns;
-            pp.part_lo = net->d_part_lo;
+            pp.part_lo = g->part_lo;
             pp.wtab = net->d_wtab;
             pp.wbase = g->wbase;
             pp.tr_u = g->tr_u + tr_off;
@@ -743,7 +783,7 @@ int snn_grad_backward(snn_net* net, const double* g_rate, double* g_alpha, doubl
         GCK(cudaLaunchKernelExC(&cfg, adj_fn, args));
     }
     if (g->part)
-        GCK(launch_adjoint_part_fold(n, P, net->n_pop, net->d_part_lo, g->pop_start, g->gAc, g->gA, s));
+        GCK(launch_adjoint_part_fold(n, PA, net->n_pop, g->part_lo, g->pop_start, g->gAc, g->gA, s));
     k_grad_reduce<<<kMaxPop * kMaxPop + 1, 512, 0, s>>>(n, net->n_pop, g->pop_start, g->gA, g->gN, g->out + kMaxPop * kMaxPop + 1,
                                      g->out);
     GCK(cudaGetLastError());

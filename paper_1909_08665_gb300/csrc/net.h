@@ -20,6 +20,7 @@ struct snn_net {
     cudaStream_t stream;
     int n, n_pop, P, ncmax, npt;
     bool smem_ring;
+    int adj_part = 1;                      // partitions of the partition-local adjoint
     size_t smem;
     int32_t pop_start[kMaxPop + 1];
     std::vector<int32_t> part_lo;
