@@ -260,8 +260,8 @@ int plan(snn_net* net, const snn_options* opt) {
     // fewer neurons per CTA those come sooner, until reading more partitions'
     // messages costs as much: us per step at scale 0.05 with 8 / 24 partitions
     // 1.71 / 1.58, at 0.1 with 16 / 48 1.74 / 1.63, at 0.2 with 31 / 64 1.82 /
-    // 1.69; at 0.37 with 57 / 76 / 152 1.87 / 1.93 / 2.08.  The adjoint keeps partitions of 512 neurons (adj_part): its
-    // sums go over them.
+    // 1.69; at 0.37 with 57 / 76 / 152 1.87 / 1.93 / 2.08.  The adjoint keeps
+    // partitions of 512 neurons (adj_part): its sums go over them.
     const int need = std::max(1, (net->n + 511) / 512);
     net->adj_part = P > 0 ? P : std::min(sms, need);
     if (P <= 0) P = std::min(sms, std::max(need, std::min(64, (net->n + 159) / 160)));

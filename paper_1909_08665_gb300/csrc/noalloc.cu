@@ -30,12 +30,13 @@
 // 1 KB per (spike, partition).  Measured, us per step at full size: 64 probes
 // over the whole row 6.07; every word of the window loaded and tested 6.34;
 // 32 probes of the window, four rows per warp at once 5.15, one row 4.48 (16
-// or 8 probes: 4.80, 4.90); 1024 threads 4.13.
+// or 8 probes: 4.80, 4.90); 1024 threads 4.13; the count published by the last
+// warp on a barrier of its own 3.91.
 //
 // What it replaced, one warp walking each spike's whole row with an L2 atomic
 // per word between two grid barriers, was bound by the chain of a row's
 // dependent loads: 130 us per step at full size, 48 us at the 10 % scale; now
-// 4.13 and 1.81.
+// 3.91 and 1.69.
 //
 // The paper has no counterpart of this entry point.
 #include <algorithm>
@@ -310,7 +311,8 @@ __global__ void __launch_bounds__(THREADS, 1) k_step_noalloc(const __grid_consta
     const NaSmem L = na_smem(p.ncmax, p.w_span, SMEM_RING);
     uint32_t* s_pois = reinterpret_cast<uint32_t*>(smem + L.pois);
     uint32_t* s_warp = reinterpret_cast<uint32_t*>(smem + L.warp);
-    // [0], [1] this CTA's spikes of even / odd launch steps, [2] abort, [3] listed rows
+    // [0], [1] this CTA's spikes of even / odd launch steps, [2] abort, [3], [4]
+    // listed rows of lists of even / odd launch steps
     volatile uint32_t* s_misc = reinterpret_cast<uint32_t*>(smem + L.misc);
     const NaList list = {reinterpret_cast<unsigned long long*>(smem + L.rs),
                          reinterpret_cast<uint32_t*>(smem + L.la),
@@ -423,7 +425,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_step_noalloc(const __grid_consta
             }
         };
         if (tid < P && my_cnt > 0u) {
-            const uint32_t at = atomicAdd(const_cast<uint32_t*>(&s_misc[3]), my_cnt);
+            const uint32_t at = atomicAdd(const_cast<uint32_t*>(&s_misc[3 + (s & 1)]), my_cnt);
             if (at + my_cnt <= (uint32_t)kNaChunk) {
 #pragma unroll
                 for (int i = 0; i < kNaInline; ++i)
@@ -432,12 +434,12 @@ __global__ void __launch_bounds__(THREADS, 1) k_step_noalloc(const __grid_consta
             }
         }
         __syncthreads();
-        const uint32_t S_fast = s_misc[3];
+        const uint32_t S_fast = s_misc[3 + (s & 1)];
+        if (tid == 0) s_misc[3 + ((s + 1) & 1)] = 0u;   // its last readers are past a barrier
         if (s_misc[2]) return false;
         if (S_fast <= (uint32_t)kNaChunk) {
             na_deliver<THREADS, SMEM_RING>(p, list, s_w, s_popo, S_fast, tb, (uint32_t)lo, (uint32_t)hi, ring, stride);
             __syncthreads();
-            if (tid == 0) s_misc[3] = 0u;
             return true;
         }
         // more than kNaChunk spikes: offsets by a block-wide scan, in chunks
@@ -447,7 +449,6 @@ __global__ void __launch_bounds__(THREADS, 1) k_step_noalloc(const __grid_consta
         uint32_t my_off = incl - my_cnt;
         for (int w = 0; w < (tid >> 5); ++w) my_off += s_warp[w];
         const uint32_t S = S_fast;
-        if (tid == 0) s_misc[3] = 0u;
         for (uint32_t base = 0; base < S; base += kNaChunk) {
             const uint32_t m = min((uint32_t)kNaChunk, S - base);
             if (tid < P) {
@@ -481,7 +482,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_step_noalloc(const __grid_consta
         unsigned long long* my_msg = p.msg + ((size_t)(s & 3) * P + c) * p.msg_stride;
         ulonglong2 h[4];
         load_head(s - 1, h);
-        // ---- A(t): membrane, threshold, publication, background draw ----
+        // ---- A(t): membrane, threshold; the spikes' message words ----
 #pragma unroll
         for (int k = 0; k < NPT; ++k) {
             const int li = tid + k * THREADS;
@@ -529,6 +530,23 @@ __global__ void __launch_bounds__(THREADS, 1) k_step_noalloc(const __grid_consta
                 }
                 if (lane == 0) ras_at[k] = atomicAdd(p.ras_n, (uint32_t)__popc(mask));
             }
+        }
+        // the count, published by the last warp once all have arrived here
+        if (tid < THREADS - 32) {
+            barrier_arrive(1, THREADS);
+        } else {
+            barrier_wait(1, THREADS);
+            if (tid == THREADS - 32) {
+                const uint32_t nsp = s_misc[s & 1];
+                s_misc[(s + 1) & 1] = 0u;       // read last in step s - 1
+                __stcg(&my_msg[0], tag | nsp);
+                spikes += nsp;
+            }
+        }
+        // ---- background counts of step t ----
+#pragma unroll
+        for (int k = 0; k < NPT; ++k) {
+            const int li = tid + k * THREADS;
             if (p.mode == 0 && li < nc) {
                 if ((t & 3) == 0 || s == 0)
                     rnd[k] = philox(make_uint4((uint32_t)(lo + li), (uint32_t)(t >> 2), kStreamPois,
@@ -544,16 +562,8 @@ __global__ void __launch_bounds__(THREADS, 1) k_step_noalloc(const __grid_consta
                 pacc[k] = kk * p.wext_q;
             }
         }
-        __syncthreads();
-        if (tid == 0) {
-            const uint32_t nsp = s_misc[s & 1];
-            // the counter of step s + 1: its readers are past a barrier (in
-            // step 0 it is still zero, and no barrier would order the store)
-            if (s > 0) s_misc[(s + 1) & 1] = 0u;
-            __stcg(&my_msg[0], tag | nsp);
-            spikes += nsp;
-        }
         // ---- D: spikes of step t - 1 ----
+        if (s == 0) __syncthreads();            // the counter's reset before step 1's adds
         if (s > 0 && !deliver(s - 1, (uint32_t)(t - 1), h)) {
             aborted = true;
             break;
@@ -600,7 +610,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_step_noalloc(const __grid_consta
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) events += __shfl_xor_sync(0xffffffffu, events, o);
     if (lane == 0 && events) atomicAdd(&p.counters[1], events);
-    if (tid == 0 && spikes) atomicAdd(&p.counters[0], spikes);
+    if (tid == THREADS - 32 && spikes) atomicAdd(&p.counters[0], spikes);
 }
 
 // one neuron per thread covers every network on the full GPU; eight take over
