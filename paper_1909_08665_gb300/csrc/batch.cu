@@ -661,7 +661,7 @@ struct snn_batch {
     std::vector<snn_net*> nets;          // empty: does not fit
     bool part = false;                   // steps run in this form
     int part_npt = 0, part_grid = 0;
-    bool part_smem_ring = false;
+    bool part_smem_ring = false, part_few = true;   // few: no instance above kFewPartsLimit partitions
     size_t part_smem = 0, part_ring_words = 0, part_msg_words = 0;
     uint32_t part_cap = 0;               // raster capacity of a partition
     std::vector<size_t> part_ring_off;   // of each instance, words
@@ -732,7 +732,7 @@ cudaError_t launch_batch(snn_batch* b, int n_steps) {
     if (e == cudaSuccess) e = cudaMemsetAsync(b->d_sync + 2, 0, sizeof(uint32_t), b->stream);
     if (b->part)
         return e != cudaSuccess ? e
-                                : launch_step_multi(b->part_npt, b->part_smem_ring, b->part_smem, b->part_grid,
+                                : launch_step_multi(b->part_npt, b->part_smem_ring, b->part_few, b->part_smem, b->part_grid,
                                                     b->d_part, b->d_part_first, b->n_inst, b->d_step, n_steps,
                                                     b->stream);
     if (e == cudaSuccess) e = cudaLaunchKernelExC(&cfg, select_batch(b->npt), args);
@@ -974,6 +974,7 @@ int setup_parts(snn_batch* b) {
     for (int k = 0; k < K; ++k) {
         const snn_net* net = b->nets[k];
         ncmax = std::max(ncmax, net->ncmax);
+        b->part_few = b->part_few && net->P <= kFewPartsLimit;
         first[k + 1] = first[k] + net->P;
         stride[k] = (net->ncmax + 2 + 7) / 8 * 8;
         msg_off[k + 1] = msg_off[k] + (size_t)4 * net->P * stride[k];
@@ -1019,7 +1020,7 @@ int setup_parts(snn_batch* b) {
     BCK(cudaMemcpy(b->d_part, sp.data(), sizeof(StepParams) * K, cudaMemcpyHostToDevice));
     BCK(cudaMemcpy(b->d_part_first, first.data(), sizeof(int32_t) * (K + 1), cudaMemcpyHostToDevice));
     int per_sm = 0;
-    BCK(step_multi_configure(b->part_npt, b->part_smem_ring, b->part_smem, &per_sm));
+    BCK(step_multi_configure(b->part_npt, b->part_smem_ring, b->part_few, b->part_smem, &per_sm));
     if (per_sm * sms < b->part_grid) return set_error(SNN_ERR_UNSUPPORTED, "batch partitions exceed co-resident CTAs");
     b->part = true;
     BCK(reset_state(b));

@@ -25,7 +25,7 @@
 #include "snn_internal.cuh"
 
 namespace snn {
-cudaError_t step_max_blocks(int npt, bool smem_ring, size_t smem, int* blocks_per_sm);
+cudaError_t step_max_blocks(int npt, bool smem_ring, bool few, size_t smem, int* blocks_per_sm);
 }
 
 using namespace snn;
@@ -289,9 +289,9 @@ int plan(snn_net* net, const snn_options* opt) {
     const size_t with_ring = step_shared_bytes(ncmax, P, net->w_span, true);
     net->smem_ring = with_ring <= (size_t)smem_max;
     net->smem = step_shared_bytes(ncmax, P, net->w_span, net->smem_ring);
-    CK(step_kernel_configure(npt, net->smem_ring, net->smem));
+    CK(step_kernel_configure(npt, net->smem_ring, P <= kFewPartsLimit, net->smem));
     int per_sm = 0;
-    CK(step_max_blocks(npt, net->smem_ring, net->smem, &per_sm));
+    CK(step_max_blocks(npt, net->smem_ring, P <= kFewPartsLimit, net->smem, &per_sm));
     if (per_sm * sms < P)
         return fail(SNN_ERR_UNSUPPORTED, "partitions exceed co-resident CTAs of the step kernel");
     const double tmo = (opt && opt->timeout_s > 0) ? opt->timeout_s : 2.0;

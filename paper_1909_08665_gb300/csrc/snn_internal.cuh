@@ -314,12 +314,14 @@ cudaError_t launch_ring_layout(const int32_t* part_lo, int n_part, int ncmax, in
                                int32_t* abi, bool to_abi, cudaStream_t s);
 cudaError_t launch_init_state(int n, uint32_t key0, uint32_t key1, float lo, float hi,
                               float* u, cudaStream_t s);
-int step_kernel_variant(int npt, bool smem_ring);
+int step_kernel_variant(int npt, bool smem_ring, bool few);
+constexpr int kFewPartsLimit = 64;   // kFewParts of the step kernel
 size_t step_shared_bytes(int ncmax, int n_part, int w_span, bool smem_ring);
 // target populations spanned by the widest of the partitions [part_lo[c],
 // part_lo[c+1]) (the rows of the weight table a CTA of the step kernel keeps)
 int partition_pop_span(const int32_t* part_lo, int n_part, const int32_t* pop_start, int n_pop);
-cudaError_t step_kernel_configure(int npt, bool smem_ring, size_t smem);
+// few: at most kFewParts partitions
+cudaError_t step_kernel_configure(int npt, bool smem_ring, bool few, size_t smem);
 cudaError_t launch_step(const StepParams& sp, int npt, bool smem_ring, size_t smem,
                         cudaStream_t s);
 cudaError_t launch_deliver(const DeliverParams& dp, int tiling, cudaStream_t s);
@@ -392,8 +394,8 @@ cudaError_t launch_adjoint_part_fold(int n, int n_part, int n_pop, const int32_t
 // The step kernel over several networks in one launch (step_multi.cu): CTA b
 // runs partition b - first[k] of network k, first[k] <= b < first[k + 1], from
 // step *step on; *step is advanced afterwards.
-cudaError_t step_multi_configure(int npt, bool smem_ring, size_t smem, int* blocks_per_sm);
-cudaError_t launch_step_multi(int npt, bool smem_ring, size_t smem, int grid, const StepParams* params,
+cudaError_t step_multi_configure(int npt, bool smem_ring, bool few, size_t smem, int* blocks_per_sm);
+cudaError_t launch_step_multi(int npt, bool smem_ring, bool few, size_t smem, int grid, const StepParams* params,
                               const int32_t* first, int n_net, long long* step, int n_steps, cudaStream_t s);
 // stand-alone delivery through the step kernel's runs (one CTA per partition)
 cudaError_t launch_deliver_part(const StepParams& sp, const uint32_t* spikes, int n, int64_t t,

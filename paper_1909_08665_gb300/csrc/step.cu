@@ -65,23 +65,23 @@ size_t step_shared_bytes(int ncmax, int n_part, int w_span, bool smem_ring) {
     return smem_layout(ncmax, n_part, w_span, smem_ring).total;
 }
 
-static const void* select_step(int npt, bool smem_ring, int mode) {
+static const void* select_step(int npt, bool smem_ring, bool few, int mode) {
     switch (mode) {
-        case 0: return step_fn_mode<0>(npt, smem_ring);
-        case kModePaced: return step_fn_mode<kModePaced>(npt, smem_ring);
-        case kModeSat: return step_fn_mode<kModeSat>(npt, smem_ring);
-        case kModeSat | kModePaced: return step_fn_mode<kModeSat | kModePaced>(npt, smem_ring);
+        case 0: return step_fn_mode<0>(npt, smem_ring, few);
+        case kModePaced: return step_fn_mode<kModePaced>(npt, smem_ring, few);
+        case kModeSat: return step_fn_mode<kModeSat>(npt, smem_ring, few);
+        case kModeSat | kModePaced: return step_fn_mode<kModeSat | kModePaced>(npt, smem_ring, few);
         default: return nullptr;
     }
 }
 
-int step_kernel_variant(int npt, bool smem_ring) {
-    return select_step(npt, smem_ring, 0) != nullptr;
+int step_kernel_variant(int npt, bool smem_ring, bool few) {
+    return select_step(npt, smem_ring, few, 0) != nullptr;
 }
 
-cudaError_t step_kernel_configure(int npt, bool smem_ring, size_t smem) {
+cudaError_t step_kernel_configure(int npt, bool smem_ring, bool few, size_t smem) {
     for (int mode = 0; mode < 4; ++mode) {
-        const void* fn = select_step(npt, smem_ring, mode);
+        const void* fn = select_step(npt, smem_ring, few, mode);
         if (!fn) return cudaErrorInvalidValue;
         const cudaError_t e =
             cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -91,10 +91,10 @@ cudaError_t step_kernel_configure(int npt, bool smem_ring, size_t smem) {
 }
 
 // co-resident CTAs per SM: the smallest of the variants' figures
-cudaError_t step_max_blocks(int npt, bool smem_ring, size_t smem, int* blocks_per_sm) {
+cudaError_t step_max_blocks(int npt, bool smem_ring, bool few, size_t smem, int* blocks_per_sm) {
     int best = 1 << 30;
     for (int mode = 0; mode < 4; ++mode) {
-        const void* fn = select_step(npt, smem_ring, mode);
+        const void* fn = select_step(npt, smem_ring, few, mode);
         if (!fn) return cudaErrorInvalidValue;
         int b = 0;
         const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, fn, kStepThreads, smem);
@@ -108,7 +108,7 @@ cudaError_t step_max_blocks(int npt, bool smem_ring, size_t smem, int* blocks_pe
 cudaError_t launch_step(const StepParams& sp, int npt, bool smem_ring, size_t smem,
                         cudaStream_t s) {
     const int mode = (sp.rt_period_ns != 0ull ? kModePaced : 0) | (sp.wrap != nullptr ? kModeSat : 0);
-    const void* fn = select_step(npt, smem_ring, mode);
+    const void* fn = select_step(npt, smem_ring, sp.n_part <= kFewParts, mode);
     if (!fn) return cudaErrorInvalidValue;
     void* args[] = {const_cast<StepParams*>(&sp)};
     return cudaLaunchCooperativeKernel(fn, dim3(sp.n_part), dim3(kStepThreads), args, smem, s);

@@ -56,7 +56,13 @@ namespace snn {
 
 constexpr int kWarps = kStepThreads / 32;
 constexpr uint32_t kStatusRasterOverflow = 2u;
-constexpr int kInline = 7;              // ids read together with a message header (64 B)
+// Ids read together with a message header: INL = 7 (64 bytes), or 3 (32 bytes)
+// where there are few partitions (kFewParts) and hardly ever more spikes in
+// one.  us per step with 7 / 3: scale 0.02 1.54 / 1.49, 0.1 1.63 / 1.59, 0.37
+// (57 partitions) 1.97 / 1.91, 0.6 (91) 2.21 / 2.36, 1 (151) 2.60 / 2.87.
+constexpr int kInline = 7;
+constexpr int kInlineFew = 3;
+constexpr int kFewParts = kFewPartsLimit;
 // A warp takes kBatchSpikes spikes at once and loads the first 32 kRunWave
 // entries of each of their runs in one wave (runs: mean 26 entries at scale 1
 // and 4, rarely above 96).  The spikes are dealt round-robin over the warps,
@@ -288,28 +294,31 @@ __device__ __forceinline__ void store_runs(const StepParams& sp, int c, const ui
         }
 }
 
-// The run bounds of one partition's first kInline spikes of step tb, looked
+// The run bounds of one partition's first INL spikes of step tb, looked
 // up from the message head as loaded before A(tb + 1): valid (ok) only if the
 // head and each of those id words already carried the tag tb + 1.
+template <int INL>
 struct EarlyRuns {
     bool ok;
-    uint32_t b[kInline], e[kInline];
+    uint32_t b[INL], e[INL];
 };
 
-__device__ __forceinline__ void early_runs(const StepParams& sp, int c, const ulonglong2 (&pre)[4],
-                                           uint32_t tag, EarlyRuns& er) {
+template <int INL>
+__device__ __forceinline__ void early_runs(const StepParams& sp, int c, const ulonglong2 (&pre)[(INL + 1) / 2],
+                                           uint32_t tag, EarlyRuns<INL>& er) {
     if (tag_of(pre[0].x) != tag) return;
-    const uint32_t g = min((uint32_t)pre[0].x, (uint32_t)kInline);
-    const unsigned long long w[kInline] = {pre[0].y, pre[1].x, pre[1].y, pre[2].x,
-                                           pre[2].y, pre[3].x, pre[3].y};
+    const uint32_t g = min((uint32_t)pre[0].x, (uint32_t)INL);
+    unsigned long long w[INL];
+#pragma unroll
+    for (int i = 0; i < INL; ++i) w[i] = (i & 1) ? pre[(i + 1) / 2].x : pre[i / 2].y;
     bool ok = true;
 #pragma unroll
-    for (int i = 0; i < kInline; ++i)
+    for (int i = 0; i < INL; ++i)
         if ((uint32_t)i < g && tag_of(w[i]) != tag) ok = false;
     if (!ok) return;
     const size_t stride = (size_t)sp.n_part + 1;
 #pragma unroll
-    for (int i = 0; i < kInline; ++i) {
+    for (int i = 0; i < INL; ++i) {
         er.b[i] = er.e[i] = 0u;
         if ((uint32_t)i < g) {
             const uint32_t* sg = sp.seg + (size_t)(uint32_t)w[i] * stride + c;
@@ -324,13 +333,14 @@ __device__ __forceinline__ void early_runs(const StepParams& sp, int c, const ul
 // delivery of the spikes of step tb (message tag tb+1) into this CTA's ring;
 // returns false if a wait timed out or another CTA aborted
 // ---------------------------------------------------------------------------
-template <bool SAT>
+template <bool SAT, int INL>
 __device__ __forceinline__ bool deliver_list(const StepParams& sp, unsigned char* smem,
                                              const SmemLayout& L, int c, uint32_t wbase,
                                              int64_t tb, int par, int32_t* ring, int32_t* wrap,
                                              unsigned long long& events,
-                                             const ulonglong2 (&pre)[4],
-                                             const EarlyRuns& early) {
+                                             const ulonglong2 (&pre)[(INL + 1) / 2],
+                                             const EarlyRuns<INL>& early) {
+    constexpr int kHead = (INL + 1) / 2;             // 16-byte vectors of a message head
     const int tid = threadIdx.x;
     const int P = sp.n_part;
     const int list = (int)(tb & 3);
@@ -360,19 +370,21 @@ __device__ __forceinline__ bool deliver_list(const StepParams& sp, unsigned char
         }
     };
 
-    // 1. every partition's 64-byte message head: the header word (the wait and
-    //    the spike count at once) and the first kInline ids.  pre[] is the
+    // 1. every partition's message head: the header word (the wait and the
+    //    spike count at once) and the first INL ids.  pre[] is the
     //    head as loaded by the caller, early; a stale head is polled again.
     uint32_t cnt[1] = {0u};
     const unsigned long long* m_mine = msg + (size_t)tid * sp.msg_stride;
     if (tid < P) {
-        ulonglong2 h[4] = {pre[0], pre[1], pre[2], pre[3]};
+        ulonglong2 h[kHead];
+#pragma unroll
+        for (int q = 0; q < kHead; ++q) h[q] = pre[q];
         if (tag_of(h[0].x) != tag) {
             uint64_t t_start = globaltimer_ns();
             uint32_t iter = 0;
             do {
 #pragma unroll
-                for (int q = 0; q < 4; ++q)
+                for (int q = 0; q < kHead; ++q)
                     h[q] = __ldcg(reinterpret_cast<const ulonglong2*>(m_mine + 2 * q));
                 if ((++iter & 31u) == 0u) {
                     if (ld_relaxed_gpu(sp.abort_flag) != 0u ||
@@ -388,11 +400,11 @@ __device__ __forceinline__ bool deliver_list(const StepParams& sp, unsigned char
             } while (tag_of(h[0].x) != tag);
         }
         cnt[0] = (uint32_t)h[0].x;
-        s_inl[tid * kInline + 0] = h[0].y;
+        s_inl[tid * INL + 0] = h[0].y;
 #pragma unroll
-        for (int q = 1; q < 4; ++q) {
-            s_inl[tid * kInline + 2 * q - 1] = h[q].x;
-            s_inl[tid * kInline + 2 * q] = h[q].y;
+        for (int q = 1; q < kHead; ++q) {
+            s_inl[tid * INL + 2 * q - 1] = h[q].x;
+            s_inl[tid * INL + 2 * q] = h[q].y;
         }
     }
     const uint32_t my_cnt = cnt[0];
@@ -405,26 +417,26 @@ __device__ __forceinline__ bool deliver_list(const StepParams& sp, unsigned char
         if (at + my_cnt <= (uint32_t)kChunk) {
             if (early.ok) {                          // bounds looked up during A(tb + 1)
 #pragma unroll
-                for (int i = 0; i < kInline; ++i)
+                for (int i = 0; i < INL; ++i)
                     if ((uint32_t)i < my_cnt) {
                         s_rb[at + i] = early.b[i];
                         s_rl[at + i] = early.e[i] - early.b[i];
                     }
             } else {
-                uint32_t ids[kInline];
+                uint32_t ids[INL];
 #pragma unroll
-                for (int i = 0; i < kInline; ++i) {
+                for (int i = 0; i < INL; ++i) {
                     ids[i] = 0u;                     // in range if a wait gives up
                     if ((uint32_t)i < my_cnt) {
-                        unsigned long long e = s_inl[tid * kInline + i];
+                        unsigned long long e = s_inl[tid * INL + i];
                         if (poll_word(sp, m_mine + 1 + i, tag, e)) ids[i] = (uint32_t)e;
                         else s_misc[2] = 1u;
                     }
                 }
-                store_runs<kInline>(sp, c, ids, min(my_cnt, (uint32_t)kInline), s_rb + at,
+                store_runs<INL>(sp, c, ids, min(my_cnt, (uint32_t)INL), s_rb + at,
                                     s_rl + at);
             }
-            for (uint32_t i = kInline; i < my_cnt; i += 8) {
+            for (uint32_t i = INL; i < my_cnt; i += 8) {
                 ulonglong2 v[4];                     // entries 1+i.. are 16-B aligned
 #pragma unroll
                 for (int q = 0; q < 4; ++q)
@@ -477,7 +489,7 @@ __device__ __forceinline__ bool deliver_list(const StepParams& sp, unsigned char
                     ids8[q] = 0u;                    // in range if a wait gives up
                     if (k < i1) {
                         const unsigned long long* mp = m_mine + 1 + k;
-                        unsigned long long e = k < (uint32_t)kInline ? s_inl[tid * kInline + k] : __ldcg(mp);
+                        unsigned long long e = k < (uint32_t)INL ? s_inl[tid * INL + k] : __ldcg(mp);
                         if (poll_word(sp, mp, tag, e)) ids8[q] = (uint32_t)e;
                         else s_misc[2] = 1u;
                     }
@@ -531,11 +543,12 @@ __device__ __forceinline__ void barrier_wait(int id, int n) {
 }
 
 // One CTA's steps: partition c of the network sp describes.
-template <int NPT, bool SMEM_RING, int MODE>
+template <int NPT, bool SMEM_RING, int MODE, int INL>
 __device__ __forceinline__ void step_body(const StepParams& sp, const int c, unsigned char* smem) {
+    constexpr int kHead = (INL + 1) / 2;
     constexpr bool PACED = (MODE & kModePaced) != 0;
     constexpr bool SAT = (MODE & kModeSat) != 0;
-    // early run lookups keep 2 x kInline more registers live until the delivery:
+    // early run lookups keep 2 x INL more registers live until the delivery:
     // not in the widest variant (us per step without / with: 1.3x 3.44 / 3.12,
     // 2x 4.78 / 4.46, 4x 8.23 / 8.15)
     constexpr bool EARLY = NPT <= 4;
@@ -615,13 +628,13 @@ __device__ __forceinline__ void step_body(const StepParams& sp, const int c, uns
         uint32_t* my_cnt = &s_misc[s & 1];
         // headers of step t-1 were published one step ago: load them now so
         // the round trip overlaps A(t)
-        ulonglong2 pre[4];
+        ulonglong2 pre[kHead];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) pre[q] = make_ulonglong2(0ull, 0ull);
+        for (int q = 0; q < kHead; ++q) pre[q] = make_ulonglong2(0ull, 0ull);
         if (s > 0 && tid < P) {
             const unsigned long long* m = sp.msg + ((size_t)((t - 1) & 3) * P + tid) * sp.msg_stride;
 #pragma unroll
-            for (int q = 0; q < 4; ++q) pre[q] = __ldcg(reinterpret_cast<const ulonglong2*>(m + 2 * q));
+            for (int q = 0; q < kHead; ++q) pre[q] = __ldcg(reinterpret_cast<const ulonglong2*>(m + 2 * q));
         }
         // ---- A(t): membrane, threshold, compaction, publication ----
 #pragma unroll
@@ -718,12 +731,12 @@ __device__ __forceinline__ void step_body(const StepParams& sp, const int c, uns
         // header thread already holds (the head loaded before A(t), arrived
         // by now): looked up here, so that they return while the CTA meets
         // at the barrier and the header is published
-        EarlyRuns early;
+        EarlyRuns<INL> early;
         early.ok = false;
         if (EARLY && s > 0 && tid < P) early_runs(sp, c, pre, (uint32_t)t, early);
         // ---- D: spikes of step t-1 ----
         if (s > 0) {
-            if (!deliver_list<SAT>(
+            if (!deliver_list<SAT, INL>(
                     sp, smem, L, c, wt_base, t - 1, s & 1, ring, wrap, events, pre, early)) {
                 aborted = true;
                 break;
@@ -785,17 +798,17 @@ __device__ __forceinline__ void step_body(const StepParams& sp, const int c, uns
     // ---- epilogue: deliver the spikes of the last step ----
     if (!aborted && sp.n_steps > 0) {
         const int64_t tl = sp.t0 + sp.n_steps - 1;
-        ulonglong2 pre[4];
+        ulonglong2 pre[kHead];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) pre[q] = make_ulonglong2(0ull, 0ull);
+        for (int q = 0; q < kHead; ++q) pre[q] = make_ulonglong2(0ull, 0ull);
         if (tid < P) {
             const unsigned long long* m = sp.msg + ((size_t)(tl & 3) * P + tid) * sp.msg_stride;
 #pragma unroll
-            for (int q = 0; q < 4; ++q) pre[q] = __ldcg(reinterpret_cast<const ulonglong2*>(m + 2 * q));
+            for (int q = 0; q < kHead; ++q) pre[q] = __ldcg(reinterpret_cast<const ulonglong2*>(m + 2 * q));
         }
-        EarlyRuns none;
+        EarlyRuns<INL> none;
         none.ok = false;
-        deliver_list<SAT>(
+        deliver_list<SAT, INL>(
             sp, smem, L, c, wt_base, tl, sp.n_steps & 1, ring, wrap, events, pre, none);
     }
     __syncthreads();
@@ -818,17 +831,19 @@ __device__ __forceinline__ void step_body(const StepParams& sp, const int c, uns
     if (lane == 0 && events) atomicAdd(&sp.counters[1], events);   // per-warp counts
 }
 
-template <int NPT, bool SMEM_RING, int MODE>
+template <int NPT, bool SMEM_RING, int MODE, int INL = kInline>
 __global__ void __launch_bounds__(kStepThreads, 1)
 k_step(const __grid_constant__ StepParams sp) {
     extern __shared__ __align__(16) unsigned char smem[];
-    step_body<NPT, SMEM_RING, MODE>(sp, (int)blockIdx.x, smem);
+    step_body<NPT, SMEM_RING, MODE, INL>(sp, (int)blockIdx.x, smem);
 }
 
 // the kernel of one MODE for a launch shape (neurons per thread, ring in
-// shared memory or not); nullptr for an unknown shape
+// shared memory or not, at most kFewParts partitions); nullptr for an unknown
+// shape
 template <int MODE>
-const void* step_fn_mode(int npt, bool smem_ring) {
+const void* step_fn_mode(int npt, bool smem_ring, bool few) {
+    if (few && npt == 1 && smem_ring) return reinterpret_cast<const void*>(&k_step<1, true, MODE, kInlineFew>);
     switch (npt) {
         case 1: return smem_ring ? reinterpret_cast<const void*>(&k_step<1, true, MODE>)
                                  : reinterpret_cast<const void*>(&k_step<1, false, MODE>);
@@ -841,9 +856,9 @@ const void* step_fn_mode(int npt, bool smem_ring) {
         default: return nullptr;
     }
 }
-extern template const void* step_fn_mode<0>(int, bool);
-extern template const void* step_fn_mode<kModePaced>(int, bool);
-extern template const void* step_fn_mode<kModeSat>(int, bool);
-extern template const void* step_fn_mode<kModeSat | kModePaced>(int, bool);
+extern template const void* step_fn_mode<0>(int, bool, bool);
+extern template const void* step_fn_mode<kModePaced>(int, bool, bool);
+extern template const void* step_fn_mode<kModeSat>(int, bool, bool);
+extern template const void* step_fn_mode<kModeSat | kModePaced>(int, bool, bool);
 
 }  // namespace snn

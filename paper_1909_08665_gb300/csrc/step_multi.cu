@@ -12,7 +12,7 @@
 namespace snn {
 namespace {
 
-template <int NPT, bool SMEM_RING>
+template <int NPT, bool SMEM_RING, int INL>
 __global__ void __launch_bounds__(kStepThreads, 1)
 k_step_multi(const StepParams* __restrict__ params, const int32_t* __restrict__ first, int n_net,
              const long long* step, int n_steps) {
@@ -34,36 +34,37 @@ k_step_multi(const StepParams* __restrict__ params, const int32_t* __restrict__ 
         s_sp.n_steps = n_steps;
     }
     __syncthreads();
-    step_body<NPT, SMEM_RING, 0>(s_sp, (int)blockIdx.x - __ldg(&first[a]), smem);
+    step_body<NPT, SMEM_RING, 0, INL>(s_sp, (int)blockIdx.x - __ldg(&first[a]), smem);
 }
 
 // after the launch, when every CTA has read it
 __global__ void k_advance(long long* step, int n_steps) { *step += n_steps; }
 
-const void* multi_fn(int npt, bool smem_ring) {
+const void* multi_fn(int npt, bool smem_ring, bool few) {
+    if (few && npt == 1 && smem_ring) return reinterpret_cast<const void*>(&k_step_multi<1, true, kInlineFew>);
     switch (npt) {
-        case 1: return smem_ring ? reinterpret_cast<const void*>(&k_step_multi<1, true>) : nullptr;
-        case 2: return smem_ring ? reinterpret_cast<const void*>(&k_step_multi<2, true>)
-                                 : reinterpret_cast<const void*>(&k_step_multi<2, false>);
-        case 4: return smem_ring ? nullptr : reinterpret_cast<const void*>(&k_step_multi<4, false>);
-        case 8: return smem_ring ? nullptr : reinterpret_cast<const void*>(&k_step_multi<8, false>);
+        case 1: return smem_ring ? reinterpret_cast<const void*>(&k_step_multi<1, true, kInline>) : nullptr;
+        case 2: return smem_ring ? reinterpret_cast<const void*>(&k_step_multi<2, true, kInline>)
+                                 : reinterpret_cast<const void*>(&k_step_multi<2, false, kInline>);
+        case 4: return smem_ring ? nullptr : reinterpret_cast<const void*>(&k_step_multi<4, false, kInline>);
+        case 8: return smem_ring ? nullptr : reinterpret_cast<const void*>(&k_step_multi<8, false, kInline>);
         default: return nullptr;
     }
 }
 
 }  // namespace
 
-cudaError_t step_multi_configure(int npt, bool smem_ring, size_t smem, int* blocks_per_sm) {
-    const void* fn = multi_fn(npt, smem_ring);
+cudaError_t step_multi_configure(int npt, bool smem_ring, bool few, size_t smem, int* blocks_per_sm) {
+    const void* fn = multi_fn(npt, smem_ring, few);
     if (!fn) return cudaErrorInvalidValue;
     const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, fn, kStepThreads, smem);
 }
 
-cudaError_t launch_step_multi(int npt, bool smem_ring, size_t smem, int grid, const StepParams* params,
+cudaError_t launch_step_multi(int npt, bool smem_ring, bool few, size_t smem, int grid, const StepParams* params,
                               const int32_t* first, int n_net, long long* step, int n_steps, cudaStream_t s) {
-    const void* fn = multi_fn(npt, smem_ring);
+    const void* fn = multi_fn(npt, smem_ring, few);
     if (!fn) return cudaErrorInvalidValue;
     // the attribute is the kernel's: another batch may have set it lower
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
