@@ -640,7 +640,7 @@ int adjoint_part_plan(int n, int n_pop, const int32_t* pop_start, int n_part, co
     if (e == cudaSuccess)
         e = cudaMemcpy(plan->d_img_off, off.data(), sizeof(uint32_t) * off.size(), cudaMemcpyHostToDevice);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_adjoint_part, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        e = allow_shared(reinterpret_cast<const void*>(&k_adjoint_part));
     int per_sm = 0;
     if (e == cudaSuccess)
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_adjoint_part, kApLaunch, smem);
@@ -659,10 +659,6 @@ void adjoint_part_free(AdjPartPlan* plan) {
 }
 
 cudaError_t launch_adjoint_part(const AdjPartPlan& plan, AdjPartParams& ap, cudaStream_t s) {
-    // the attribute is the kernel's, not the plan's: another network's plan may
-    // have set it lower
-    cudaError_t e = cudaFuncSetAttribute(k_adjoint_part, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)plan.smem);
-    if (e != cudaSuccess) return e;
     ap.groups = plan.groups;
     ap.ring_r = plan.ring_r;
     ap.span_max = plan.span_max;

@@ -1228,9 +1228,7 @@ int snn_batch_create(const snn_config* cfgs, const uint64_t* seeds, int32_t n_in
     for (int npt : kNptVariants) {
         if ((long long)npt * kBThreads * b->blocks < ntot) continue;
         const size_t smem = batch_smem(npt, n_inst);
-        if (cudaFuncSetAttribute(select_batch(npt), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)smem) != cudaSuccess)
-            break;
+        if (allow_shared(select_batch(npt)) != cudaSuccess) break;
         int ps = 0;
         if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ps, select_batch(npt), kBThreads, smem) !=
                 cudaSuccess ||
@@ -1334,8 +1332,7 @@ int snn_batch_create(const snn_config* cfgs, const uint64_t* seeds, int32_t n_in
     p.barrier = b->d_sync;
     p.status = b->d_sync + 1;
     p.abort_flag = b->d_sync + 2;
-    if (cudaFuncSetAttribute(k_probe_deliver, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)flat_smem_bytes(n_inst)) != cudaSuccess) {
+    if (allow_shared(reinterpret_cast<const void*>(&k_probe_deliver)) != cudaSuccess) {
         free_batch(b);
         return set_error(SNN_ERR_CUDA, "probe kernel shared memory");
     }

@@ -289,7 +289,7 @@ int plan(snn_net* net, const snn_options* opt) {
     const size_t with_ring = step_shared_bytes(ncmax, P, net->w_span, true);
     net->smem_ring = with_ring <= (size_t)smem_max;
     net->smem = step_shared_bytes(ncmax, P, net->w_span, net->smem_ring);
-    CK(step_kernel_configure(npt, net->smem_ring, P <= kFewPartsLimit, net->smem));
+    CK(step_kernel_configure(npt, net->smem_ring, P <= kFewPartsLimit));
     int per_sm = 0;
     CK(step_max_blocks(npt, net->smem_ring, P <= kFewPartsLimit, net->smem, &per_sm));
     if (per_sm * sms < P)

@@ -237,6 +237,19 @@ __device__ __forceinline__ int pop_index(const int32_t* pop_start, int n_pop, in
     return p;
 }
 
+// A kernel's dynamic shared memory limit raised to all a CTA may have.  The
+// limit belongs to the kernel, for the whole process: set to what one network
+// needs, it would fail the launches of a larger one made before.
+inline cudaError_t allow_shared(const void* fn) {
+    int dev = 0, optin = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    cudaFuncAttributes a;
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, fn);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)a.sharedSizeBytes);
+}
+
 // host-side launchers (defined in the .cu files)
 cudaError_t launch_build_count(const BuildParams& bp, uint32_t* rowlen, cudaStream_t s);
 cudaError_t launch_build_scan(const uint32_t* rowlen, int n, unsigned long long* row_start,
@@ -321,7 +334,7 @@ size_t step_shared_bytes(int ncmax, int n_part, int w_span, bool smem_ring);
 // part_lo[c+1]) (the rows of the weight table a CTA of the step kernel keeps)
 int partition_pop_span(const int32_t* part_lo, int n_part, const int32_t* pop_start, int n_pop);
 // few: at most kFewParts partitions
-cudaError_t step_kernel_configure(int npt, bool smem_ring, bool few, size_t smem);
+cudaError_t step_kernel_configure(int npt, bool smem_ring, bool few);
 cudaError_t launch_step(const StepParams& sp, int npt, bool smem_ring, size_t smem,
                         cudaStream_t s);
 cudaError_t launch_deliver(const DeliverParams& dp, int tiling, cudaStream_t s);

@@ -79,12 +79,11 @@ int step_kernel_variant(int npt, bool smem_ring, bool few) {
     return select_step(npt, smem_ring, few, 0) != nullptr;
 }
 
-cudaError_t step_kernel_configure(int npt, bool smem_ring, bool few, size_t smem) {
+cudaError_t step_kernel_configure(int npt, bool smem_ring, bool few) {
     for (int mode = 0; mode < 4; ++mode) {
         const void* fn = select_step(npt, smem_ring, few, mode);
         if (!fn) return cudaErrorInvalidValue;
-        const cudaError_t e =
-            cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        const cudaError_t e = allow_shared(fn);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;

@@ -57,7 +57,7 @@ const void* multi_fn(int npt, bool smem_ring, bool few) {
 cudaError_t step_multi_configure(int npt, bool smem_ring, bool few, size_t smem, int* blocks_per_sm) {
     const void* fn = multi_fn(npt, smem_ring, few);
     if (!fn) return cudaErrorInvalidValue;
-    const cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = allow_shared(fn);
     if (e != cudaSuccess) return e;
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, fn, kStepThreads, smem);
 }
@@ -66,11 +66,8 @@ cudaError_t launch_step_multi(int npt, bool smem_ring, bool few, size_t smem, in
                               const int32_t* first, int n_net, long long* step, int n_steps, cudaStream_t s) {
     const void* fn = multi_fn(npt, smem_ring, few);
     if (!fn) return cudaErrorInvalidValue;
-    // the attribute is the kernel's: another batch may have set it lower
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
     void* args[] = {&params, &first, &n_net, &step, &n_steps};
-    e = cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(kStepThreads), args, smem, s);
+    const cudaError_t e = cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(kStepThreads), args, smem, s);
     if (e != cudaSuccess) return e;
     k_advance<<<1, 1, 0, s>>>(step, n_steps);
     return cudaGetLastError();
