@@ -1065,6 +1065,7 @@ int drain_raster(snn_batch* b) {
     const int lists = b->part ? b->part_grid : 1;
     const RasterList in = {counts, b->d_ras_step, b->d_ras_id, b->part ? b->part_cap : b->ras_cap, lists,
                            b->n_inst, b->d_goff, (uint32_t)b->ras_lo, b->step - b->ras_lo, (uint32_t)b->ntot};
+    std::lock_guard<std::mutex> hold(b->stage.mu);
     RasterSmall small;
     BCK(raster_read_small(in, counts, &b->stage, b->stream, &small));
     const uint32_t m = small.n;

@@ -756,6 +756,7 @@ int net_update_saturation(snn_net* net) {
 
 int net_ring_to_host(snn_net* net, int32_t* host) {
     const size_t words = (size_t)kRing * net->n;
+    std::lock_guard<std::mutex> hold(net->stage.mu);
     if (!net->d_ring_io) CALL(dalloc(&net->d_ring_io, words, "ring staging"));
     CK(launch_ring_layout(net->d_part_lo, net->P, net->ncmax, net->n, net->d_ring, net->d_ring_io, true,
                           net->stream));
@@ -766,6 +767,7 @@ int net_ring_to_host(snn_net* net, int32_t* host) {
 
 int net_ring_from_host(snn_net* net, const int32_t* host) {
     const size_t words = (size_t)kRing * net->n;
+    std::lock_guard<std::mutex> hold(net->stage.mu);
     if (!net->d_ring_io) CALL(dalloc(&net->d_ring_io, words, "ring staging"));
     CK(cudaMemcpyAsync(net->d_ring_io, host, sizeof(int32_t) * words, cudaMemcpyHostToDevice, net->stream));
     CK(launch_ring_layout(net->d_part_lo, net->P, net->ncmax, net->n, net->d_ring, net->d_ring_io, false,
@@ -907,6 +909,7 @@ int snn_read_spikes(snn_net* net, uint32_t* steps_host, uint32_t* ids_host, int6
                            (uint32_t)net->ras_lo, net->ras_hi - net->ras_lo, (uint32_t)net->n};
     int64_t total = 0;
     bool lost = false;
+    std::lock_guard<std::mutex> hold(net->stage.mu);
     if (net->P < kStepThreads) {
         RasterSmall r;
         CK(raster_read_small(in, net->d_ras_n, &net->stage, net->stream, &r));

@@ -316,11 +316,13 @@ cudaError_t host_stage(HostStage* st, size_t bytes, uint32_t** host, uint32_t** 
 
 void host_stage_free(HostStage* st) {
     if (st->host) cudaFreeHost(st->host);
-    *st = HostStage();
+    st->host = st->dev = nullptr;
+    st->bytes = 0;
 }
 
 cudaError_t read_arrays(int count, const uint32_t* const* dev_src, uint32_t* const* host_dst, int n,
                         HostStage* stage, cudaStream_t s) {
+    std::lock_guard<std::mutex> hold(stage->mu);
     uint32_t *host = nullptr, *dev = nullptr;
     const int total = count * n;
     cudaError_t e = host_stage(stage, sizeof(uint32_t) * (size_t)total, &host, &dev);

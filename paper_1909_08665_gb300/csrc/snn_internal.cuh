@@ -2,6 +2,7 @@
 // GB300 microcircuit library (not part of the public ABI).
 #pragma once
 #include <cstdint>
+#include <mutex>
 #include <cuda_runtime.h>
 
 namespace snn {
@@ -296,7 +297,11 @@ struct RasterSort {
 };
 cudaError_t raster_sort(RasterSort* w, const RasterList& in, size_t n, cudaStream_t s);
 // Pinned host memory that kernels write small results into (grows, is kept).
+// mu is held from the launch until the result is copied out: one handle may be
+// read from several threads.  read_arrays takes it, callers of
+// raster_read_small hold it.
 struct HostStage {
+    std::mutex mu;
     void* host = nullptr;
     void* dev = nullptr;
     size_t bytes = 0;

@@ -94,3 +94,32 @@ def test_batch_reads_are_sorted():
         st, ids = net.read_spikes()
         np.testing.assert_array_equal(np.concatenate([g[0] for g in got[k]]), st)
         np.testing.assert_array_equal(np.concatenate([g[1] for g in got[k]]), ids)
+
+
+def test_reads_from_several_threads():
+    """One handle read from several threads at once: every read is whole."""
+    import threading
+
+    net = _net(0.05)
+    net.step(300)
+    net.sync()
+    want, counts, ring = net.state(), net.counters(), net.ring()
+    wrong = []
+
+    def read(kind):
+        for _ in range(60):
+            if kind == 0:
+                ok = all(np.array_equal(a.view(np.uint32), b.view(np.uint32)) for a, b in zip(net.state(), want))
+            elif kind == 1:
+                ok = net.counters() == counts and net.raster_size() == counts["spikes"]
+            else:
+                ok = np.array_equal(net.ring(), ring)
+            if not ok:
+                wrong.append(kind)
+
+    threads = [threading.Thread(target=read, args=(k % 3,)) for k in range(6)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not wrong
