@@ -25,8 +25,9 @@
 //         go on; the last warp waits at it and publishes the count.  (With a
 //         CTA barrier there, the count waited for the warps that had to have
 //         the other partitions' message heads first: us per step at scale
-//         0.02 1.72, 0.1 1.78, 4 14.6; now 1.64, 1.73 and 12.7; at scale 1
-//         2.57 either way.)
+//         0.02 1.72, 0.1 1.78, 4 14.6; so 1.64, 1.73 and 12.7.  With one
+//         neuron per thread and more than kFewParts partitions the CTA
+//         barrier is the faster one, see PUB_EARLY.)
 //   D     wait for every partition's message of step t-1 (each word carries
 //         its own tag, so a matching tag is both the grid-wide barrier and
 //         the data; no fence, no counter), look up each spike's run for this
@@ -59,7 +60,8 @@ constexpr uint32_t kStatusRasterOverflow = 2u;
 // Ids read together with a message header: INL = 7 (64 bytes), or 3 (32 bytes)
 // where there are few partitions (kFewParts) and hardly ever more spikes in
 // one.  us per step with 7 / 3: scale 0.02 1.54 / 1.49, 0.1 1.63 / 1.59, 0.37
-// (57 partitions) 1.97 / 1.91, 0.6 (91) 2.21 / 2.36, 1 (151) 2.60 / 2.87.
+// (57 partitions) 1.97 / 1.91, 0.6 (91) 2.21 / 2.36, 1 (151) 2.60 / 2.87 (with 7
+// now 2.14 and 2.56, see PUB_EARLY).
 constexpr int kInline = 7;
 constexpr int kInlineFew = 3;
 constexpr int kFewParts = kFewPartsLimit;
@@ -347,8 +349,8 @@ __device__ __forceinline__ bool deliver_list(const StepParams& sp, unsigned char
     const uint32_t tag = (uint32_t)(tb + 1);
     uint32_t* s_warp = reinterpret_cast<uint32_t*>(smem + L.warp);
     volatile uint32_t* s_misc = reinterpret_cast<uint32_t*>(smem + L.misc);
-    // listed spikes, in the counter of this list's parity; the other one is
-    // cleared after the barrier below, when its last readers are done
+    // listed spikes, in the counter of this list's parity; the publisher of
+    // the step clears the other one, whose last readers are done
     volatile uint32_t* s_list = s_misc + 6 + par;
     unsigned long long* s_inl = reinterpret_cast<unsigned long long*>(smem + L.inl);
     uint32_t* s_rb = reinterpret_cast<uint32_t*>(smem + L.rb);
@@ -460,7 +462,6 @@ __device__ __forceinline__ bool deliver_list(const StepParams& sp, unsigned char
     }
     __syncthreads();
     const uint32_t S_fast = *s_list;
-    if (tid == 0) s_misc[6 + (par ^ 1)] = 0u;
     if (s_misc[2]) return false;
     if (S_fast <= (uint32_t)kChunk) {
         deliver_batches<SAT>(sp, s_rb, s_rl, s_w, wbase, S_fast, tb, ring, wrap, events,
@@ -542,8 +543,9 @@ __device__ __forceinline__ void barrier_wait(int id, int n) {
     asm volatile("barrier.cta.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
 }
 
-// One CTA's steps: partition c of the network sp describes.
-template <int NPT, bool SMEM_RING, int MODE, int INL>
+// One CTA's steps: partition c of the network sp describes (MULTI: one of
+// several networks of the launch, whose recorded ids are offset).
+template <int NPT, bool SMEM_RING, int MODE, int INL, bool MULTI>
 __device__ __forceinline__ void step_body(const StepParams& sp, const int c, unsigned char* smem) {
     constexpr int kHead = (INL + 1) / 2;
     constexpr bool PACED = (MODE & kModePaced) != 0;
@@ -552,6 +554,11 @@ __device__ __forceinline__ void step_body(const StepParams& sp, const int c, uns
     // not in the widest variant (us per step without / with: 1.3x 3.44 / 3.12,
     // 2x 4.78 / 4.46, 4x 8.23 / 8.15)
     constexpr bool EARLY = NPT <= 4;
+    // the count published ahead of the CTA barrier, or at it: with one neuron
+    // per thread and many partitions the header warps are the slow ones either
+    // way, and they gain from the others' wait (us per step ahead / at it:
+    // scale 0.6 2.16 / 2.14, 1 2.59 / 2.56)
+    constexpr bool PUB_EARLY = NPT > 1 || INL == kInlineFew;
     const int tid = threadIdx.x;
     const int lane = tid & 31;
     const int P = sp.n_part;
@@ -681,30 +688,47 @@ __device__ __forceinline__ void step_body(const StepParams& sp, const int c, uns
                     const uint32_t rp = ras_base + pos;
                     if (rp < sp.ras_cap) {
                         sp.ras_step[(size_t)c * sp.ras_cap + rp] = (uint32_t)t;
-                        sp.ras_id[(size_t)c * sp.ras_cap + rp] = sp.ras_id0 + id;
+                        sp.ras_id[(size_t)c * sp.ras_cap + rp] = MULTI ? sp.ras_id0 + id : id;
                     }
                 }
             }
         }
+        auto publish = [&]() {
+            const uint32_t nsp = *my_cnt;
+            // counter of step s+1 (last read in step s-1, before this barrier)
+            // and of the next delivery's list (last read in the delivery of
+            // step s-1, likewise)
+            s_misc[(s + 1) & 1] = 0u;
+            s_misc[6 + ((s + 1) & 1)] = 0u;
+            if (!(sp.inject_fault == 1 && c == 0)) __stcg(&my_msg[0], tag | nsp);
+            spikes += nsp;
+            if (ras_base + nsp > sp.ras_cap) atomicOr(sp.status, kStatusRasterOverflow);
+            if (sp.st_counts != nullptr && nsp > 0u) {
+                const int64_t r = t - sp.sc_t0;
+                if (r >= 0 && r < sp.sc_cap) atomicAdd(&sp.st_counts[4 * r], nsp);
+            }
+        };
         // every warp has counted its spikes: the last one waits for that and
         // publishes the count; the others only arrive and go on
-        if (tid < kPublisher) {
-            barrier_arrive(1, kStepThreads);
-        } else {
-            barrier_wait(1, kStepThreads);
-            if (tid == kPublisher) {
-                const uint32_t nsp = *my_cnt;
-                // counter of step s+1 (last read in step s-1, before this barrier)
-                s_misc[(s + 1) & 1] = 0u;
-                if (!(sp.inject_fault == 1 && c == 0)) __stcg(&my_msg[0], tag | nsp);
-                spikes += nsp;
-                if (ras_base + nsp > sp.ras_cap) atomicOr(sp.status, kStatusRasterOverflow);
-                if (sp.st_counts != nullptr && nsp > 0u) {
-                    const int64_t r = t - sp.sc_t0;
-                    if (r >= 0 && r < sp.sc_cap) atomicAdd(&sp.st_counts[4 * r], nsp);
-                }
+        if (PUB_EARLY) {
+            if (tid < kPublisher) {
+                barrier_arrive(1, kStepThreads);
+            } else {
+                barrier_wait(1, kStepThreads);
+                if (tid == kPublisher) publish();
             }
         }
+        // the run bounds of the step t-1 spikes whose message words this
+        // header thread already holds (the head loaded before A(t), arrived
+        // by now): with several neurons per thread looked up here, so that
+        // they return during the background draws (4x 7.99 us per step with
+        // the lookups after them, 7.72 before); with one the draw is short and
+        // the heads may still be on their way (scale 0.1 1.57 before it, 1.56
+        // after)
+        EarlyRuns<INL> early;
+        early.ok = false;
+        const bool look_up = EARLY && s > 0 && tid < P;
+        if (NPT > 1 && look_up) early_runs(sp, c, pre, (uint32_t)t, early);
 #pragma unroll
         for (int k = 0; k < NPT; ++k) {
             const int li = tid + k * kStepThreads;
@@ -727,13 +751,13 @@ __device__ __forceinline__ void step_body(const StepParams& sp, const int c, uns
                 pacc[k] = kk * sp.wext_q;
             }
         }
-        // the run bounds of the step t-1 spikes whose message words this
-        // header thread already holds (the head loaded before A(t), arrived
-        // by now): looked up here, so that they return while the CTA meets
-        // at the barrier and the header is published
-        EarlyRuns<INL> early;
-        early.ok = false;
-        if (EARLY && s > 0 && tid < P) early_runs(sp, c, pre, (uint32_t)t, early);
+        if (NPT == 1 && look_up) early_runs(sp, c, pre, (uint32_t)t, early);
+        if (!PUB_EARLY) {                        // the lookups return meanwhile
+            __syncthreads();
+            const uint32_t nsp = *my_cnt;
+            if (tid == kPublisher) publish();
+            ras_base += nsp;
+        }
         // ---- D: spikes of step t-1 ----
         if (s > 0) {
             if (!deliver_list<SAT, INL>(
@@ -744,7 +768,7 @@ __device__ __forceinline__ void step_body(const StepParams& sp, const int c, uns
         } else {
             __syncthreads();                     // the counts of step 0, as after a delivery
         }
-        ras_base += *my_cnt;
+        if (PUB_EARLY) ras_base += *my_cnt;
         // ---- C(t): ring slot t, Poisson background, synaptic current ----
         const uint32_t slot = (uint32_t)t & (kRing - 1);
         // all of the thread's cells are in flight before the first is cleared
@@ -754,14 +778,14 @@ __device__ __forceinline__ void step_body(const StepParams& sp, const int c, uns
 #pragma unroll
         for (int k = 0; k < NPT; ++k) {
             const int li = tid + k * kStepThreads;
-            cells[k] = li < nc ? ring[slot * (uint32_t)sp.ncmax + (uint32_t)li] : 0;
+            if (NPT > 1) cells[k] = li < nc ? ring[slot * (uint32_t)sp.ncmax + (uint32_t)li] : 0;
         }
 #pragma unroll
         for (int k = 0; k < NPT; ++k) {
             const int li = tid + k * kStepThreads;
             if (li < nc) {
                 const uint32_t cell = slot * (uint32_t)sp.ncmax + (uint32_t)li;
-                const int32_t r = cells[k];
+                const int32_t r = NPT > 1 ? cells[k] : ring[cell];
                 ring[cell] = 0;
                 // the input wraps modulo 2^32, as the int32 accumulation of
                 // the method does; SAT: its true value r + 2^32 wraps + pacc
@@ -835,7 +859,7 @@ template <int NPT, bool SMEM_RING, int MODE, int INL = kInline>
 __global__ void __launch_bounds__(kStepThreads, 1)
 k_step(const __grid_constant__ StepParams sp) {
     extern __shared__ __align__(16) unsigned char smem[];
-    step_body<NPT, SMEM_RING, MODE, INL>(sp, (int)blockIdx.x, smem);
+    step_body<NPT, SMEM_RING, MODE, INL, false>(sp, (int)blockIdx.x, smem);
 }
 
 // the kernel of one MODE for a launch shape (neurons per thread, ring in
