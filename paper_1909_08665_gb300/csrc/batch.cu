@@ -653,17 +653,21 @@ struct snn_batch {
     HostStage stage;                     // small reads
     long long ras_lo = 0;                // first step since the last drain
     bool ras_new = false;                // steps were issued since the last drain
+    unsigned long long ras_kept = 0;     // spikes drained since the last read, to make room
     std::vector<float2> u0_range;        // default initial potentials per instance
     float trial_us = 0.f;                // per-step time of the chosen assignment
     // the partitioned form (step_multi.cu): every instance a network of its own
     // partitions, all of them co-resident; d_u, d_i, d_r, the raster and the
     // counters are the batch's
     std::vector<snn_net*> nets;          // empty: does not fit
+    bool part_fits = false;              // its kernel's CTAs are co-resident
     bool part = false;                   // steps run in this form
     int part_npt = 0, part_grid = 0;
     bool part_smem_ring = false, part_few = true;   // few: no instance above kFewPartsLimit partitions
     size_t part_smem = 0, part_ring_words = 0, part_msg_words = 0;
     uint32_t part_cap = 0;               // raster capacity of a partition
+    int part_ncmax = 1;                  // most neurons of one
+    long long part_left = 0;             // steps until the fullest list is looked at (make_room)
     std::vector<size_t> part_ring_off;   // of each instance, words
     StepParams* d_part = nullptr;        // [n_inst]
     int32_t* d_part_first = nullptr;     // [n_inst + 1] first CTA of each instance
@@ -853,7 +857,7 @@ int batch_trials(snn_batch* b) {
     // The partitioned form, where the instances fit, is one more candidate;
     // with one neuron per thread the only one (it takes 1.7 to 2.6 us per step
     // there, a step of the other form never below 5).
-    const size_t n_cand = b->nets.empty() ? cand.size() : b->part_npt == 1 ? 1 : cand.size() + 1;
+    const size_t n_cand = !b->part_fits ? cand.size() : b->part_npt == 1 ? 1 : cand.size() + 1;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     BCK(cudaEventCreate(&e0));
     BCK(cudaEventCreate(&e1));
@@ -862,8 +866,8 @@ int batch_trials(snn_batch* b) {
     bool best_part = false;
     cudaError_t e = cudaSuccess;
     for (size_t x = 0; x < n_cand && e == cudaSuccess; ++x) {
-        b->part = !b->nets.empty() && x == 0;
-        const size_t c = b->nets.empty() || x == 0 ? x : x - 1;
+        b->part = b->part_fits && x == 0;
+        const size_t c = !b->part_fits || x == 0 ? x : x - 1;
         for (int k = 0; k < K; ++k) b->hot_h[k].key.z = cand[c][k];
         e = cudaMemcpyAsync(b->d_hot, b->hot_h.data(), sizeof(InstHot) * K, cudaMemcpyHostToDevice, s);
         if (e == cudaSuccess) e = reset_state(b);
@@ -934,6 +938,7 @@ int saturation_error() {
 // no faster); false when that takes more than a partition may hold, or when
 // the configurations are not valid (reported where they are built).
 constexpr int kFewest = 160, kMostPart = 8 * kStepThreads;
+constexpr long long kLeastList = 64 * kMostPart;    // raster entries of a partition's list: 64 steps of every neuron
 bool plan_parts(const snn_config* cfgs, int n_inst, int sms, std::vector<int>* n_part) {
     std::vector<long long> n(n_inst, 0);
     for (int k = 0; k < n_inst; ++k) {
@@ -958,8 +963,8 @@ bool plan_parts(const snn_config* cfgs, int n_inst, int sms, std::vector<int>* n
     return true;
 }
 
-// state, messages and parameters of the partitioned form; the form is dropped
-// (b->nets stay: they own the rows) when its kernel does not fit
+// state, messages and parameters of the partitioned form; the form is not
+// used (b->nets stay: they own the rows) when its kernel does not fit
 int setup_parts(snn_batch* b) {
     const int K = b->n_inst;
     int dev = 0, optin = 0, sms = 0, ncmax = 0;
@@ -1021,17 +1026,18 @@ int setup_parts(snn_batch* b) {
     BCK(cudaMemcpy(b->d_part_first, first.data(), sizeof(int32_t) * (K + 1), cudaMemcpyHostToDevice));
     int per_sm = 0;
     BCK(step_multi_configure(b->part_npt, b->part_smem_ring, b->part_few, b->part_smem, &per_sm));
-    if (per_sm * sms < b->part_grid) return set_error(SNN_ERR_UNSUPPORTED, "batch partitions exceed co-resident CTAs");
-    b->part = true;
+    b->part = b->part_fits = per_sm * sms >= b->part_grid;
+    b->part_ncmax = ncmax;
+    b->part_left = b->part_cap / ncmax;
     BCK(reset_state(b));
     return SNN_OK;
 }
 
-int drain_raster(snn_batch* b);
+int drain_raster(snn_batch* b, bool keep);
 
 // on to the tiled form, which steps a batch once a tiling was asked for
 int leave_parts(snn_batch* b) {
-    BCALL(drain_raster(b));
+    BCALL(drain_raster(b, true));
     cudaStream_t s = b->stream;
     int32_t* tmp = nullptr;
     int n_most = 1;
@@ -1054,12 +1060,21 @@ int leave_parts(snn_batch* b) {
     return capture_graph(b);
 }
 
+// a read ends the count of what was drained since the last one
+int kept_raster(snn_batch* b, bool keep) {
+    if (keep) return SNN_OK;
+    const bool over = b->ras_kept > b->ras_cap;
+    b->ras_kept = 0;
+    return over ? set_error(SNN_ERR_OVERFLOW, "batch raster capacity exceeded") : SNN_OK;
+}
+
 // the spikes recorded since the last drain, sorted by (instance, step, id) on
-// the device, appended to each instance's host arrays
-int drain_raster(snn_batch* b) {
+// the device, appended to each instance's host arrays; keep: not for a read,
+// what was drained still counts against the capacity
+int drain_raster(snn_batch* b, bool keep) {
     if (!b->ras_new) {                          // no step issued since: nothing recorded
         BCK(cudaStreamSynchronize(b->stream));
-        return SNN_OK;
+        return kept_raster(b, keep);
     }
     uint32_t* counts = b->part ? b->d_part_n : b->d_ras_n;
     const int lists = b->part ? b->part_grid : 1;
@@ -1093,7 +1108,29 @@ int drain_raster(snn_batch* b) {
         for (size_t i = at; i < out.size(); ++i) out[i] -= lo;
         r = e;
     }
-    if (small.lost) return set_error(SNN_ERR_OVERFLOW, "batch raster capacity exceeded");
+    b->part_left = b->part_cap / b->part_ncmax;
+    b->ras_kept += small.lost ? (unsigned long long)b->ras_cap + 1ull : m;
+    return kept_raster(b, keep);
+}
+
+int part_counts(snn_batch* b, std::vector<uint32_t>* n) {
+    n->resize(b->part_grid);
+    BCK(cudaStreamSynchronize(b->stream));
+    BCK(cudaMemcpy(n->data(), b->d_part_n, sizeof(uint32_t) * b->part_grid, cudaMemcpyDeviceToHost));
+    return SNN_OK;
+}
+
+// Steps that may be issued before a partition's raster list could be full: a
+// neuron spikes at most once a step.  A list that holds the whole capacity
+// needs no look.  Otherwise, when they are used up, the counts are read and
+// lists more than half full drained.
+int make_room(snn_batch* b) {
+    if (!b->part || b->part_cap >= b->ras_cap || b->part_left > 0) return SNN_OK;
+    std::vector<uint32_t> n;
+    BCALL(part_counts(b, &n));
+    const uint32_t most = *std::max_element(n.begin(), n.end());
+    if (most > b->part_cap / 2) return drain_raster(b, true);
+    b->part_left = (b->part_cap - most) / b->part_ncmax;
     return SNN_OK;
 }
 
@@ -1249,9 +1286,11 @@ int snn_batch_create(const snn_config* cfgs, const uint64_t* seeds, int32_t n_in
     long long ras_words = b->ras_cap;
     if (parts) {
         // a list per partition; four times its share of the capacity each, as
-        // the populations' rates differ
+        // the populations' rates differ, and no less than kLeastList (one that
+        // could fill up all the same is drained in time, make_room)
         for (int P : n_part) b->part_grid += P;
-        b->part_cap = (uint32_t)std::min<long long>(std::max<long long>(4 * (long long)b->ras_cap / b->part_grid, 1), b->ras_cap);
+        b->part_cap = (uint32_t)std::min<long long>(
+            std::max<long long>(4 * (long long)b->ras_cap / b->part_grid, kLeastList), b->ras_cap);
         ras_words = std::max<long long>(ras_words, (long long)b->part_cap * b->part_grid);
     }
     if (rc == SNN_OK) rc = balloc(&b->d_hot, n_inst, "batch instance constants");
@@ -1352,18 +1391,17 @@ int snn_batch_create(const snn_config* cfgs, const uint64_t* seeds, int32_t n_in
 int snn_batch_step(snn_batch* b, int64_t n_steps) {
     if (!b || n_steps < 0) return set_error(SNN_ERR_INVALID, "bad arguments");
     int64_t left = n_steps;
-    if (left > 0) b->ras_new = true;
     while (left > 0) {
-        if (b->graph_ok && left >= kGraphChunk) {
-            BCK(cudaGraphLaunch(b->graph, b->stream));
-            left -= kGraphChunk;
-            b->step += kGraphChunk;
-        } else {
-            const int chunk = (int)std::min<int64_t>(left, 1 << 20);
-            BCK(launch_batch(b, chunk));
-            left -= chunk;
-            b->step += chunk;
-        }
+        BCALL(make_room(b));
+        b->ras_new = true;
+        const int64_t room = b->part && b->part_cap < b->ras_cap ? std::min<int64_t>(left, b->part_left) : left;
+        const bool graph = b->graph_ok && room >= kGraphChunk;
+        const int chunk = graph ? kGraphChunk : (int)std::min<int64_t>(room, 1 << 20);
+        if (graph) BCK(cudaGraphLaunch(b->graph, b->stream));
+        else BCK(launch_batch(b, chunk));
+        left -= chunk;
+        b->part_left -= chunk;
+        b->step += chunk;
     }
     return SNN_OK;
 }
@@ -1375,6 +1413,15 @@ int snn_batch_sync(snn_batch* b) {
     BCK(cudaMemcpy(&st, b->d_sync + 1, sizeof(st), cudaMemcpyDeviceToHost));
     if (st & kStatusTimeout) return set_error(SNN_ERR_TIMEOUT, "a grid-barrier wait timed out");
     if (st & kBatchRasterOverflow) return set_error(SNN_ERR_OVERFLOW, "batch raster capacity exceeded");
+    // side by side the lists together hold more than the capacity
+    if (b->part && b->ras_new &&
+        b->ras_kept + (unsigned long long)(b->step - b->ras_lo) * (unsigned long long)b->ntot > b->ras_cap) {
+        std::vector<uint32_t> n;
+        BCALL(part_counts(b, &n));
+        unsigned long long total = b->ras_kept;
+        for (uint32_t x : n) total += x;
+        if (total > b->ras_cap) return set_error(SNN_ERR_OVERFLOW, "batch raster capacity exceeded");
+    }
     return SNN_OK;
 }
 
@@ -1382,7 +1429,7 @@ int snn_batch_read_spikes(snn_batch* b, int32_t k, uint32_t* steps_host, uint32_
                           int64_t cap, int64_t* n) {
     if (!b || k < 0 || k >= b->n_inst || !n || cap < 0)
         return set_error(SNN_ERR_INVALID, "bad arguments");
-    const int rc = drain_raster(b);
+    const int rc = drain_raster(b, false);
     auto& st = b->host_steps[k];
     auto& id = b->host_ids[k];
     const int64_t m = std::min<int64_t>(cap, (int64_t)st.size());

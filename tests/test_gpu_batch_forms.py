@@ -2,6 +2,8 @@
 their own (no barrier over the batch); asking for a tiling takes it on to the
 batch kernel.  Every instance against a single network of its own, bit for
 bit, in both forms and across the change."""
+import copy
+
 import numpy as np
 import pytest
 
@@ -68,4 +70,32 @@ def test_tiling_asked_for_in_mid_run(before):
     batch.step(1003)
     batch.sync()
     _check(batch, cfgs, before + 1005, reads)
+    batch.close()
+
+
+# 267,703 spikes (the oracle's count), all of one partition, whose list holds 262,144
+@pytest.mark.parametrize("capacity,fits", [(267_703, True), (267_702, False)])
+def test_one_partition_may_use_the_whole_capacity(capacity, fits):
+    hot = copy.deepcopy(workload.dc_variant(workload.microcircuit(0.002)))
+    hot["i_dc"] = [20000.0] * 8
+    cold = copy.deepcopy(workload.dc_variant(workload.microcircuit(0.008)))
+    cold["i_dc"] = [0.0] * 8
+    cfgs = [cold, hot, cold, cold, cold]
+    batch = pkg.MicrocircuitBatch(cfgs, stream=torch.cuda.current_stream(), raster_capacity=capacity)
+    assert batch.info(0)["neurons_per_thread"] == 1
+    net = pkg.Microcircuit(hot, stream=torch.cuda.current_stream())
+    batch.step(90_000)
+    net.step(90_000)
+    st, ids = net.read_spikes()
+    assert st.size == 267_703
+    if fits:
+        batch.sync()
+        got = batch.read_spikes(1)
+        np.testing.assert_array_equal(got[0], st)
+        np.testing.assert_array_equal(got[1], ids)
+    else:
+        for call in (batch.sync, lambda: batch.read_spikes(1)):
+            with pytest.raises(pkg.SnnError) as e:
+                call()
+            assert e.value.code == pkg.SNN_ERR_OVERFLOW
     batch.close()
