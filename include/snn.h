@@ -469,9 +469,7 @@ typedef struct snn_batch_info {
  *   cfgs[n_inst], seeds[n_inst]   host arrays, read during the call
  *   opt                           may be NULL; raster_capacity is the total
  *                                 raster capacity of the batch (default
- *                                 64 Mi spikes; side by side, a partition
- *                                 takes up to four times its share and is
- *                                 drained to the host before it is full),
+ *                                 64 Mi spikes, 8 bytes each),
  *                                 timeout_s the barrier limit,
  *                                 inject_fault = 1 makes CTA 0 withhold its
  *                                 arrivals (tests the bounded wait:

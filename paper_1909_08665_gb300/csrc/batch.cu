@@ -653,7 +653,6 @@ struct snn_batch {
     HostStage stage;                     // small reads
     long long ras_lo = 0;                // first step since the last drain
     bool ras_new = false;                // steps were issued since the last drain
-    unsigned long long ras_kept = 0;     // spikes drained since the last read, to make room
     std::vector<float2> u0_range;        // default initial potentials per instance
     float trial_us = 0.f;                // per-step time of the chosen assignment
     // the partitioned form (step_multi.cu): every instance a network of its own
@@ -665,15 +664,11 @@ struct snn_batch {
     int part_npt = 0, part_grid = 0;
     bool part_smem_ring = false, part_few = true;   // few: no instance above kFewPartsLimit partitions
     size_t part_smem = 0, part_ring_words = 0, part_msg_words = 0;
-    uint32_t part_cap = 0;               // raster capacity of a partition
-    int part_ncmax = 1;                  // most neurons of one
-    long long part_left = 0;             // steps until the fullest list is looked at (make_room)
     std::vector<size_t> part_ring_off;   // of each instance, words
     StepParams* d_part = nullptr;        // [n_inst]
     int32_t* d_part_first = nullptr;     // [n_inst + 1] first CTA of each instance
     int32_t* d_part_ring = nullptr;      // [partition][64][ncmax of its instance]
     unsigned long long* d_part_msg = nullptr;
-    uint32_t* d_part_n = nullptr;        // [part_grid] recorded spikes
 };
 
 namespace {
@@ -708,7 +703,7 @@ void free_batch(snn_batch* b) {
         for (auto* x : b->row_start) cudaFree(x);
         for (auto* x : b->words) cudaFree(x);
     }
-    void* ptrs[] = {b->d_part, b->d_part_first, b->d_part_ring, b->d_part_msg, b->d_part_n, b->d_wtab_all, b->d_ps_all, b->d_hot, b->d_cold, b->d_pois, b->d_cdc, b->d_goff, b->d_u, b->d_i,
+    void* ptrs[] = {b->d_part, b->d_part_first, b->d_part_ring, b->d_part_msg, b->d_wtab_all, b->d_ps_all, b->d_hot, b->d_cold, b->d_pois, b->d_cdc, b->d_goff, b->d_u, b->d_i,
                     b->d_r, b->d_ring, b->d_list, b->d_cnt, b->d_ras_step, b->d_ras_id,
                     b->d_ras_n, b->d_ic, b->d_step, b->d_sync};
     for (void* x : ptrs)
@@ -816,7 +811,6 @@ cudaError_t reset_state(snn_batch* b) {
         // (message tags count steps: the rewound run must not meet old ones)
         e = cudaMemsetAsync(b->d_part_ring, 0, sizeof(int32_t) * b->part_ring_words, s);
         if (e == cudaSuccess) e = cudaMemsetAsync(b->d_part_msg, 0, sizeof(unsigned long long) * b->part_msg_words, s);
-        if (e == cudaSuccess) e = cudaMemsetAsync(b->d_part_n, 0, sizeof(uint32_t) * b->part_grid, s);
     }
     for (int k = 0; k < b->n_inst && e == cudaSuccess; ++k) {
         const InstHot& H = b->hot_h[k];
@@ -938,7 +932,6 @@ int saturation_error() {
 // no faster); false when that takes more than a partition may hold, or when
 // the configurations are not valid (reported where they are built).
 constexpr int kFewest = 160, kMostPart = 8 * kStepThreads;
-constexpr long long kLeastList = 64 * kMostPart;    // raster entries of a partition's list: 64 steps of every neuron
 bool plan_parts(const snn_config* cfgs, int n_inst, int sms, std::vector<int>* n_part) {
     std::vector<long long> n(n_inst, 0);
     for (int k = 0; k < n_inst; ++k) {
@@ -998,7 +991,6 @@ int setup_parts(snn_batch* b) {
     BCALL(balloc(&b->d_part_first, K + 1, "batch partitions"));
     BCALL(balloc(&b->d_part_ring, b->part_ring_words, "batch ring buffers"));
     BCALL(balloc(&b->d_part_msg, b->part_msg_words, "batch spike messages"));
-    BCALL(balloc(&b->d_part_n, b->part_grid, "batch raster counts"));
     std::vector<StepParams> sp(K);
     for (int k = 0; k < K; ++k) {
         StepParams& x = sp[k];
@@ -1010,10 +1002,10 @@ int setup_parts(snn_batch* b) {
         x.ring = b->d_part_ring + b->part_ring_off[k];
         x.msg = b->d_part_msg + msg_off[k];
         x.msg_stride = stride[k];
-        x.ras_step = b->d_ras_step + (size_t)first[k] * b->part_cap;
-        x.ras_id = b->d_ras_id + (size_t)first[k] * b->part_cap;
-        x.ras_n = b->d_part_n + first[k];
-        x.ras_cap = b->part_cap;
+        x.ras_step = b->d_ras_step;
+        x.ras_id = b->d_ras_id;
+        x.ras_n = b->d_ras_n;
+        x.ras_cap = b->ras_cap;
         x.ras_id0 = (uint32_t)at;
         x.counters = b->d_ic + 2 * k;
         x.pop_spikes = nullptr;
@@ -1027,17 +1019,12 @@ int setup_parts(snn_batch* b) {
     int per_sm = 0;
     BCK(step_multi_configure(b->part_npt, b->part_smem_ring, b->part_few, b->part_smem, &per_sm));
     b->part = b->part_fits = per_sm * sms >= b->part_grid;
-    b->part_ncmax = ncmax;
-    b->part_left = b->part_cap / ncmax;
     BCK(reset_state(b));
     return SNN_OK;
 }
 
-int drain_raster(snn_batch* b, bool keep);
-
 // on to the tiled form, which steps a batch once a tiling was asked for
 int leave_parts(snn_batch* b) {
-    BCALL(drain_raster(b, true));
     cudaStream_t s = b->stream;
     int32_t* tmp = nullptr;
     int n_most = 1;
@@ -1060,29 +1047,18 @@ int leave_parts(snn_batch* b) {
     return capture_graph(b);
 }
 
-// a read ends the count of what was drained since the last one
-int kept_raster(snn_batch* b, bool keep) {
-    if (keep) return SNN_OK;
-    const bool over = b->ras_kept > b->ras_cap;
-    b->ras_kept = 0;
-    return over ? set_error(SNN_ERR_OVERFLOW, "batch raster capacity exceeded") : SNN_OK;
-}
-
 // the spikes recorded since the last drain, sorted by (instance, step, id) on
-// the device, appended to each instance's host arrays; keep: not for a read,
-// what was drained still counts against the capacity
-int drain_raster(snn_batch* b, bool keep) {
+// the device, appended to each instance's host arrays
+int drain_raster(snn_batch* b) {
     if (!b->ras_new) {                          // no step issued since: nothing recorded
         BCK(cudaStreamSynchronize(b->stream));
-        return kept_raster(b, keep);
+        return SNN_OK;
     }
-    uint32_t* counts = b->part ? b->d_part_n : b->d_ras_n;
-    const int lists = b->part ? b->part_grid : 1;
-    const RasterList in = {counts, b->d_ras_step, b->d_ras_id, b->part ? b->part_cap : b->ras_cap, lists,
-                           b->n_inst, b->d_goff, (uint32_t)b->ras_lo, b->step - b->ras_lo, (uint32_t)b->ntot};
+    const RasterList in = {b->d_ras_n, b->d_ras_step, b->d_ras_id, b->ras_cap, 1, b->n_inst, b->d_goff,
+                           (uint32_t)b->ras_lo, b->step - b->ras_lo, (uint32_t)b->ntot};
     std::lock_guard<std::mutex> hold(b->stage.mu);
     RasterSmall small;
-    BCK(raster_read_small(in, counts, &b->stage, b->stream, &small));
+    BCK(raster_read_small(in, b->d_ras_n, &b->stage, b->stream, &small));
     const uint32_t m = small.n;
     std::vector<uint32_t> st(m), id(m);
     if (small.done) {
@@ -1092,7 +1068,7 @@ int drain_raster(snn_batch* b, bool keep) {
         BCK(raster_sort(&b->ras_sort, in, m, b->stream));
         BCK(cudaMemcpyAsync(st.data(), b->ras_sort.step, sizeof(uint32_t) * m, cudaMemcpyDeviceToHost, b->stream));
         BCK(cudaMemcpyAsync(id.data(), b->ras_sort.id, sizeof(uint32_t) * m, cudaMemcpyDeviceToHost, b->stream));
-        BCK(cudaMemsetAsync(counts, 0, sizeof(uint32_t) * lists, b->stream));
+        BCK(cudaMemsetAsync(b->d_ras_n, 0, sizeof(uint32_t), b->stream));
         BCK(cudaStreamSynchronize(b->stream));
     }
     b->ras_new = false;
@@ -1108,30 +1084,7 @@ int drain_raster(snn_batch* b, bool keep) {
         for (size_t i = at; i < out.size(); ++i) out[i] -= lo;
         r = e;
     }
-    b->part_left = b->part_cap / b->part_ncmax;
-    b->ras_kept += small.lost ? (unsigned long long)b->ras_cap + 1ull : m;
-    return kept_raster(b, keep);
-}
-
-int part_counts(snn_batch* b, std::vector<uint32_t>* n) {
-    n->resize(b->part_grid);
-    BCK(cudaStreamSynchronize(b->stream));
-    BCK(cudaMemcpy(n->data(), b->d_part_n, sizeof(uint32_t) * b->part_grid, cudaMemcpyDeviceToHost));
-    return SNN_OK;
-}
-
-// Steps that may be issued before a partition's raster list could be full: a
-// neuron spikes at most once a step.  A list that holds the whole capacity
-// needs no look.  Otherwise, when they are used up, the counts are read and
-// lists more than half full drained.
-int make_room(snn_batch* b) {
-    if (!b->part || b->part_cap >= b->ras_cap || b->part_left > 0) return SNN_OK;
-    std::vector<uint32_t> n;
-    BCALL(part_counts(b, &n));
-    const uint32_t most = *std::max_element(n.begin(), n.end());
-    if (most > b->part_cap / 2) return drain_raster(b, true);
-    b->part_left = (b->part_cap - most) / b->part_ncmax;
-    return SNN_OK;
+    return small.lost ? set_error(SNN_ERR_OVERFLOW, "batch raster capacity exceeded") : SNN_OK;
 }
 
 }  // namespace
@@ -1283,16 +1236,8 @@ int snn_batch_create(const snn_config* cfgs, const uint64_t* seeds, int32_t n_in
     }
     const long long cap = (opt && opt->raster_capacity > 0) ? opt->raster_capacity : (64ll << 20);
     b->ras_cap = (uint32_t)std::min<long long>(cap, 0x7fffffff);
-    long long ras_words = b->ras_cap;
-    if (parts) {
-        // a list per partition; four times its share of the capacity each, as
-        // the populations' rates differ, and no less than kLeastList (one that
-        // could fill up all the same is drained in time, make_room)
+    if (parts)
         for (int P : n_part) b->part_grid += P;
-        b->part_cap = (uint32_t)std::min<long long>(
-            std::max<long long>(4 * (long long)b->ras_cap / b->part_grid, kLeastList), b->ras_cap);
-        ras_words = std::max<long long>(ras_words, (long long)b->part_cap * b->part_grid);
-    }
     if (rc == SNN_OK) rc = balloc(&b->d_hot, n_inst, "batch instance constants");
     if (rc == SNN_OK) rc = balloc(&b->d_cold, n_inst, "batch instance rows");
     if (rc == SNN_OK) rc = balloc(&b->d_pois, pois.size(), "batch background tables");
@@ -1304,8 +1249,8 @@ int snn_batch_create(const snn_config* cfgs, const uint64_t* seeds, int32_t n_in
     if (rc == SNN_OK) rc = balloc(&b->d_ring, (size_t)b->ring_depth * ntot, "batch ring buffers");
     if (rc == SNN_OK) rc = balloc(&b->d_list, (size_t)2 * kTilings * ntot, "batch spike lists");
     if (rc == SNN_OK) rc = balloc(&b->d_cnt, 4 * kTilings, "batch list counters");
-    if (rc == SNN_OK) rc = balloc(&b->d_ras_step, ras_words, "batch raster");
-    if (rc == SNN_OK) rc = balloc(&b->d_ras_id, ras_words, "batch raster");
+    if (rc == SNN_OK) rc = balloc(&b->d_ras_step, b->ras_cap, "batch raster");
+    if (rc == SNN_OK) rc = balloc(&b->d_ras_id, b->ras_cap, "batch raster");
     if (rc == SNN_OK) rc = balloc(&b->d_ras_n, 1, "batch raster count");
     if (rc == SNN_OK) rc = balloc(&b->d_ic, (size_t)2 * n_inst, "batch counters");
     if (rc == SNN_OK) rc = balloc(&b->d_step, 1, "batch step");
@@ -1392,15 +1337,12 @@ int snn_batch_step(snn_batch* b, int64_t n_steps) {
     if (!b || n_steps < 0) return set_error(SNN_ERR_INVALID, "bad arguments");
     int64_t left = n_steps;
     while (left > 0) {
-        BCALL(make_room(b));
         b->ras_new = true;
-        const int64_t room = b->part && b->part_cap < b->ras_cap ? std::min<int64_t>(left, b->part_left) : left;
-        const bool graph = b->graph_ok && room >= kGraphChunk;
-        const int chunk = graph ? kGraphChunk : (int)std::min<int64_t>(room, 1 << 20);
+        const bool graph = b->graph_ok && left >= kGraphChunk;
+        const int chunk = graph ? kGraphChunk : (int)std::min<int64_t>(left, 1 << 20);
         if (graph) BCK(cudaGraphLaunch(b->graph, b->stream));
         else BCK(launch_batch(b, chunk));
         left -= chunk;
-        b->part_left -= chunk;
         b->step += chunk;
     }
     return SNN_OK;
@@ -1413,15 +1355,6 @@ int snn_batch_sync(snn_batch* b) {
     BCK(cudaMemcpy(&st, b->d_sync + 1, sizeof(st), cudaMemcpyDeviceToHost));
     if (st & kStatusTimeout) return set_error(SNN_ERR_TIMEOUT, "a grid-barrier wait timed out");
     if (st & kBatchRasterOverflow) return set_error(SNN_ERR_OVERFLOW, "batch raster capacity exceeded");
-    // side by side the lists together hold more than the capacity
-    if (b->part && b->ras_new &&
-        b->ras_kept + (unsigned long long)(b->step - b->ras_lo) * (unsigned long long)b->ntot > b->ras_cap) {
-        std::vector<uint32_t> n;
-        BCALL(part_counts(b, &n));
-        unsigned long long total = b->ras_kept;
-        for (uint32_t x : n) total += x;
-        if (total > b->ras_cap) return set_error(SNN_ERR_OVERFLOW, "batch raster capacity exceeded");
-    }
     return SNN_OK;
 }
 
@@ -1429,7 +1362,7 @@ int snn_batch_read_spikes(snn_batch* b, int32_t k, uint32_t* steps_host, uint32_
                           int64_t cap, int64_t* n) {
     if (!b || k < 0 || k >= b->n_inst || !n || cap < 0)
         return set_error(SNN_ERR_INVALID, "bad arguments");
-    const int rc = drain_raster(b, false);
+    const int rc = drain_raster(b);
     auto& st = b->host_steps[k];
     auto& id = b->host_ids[k];
     const int64_t m = std::min<int64_t>(cap, (int64_t)st.size());

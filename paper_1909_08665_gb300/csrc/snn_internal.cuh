@@ -156,7 +156,7 @@ struct StepParams {
     uint32_t key0, key1;
     int64_t t0;
     int32_t n_steps;
-    uint32_t ras_cap;                   // raster capacity per partition
+    uint32_t ras_cap;                   // raster capacity per partition (side by side: in all)
     uint64_t timeout_ns;
     int32_t inject_fault;               // 1: partition 0 never publishes
     int32_t msg_stride;                 // 64-bit words per message (>= ncmax + 1)
@@ -175,10 +175,10 @@ struct StepParams {
     int32_t* refr;
     int32_t* ring;                      // [n_part][kRing][ncmax]
     unsigned long long* msg;            // [4][n_part][msg_stride] tagged spike messages
-    uint32_t* ras_step;                 // [n_part][ras_cap]
+    uint32_t* ras_step;                 // [n_part][ras_cap] (side by side: [ras_cap])
     uint32_t* ras_id;
-    uint32_t* ras_n;                    // [n_part] spikes recorded (may exceed cap)
-    uint32_t ras_id0;                   // added to the recorded ids
+    uint32_t* ras_n;                    // [n_part] (side by side: [1]) spikes recorded (may exceed cap)
+    uint32_t ras_id0;                   // side by side: added to the recorded ids
     unsigned long long* counters;       // [0] spikes, [1] synaptic events
     unsigned long long* pop_spikes;     // [8] spikes per population
     uint32_t* status;

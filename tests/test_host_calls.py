@@ -1,0 +1,76 @@
+"""What the library's host code asks of the CUDA runtime, seen without a GPU:
+the library runs in a child process on a runtime whose kernels do nothing
+(host/fake_cudart.cpp) and the test reads the log of the calls."""
+import os
+import shutil
+import subprocess
+import sys
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+CUDA = "/usr/local/cuda"
+
+PRELUDE = """
+import ctypes, re, sys
+sys.path.insert(0, {root!r})
+rt = ctypes.CDLL("libcudart.so.13")
+rt.fake_log.restype = ctypes.c_char_p
+rt.fake_alloc_limit.argtypes = [ctypes.c_size_t]
+import numpy as np
+import paper_1909_08665_gb300 as pkg
+import workload
+
+
+def calls(kind):
+    return [x for x in rt.fake_log().decode().splitlines() if x.split()[0] == kind]
+
+
+class Stream:
+    cuda_stream = 0x40
+
+"""
+
+
+@pytest.fixture(scope="module")
+def run(tmp_path_factory):
+    if shutil.which("g++") is None or not os.path.exists(CUDA + "/include/cuda_runtime_api.h"):
+        pytest.skip("needs g++ and the CUDA headers")
+    from paper_1909_08665_gb300 import _build
+    _build.build()
+    d = tmp_path_factory.mktemp("cudart")
+    (d / "version").write_text("libcudart.so.13 { global: *; };\n")
+    subprocess.run(["g++", "-std=c++17", "-O1", "-shared", "-fPIC", "-I", CUDA + "/include",
+                    os.path.join(ROOT, "tests", "host", "fake_cudart.cpp"), "-o", str(d / "libcudart.so.13"),
+                    "-Wl,-soname,libcudart.so.13", "-Wl,--version-script," + str(d / "version")], check=True)
+
+    def go(body):
+        env = dict(os.environ, LD_LIBRARY_PATH=str(d) + ":" + os.environ.get("LD_LIBRARY_PATH", ""))
+        r = subprocess.run([sys.executable, "-c", PRELUDE.format(root=ROOT) + body], env=env, capture_output=True,
+                           text=True, timeout=300)
+        assert r.returncode == 0, r.stdout + r.stderr
+        return r.stdout
+    return go
+
+
+def test_batch_steps_do_not_wait(run):
+    """A batch side by side steps on its stream whatever the number of steps."""
+    run("""
+b = pkg.MicrocircuitBatch([workload.microcircuit(s) for s in (0.03, 0.0123, 0.05)], stream=Stream())
+assert b.info(0)["neurons_per_thread"] == 1
+rt.fake_clear()
+b.step(50_321)
+assert len(calls("graph")) == 50 and calls("launch") and not calls("sync"), rt.fake_log()
+""")
+
+
+def test_batch_raster_is_as_large_as_asked_for(run):
+    """Two arrays of the capacity, and nothing larger."""
+    run("""
+for cap in (0, 4 << 20, 65 << 20):
+    rt.fake_clear()
+    b = pkg.MicrocircuitBatch([workload.microcircuit(0.02)] * 3, stream=Stream(), raster_capacity=cap)
+    sizes = sorted(int(x.split()[-1]) for x in calls("malloc"))
+    assert sizes[-2:] == [4 * (cap or 64 << 20)] * 2 and sizes[-3] < 16 << 20, (cap, sizes[-4:])
+    b.close()
+""")
