@@ -297,11 +297,10 @@ int plan(snn_net* net, const snn_options* opt) {
     const double tmo = (opt && opt->timeout_s > 0) ? opt->timeout_s : 2.0;
     net->timeout_ns = (uint64_t)(tmo * 1e9);
     const int64_t cap = (opt && opt->raster_capacity > 0) ? opt->raster_capacity : (64ll << 20);
-    // A partition's list is its share.  Small partitions share less evenly than
-    // large ones, so of a capacity that was asked for each gets the share of a
-    // partition of 512 neurons.
-    const bool asked = opt && opt->raster_capacity > 0 && cap <= (64ll << 20);
-    net->ras_cap = (uint32_t)std::min<int64_t>(std::max<int64_t>(cap / (asked ? net->adj_part : P), 1), 0x7fffffff);
+    // A partition's list is its share of the capacity.  Small partitions share
+    // less evenly than large ones, so each gets the share of one of 512 neurons,
+    // whatever the capacity: a larger one never means a shorter list.
+    net->ras_cap = (uint32_t)std::min<int64_t>(std::max<int64_t>(cap / net->adj_part, 1), 0x7fffffff);
     net->inject_fault = opt ? opt->inject_fault : 0;
     return SNN_OK;
 }

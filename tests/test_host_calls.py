@@ -74,3 +74,21 @@ for cap in (0, 4 << 20, 65 << 20):
     assert sizes[-2:] == [4 * (cap or 64 << 20)] * 2 and sizes[-3] < 16 << 20, (cap, sizes[-4:])
     b.close()
 """)
+
+
+def test_a_larger_raster_capacity_never_shortens_a_list(run):
+    """A partition's list is the share of a partition of 512 neurons (of all
+    neurons in few), at every capacity and by default."""
+    run("""
+for scale in (0.005, 0.1, 0.3, 1.0):
+    need = -(-workload.n_neurons(workload.microcircuit(scale)) // 512)
+    last = 0
+    for cap in (1 << 20, 16 << 20, 0, 65 << 20, 200 << 20):
+        rt.fake_clear()
+        net = pkg.Microcircuit(workload.microcircuit(scale), stream=Stream(), raster_capacity=cap)
+        sizes = [int(x.split()[-1]) for x in calls("malloc")]
+        entries = (cap or 64 << 20) // min(need, 152)
+        assert sizes.count(4 * entries * net.info()["n_part"]) == 2 and entries > last, (scale, cap, sorted(sizes)[-4:])
+        last = entries
+        net.close()
+""")
