@@ -1048,7 +1048,8 @@ int leave_parts(snn_batch* b) {
 }
 
 // the spikes recorded since the last drain, sorted by (instance, step, id) on
-// the device, appended to each instance's host arrays
+// the device, appended to each instance's host arrays; the caller holds
+// stage.mu, and until it has taken its instance's spikes out of them
 int drain_raster(snn_batch* b) {
     if (!b->ras_new) {                          // no step issued since: nothing recorded
         BCK(cudaStreamSynchronize(b->stream));
@@ -1056,7 +1057,6 @@ int drain_raster(snn_batch* b) {
     }
     const RasterList in = {b->d_ras_n, b->d_ras_step, b->d_ras_id, b->ras_cap, 1, b->n_inst, b->d_goff,
                            (uint32_t)b->ras_lo, b->step - b->ras_lo, (uint32_t)b->ntot};
-    std::lock_guard<std::mutex> hold(b->stage.mu);
     RasterSmall small;
     BCK(raster_read_small(in, b->d_ras_n, &b->stage, b->stream, &small));
     const uint32_t m = small.n;
@@ -1071,8 +1071,6 @@ int drain_raster(snn_batch* b) {
         BCK(cudaMemsetAsync(b->d_ras_n, 0, sizeof(uint32_t), b->stream));
         BCK(cudaStreamSynchronize(b->stream));
     }
-    b->ras_new = false;
-    b->ras_lo = b->step;
     for (uint32_t r = 0, k = 0; r < m; ++k) {
         const uint32_t lo = (uint32_t)b->goff[k], hi = (uint32_t)b->goff[k + 1];
         const uint32_t e = (uint32_t)(std::partition_point(id.begin() + r, id.end(), [&](uint32_t x) { return x < hi; }) -
@@ -1084,6 +1082,8 @@ int drain_raster(snn_batch* b) {
         for (size_t i = at; i < out.size(); ++i) out[i] -= lo;
         r = e;
     }
+    b->ras_new = false;
+    b->ras_lo = b->step;
     return small.lost ? set_error(SNN_ERR_OVERFLOW, "batch raster capacity exceeded") : SNN_OK;
 }
 
@@ -1362,6 +1362,7 @@ int snn_batch_read_spikes(snn_batch* b, int32_t k, uint32_t* steps_host, uint32_
                           int64_t cap, int64_t* n) {
     if (!b || k < 0 || k >= b->n_inst || !n || cap < 0)
         return set_error(SNN_ERR_INVALID, "bad arguments");
+    std::lock_guard<std::mutex> hold(b->stage.mu);
     const int rc = drain_raster(b);
     auto& st = b->host_steps[k];
     auto& id = b->host_ids[k];

@@ -24,7 +24,9 @@ std::recursive_mutex g_mu;
 std::string g_text;
 std::map<const void*, std::string> g_name;
 std::map<const void*, std::pair<void*, size_t>> g_var;
+std::map<void*, size_t> g_alloc;
 size_t g_limit = SIZE_MAX;              // larger allocations fail
+uint32_t* g_count = nullptr;            // the raster count that was read last
 thread_local int g_dev = 0;
 thread_local cudaError_t g_last = cudaSuccess;
 struct Call { dim3 grid, block; size_t smem; cudaStream_t s; };
@@ -39,13 +41,13 @@ cudaError_t launch(const void* fn, void** args, cudaStream_t s) {
     const std::string name = g_name.count(fn) ? g_name[fn] : "?";
     note("launch " + name + " dev " + std::to_string(g_dev) + " stream " + std::to_string((uintptr_t)s));
     // the one kernel whose result the host code branches on: it reports the
-    // number of recorded spikes (above its own limit nothing else)
+    // number of recorded spikes (above its own limit nothing else); a test
+    // sets that of the first list (fake_raster_count)
     if (name.find("k_sort_small") != std::string::npos) {
-        const unsigned long long n = **reinterpret_cast<unsigned long long**>(args[1]);
+        g_count = *reinterpret_cast<uint32_t**>(args[1]);
         uint32_t* head = *reinterpret_cast<uint32_t**>(args[2]);
-        head[0] = (uint32_t)n;
-        head[1] = (uint32_t)(n >> 32);
-        head[2] = 0u;
+        head[0] = *g_count;
+        head[1] = 0u;
     }
     return cudaSuccess;
 }
@@ -54,6 +56,14 @@ cudaError_t launch(const void* fn, void** args, cudaStream_t s) {
 extern "C" {
 const char* fake_log() { return g_text.c_str(); }
 void fake_clear() { g_text.clear(); }
+uint32_t* fake_raster_count() { return g_count; }
+// the k-th live allocation of n bytes, by address
+void* fake_alloc(size_t n, int k) {
+    std::lock_guard<std::recursive_mutex> hold(g_mu);
+    for (const auto& a : g_alloc)
+        if (a.second == n && k-- == 0) return a.first;
+    return nullptr;
+}
 void fake_alloc_limit(size_t bytes) { g_limit = bytes; }
 void fake_set_device(int d) { g_dev = d; }
 int fake_device() { return g_dev; }
@@ -98,9 +108,16 @@ cudaError_t cudaMalloc(void** p, size_t n) {
     note("malloc dev " + std::to_string(g_dev) + " " + std::to_string(n));
     if (n > g_limit) return g_last = cudaErrorMemoryAllocation;
     *p = calloc(1, n ? n : 1);
+    std::lock_guard<std::recursive_mutex> hold(g_mu);
+    g_alloc[*p] = n;
     return *p ? cudaSuccess : (g_last = cudaErrorMemoryAllocation);
 }
-cudaError_t cudaFree(void* p) { free(p); return cudaSuccess; }
+cudaError_t cudaFree(void* p) {
+    std::lock_guard<std::recursive_mutex> hold(g_mu);
+    g_alloc.erase(p);
+    free(p);
+    return cudaSuccess;
+}
 cudaError_t cudaHostAlloc(void** p, size_t n, unsigned) { *p = calloc(1, n); return cudaSuccess; }
 cudaError_t cudaFreeHost(void* p) { free(p); return cudaSuccess; }
 cudaError_t cudaHostGetDevicePointer(void** d, void* h, unsigned) { *d = h; return cudaSuccess; }

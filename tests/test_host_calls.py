@@ -17,9 +17,17 @@ sys.path.insert(0, {root!r})
 rt = ctypes.CDLL("libcudart.so.13")
 rt.fake_log.restype = ctypes.c_char_p
 rt.fake_alloc_limit.argtypes = [ctypes.c_size_t]
+rt.fake_alloc.restype = ctypes.c_void_p
+rt.fake_alloc.argtypes = [ctypes.c_size_t, ctypes.c_int]
+rt.fake_raster_count.restype = ctypes.POINTER(ctypes.c_uint32)
 import numpy as np
 import paper_1909_08665_gb300 as pkg
 import workload
+
+
+def words(n, k):
+    # the k-th device array of n 32-bit words
+    return np.ctypeslib.as_array(ctypes.cast(rt.fake_alloc(4 * n, k), ctypes.POINTER(ctypes.c_uint32)), (n,))
 
 
 def calls(kind):
@@ -91,4 +99,38 @@ for scale in (0.005, 0.1, 0.3, 1.0):
         assert sizes.count(4 * entries * net.info()["n_part"]) == 2 and entries > last, (scale, cap, sorted(sizes)[-4:])
         last = entries
         net.close()
+""")
+
+
+def test_batch_spikes_read_by_two_threads(run):
+    """A read that finds the raster drained waits until another thread's drain
+    has handed the spikes out."""
+    run("""
+import threading, time
+n = 3_000_000
+b = pkg.MicrocircuitBatch([workload.microcircuit(0.02)] * 2, stream=Stream())
+b.step(1)
+b.read_spikes(0)
+bufs = [np.empty((2, n), np.uint32) for _ in range(2)]
+rt.fake_raster_count()[0] = n
+b.step(1)
+b.read_spikes_into(0, *bufs[0])             # makes the arrays the sorted spikes lie in
+for delay in range(200):                    # at every stage of the other's drain
+    b.step(1)
+    rt.fake_raster_count()[0] = n           # all of instance 0
+    words(n, 0)[:] = words(n, 1)[:] = delay
+    got, done = [0, 0], threading.Event()
+
+    def drain():
+        got[1] = b.read_spikes_into(1, *bufs[1])
+        done.set()
+
+    t = threading.Thread(target=drain)
+    t.start()
+    time.sleep(delay * 1.25e-4)
+    while not done.is_set():
+        got[0] += b.read_spikes_into(0, *bufs[0])
+    t.join()
+    got[0] += b.read_spikes_into(0, *bufs[0])
+    assert got == [n, 0] and (bufs[0] == delay).all(), (delay, got)
 """)
