@@ -1336,6 +1336,7 @@ int snn_batch_create(const snn_config* cfgs, const uint64_t* seeds, int32_t n_in
 int snn_batch_step(snn_batch* b, int64_t n_steps) {
     if (!b || n_steps < 0) return set_error(SNN_ERR_INVALID, "bad arguments");
     int64_t left = n_steps;
+    std::lock_guard<std::mutex> hold(b->stage.mu);      // not while another thread drains the raster
     while (left > 0) {
         b->ras_new = true;
         const bool graph = b->graph_ok && left >= kGraphChunk;
@@ -1436,6 +1437,7 @@ int snn_batch_get_info(snn_batch* b, int32_t k, snn_batch_info* info) {
 int snn_batch_set_tiling(snn_batch* b, int32_t k, int32_t tiling) {
     if (!b || k < 0 || k >= b->n_inst || tiling < 0 || tiling >= kTilings)
         return set_error(SNN_ERR_INVALID, "bad arguments");
+    std::lock_guard<std::mutex> hold(b->stage.mu);
     b->hot_h[k].key.z = (uint32_t)tiling;
     if (b->part) BCALL(leave_parts(b));
     BCK(cudaMemcpyAsync(b->d_hot + k, &b->hot_h[k], sizeof(InstHot), cudaMemcpyHostToDevice,

@@ -683,6 +683,9 @@ void fill_step_params(const snn_net* net, StepParams* out) {
 cudaError_t net_launch(snn_net* net, StepParams& sp, int64_t t0, int64_t n) {
     const int64_t kMaxLaunch = 1ll << 24;
     int64_t left = n, t = t0;
+    // a raster read by another thread sees the steps of all launches before it
+    // and of none after it
+    std::lock_guard<std::mutex> hold(net->stage.mu);
     if (n > 0) {
         net->ras_lo = std::min(net->ras_lo, t0);
         net->ras_hi = std::max(net->ras_hi, t0 + n);
@@ -908,11 +911,11 @@ int snn_sync(snn_net* net) {
 int snn_read_spikes(snn_net* net, uint32_t* steps_host, uint32_t* ids_host, int64_t cap,
                     int64_t* n) {
     if (!net || !n || cap < 0) return fail(SNN_ERR_INVALID, "bad arguments");
+    std::lock_guard<std::mutex> hold(net->stage.mu);
     const RasterList in = {net->d_ras_n, net->d_ras_step, net->d_ras_id, net->ras_cap, net->P, 1, nullptr,
                            (uint32_t)net->ras_lo, net->ras_hi - net->ras_lo, (uint32_t)net->n};
     int64_t total = 0;
     bool lost = false;
-    std::lock_guard<std::mutex> hold(net->stage.mu);
     if (net->P < kStepThreads) {
         RasterSmall r;
         CK(raster_read_small(in, net->d_ras_n, &net->stage, net->stream, &r));

@@ -45,6 +45,7 @@ struct SortParams {
     uint32_t t_lo;                   // first step that may occur
     uint32_t per_inst;               // buckets of one instance
     uint32_t n_groups;
+    uint32_t n;                      // spikes the arrays below hold
     int32_t id_bits, shift;          // 2^shift steps share a bucket
     uint32_t* group;                 // [n_groups] counts, then ends of the buckets
     unsigned long long* key;         // [n] keys, bucket by bucket
@@ -124,7 +125,7 @@ __global__ void __launch_bounds__(kThreads) k_sort_scatter(const __grid_constant
     for_each_spike(p, [&](uint32_t s, uint32_t id) {
         const uint32_t at = atomicAdd(&p.group[group_of(p, s, id)], 1u);
         const uint32_t low = (s - p.t_lo) & ((1u << p.shift) - 1u);
-        p.key[at] = ((unsigned long long)low << p.id_bits) | id;
+        if (at < p.n) p.key[at] = ((unsigned long long)low << p.id_bits) | id;
     });
 }
 
@@ -149,6 +150,13 @@ __device__ __forceinline__ void rank_keys(const SortParams& p, const unsigned lo
     }
 }
 
+// bucket g's keys are [b, b + n): within the arrays even if the lists were changed
+// since their spikes were counted
+__device__ __forceinline__ void bucket(const SortParams& p, uint32_t g, uint32_t& b, uint32_t& n) {
+    b = g ? min(p.group[g - 1], p.n) : 0u;
+    n = min(p.group[g], p.n) - b;
+}
+
 __device__ __forceinline__ uint32_t first_step(const SortParams& p, uint32_t g) {
     return p.t_lo + ((g % p.per_inst) << p.shift);
 }
@@ -156,7 +164,8 @@ __device__ __forceinline__ uint32_t first_step(const SortParams& p, uint32_t g) 
 __global__ void __launch_bounds__(kThreads) k_sort_groups(const __grid_constant__ SortParams p) {
     const uint32_t warps = gridDim.x * (kThreads / 32);
     for (uint32_t g = (blockIdx.x * kThreads + threadIdx.x) >> 5; g < p.n_groups; g += warps) {
-        const uint32_t b = g ? p.group[g - 1] : 0u, n = p.group[g] - b;
+        uint32_t b, n;
+        bucket(p, g, b, n);
         if (n <= kWarpGroup) rank_keys(p, p.key, b, n, first_step(p, g));
     }
 }
@@ -167,12 +176,14 @@ __global__ void __launch_bounds__(kBigThreads) k_sort_large(const __grid_constan
     __shared__ uint32_t s_bin[kBins + 1], s_at[kBins], s_w[kBigThreads / 32];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int bin_shift = max(0, p.id_bits + p.shift - kBinBits);
+    auto bin_of = [&](unsigned long long k) { return (uint32_t)min(k >> bin_shift, (unsigned long long)(kBins - 1)); };
     for (uint32_t g = blockIdx.x; g < p.n_groups; g += gridDim.x) {
-        const uint32_t b = g ? p.group[g - 1] : 0u, n = p.group[g] - b;
+        uint32_t b, n;
+        bucket(p, g, b, n);
         if (n <= kWarpGroup) continue;
         for (int k = tid; k < kBins; k += kBigThreads) s_bin[k] = 0u;
         __syncthreads();
-        for (uint32_t i = tid; i < n; i += kBigThreads) atomicAdd(&s_bin[p.key[b + i] >> bin_shift], 1u);
+        for (uint32_t i = tid; i < n; i += kBigThreads) atomicAdd(&s_bin[bin_of(p.key[b + i])], 1u);
         __syncthreads();
         // exclusive scan, two bins a thread
         const uint32_t v0 = s_bin[2 * tid], v1 = s_bin[2 * tid + 1];
@@ -192,7 +203,7 @@ __global__ void __launch_bounds__(kBigThreads) k_sort_large(const __grid_constan
         __syncthreads();
         for (uint32_t i = tid; i < n; i += kBigThreads) {
             const unsigned long long k = p.key[b + i];
-            p.key2[b + atomicAdd(&s_at[k >> bin_shift], 1u)] = k;
+            p.key2[b + atomicAdd(&s_at[bin_of(k)], 1u)] = k;
         }
         __syncthreads();
         for (int k = warp; k < kBins; k += kBigThreads / 32) {
@@ -375,6 +386,7 @@ cudaError_t raster_sort(RasterSort* w, const RasterList& in, size_t n, cudaStrea
     while ((((span - 1) >> p.shift) + 1) > most) ++p.shift;
     p.per_inst = (uint32_t)(((span - 1) >> p.shift) + 1);
     p.n_groups = p.per_inst * (uint32_t)in.n_inst;
+    p.n = (uint32_t)n;
     e = grow(&w->group, &w->group_cap, p.n_groups);
     if (e == cudaSuccess) e = grow(&w->key, &w->key_cap, 2 * n);
     if (e != cudaSuccess) return e;

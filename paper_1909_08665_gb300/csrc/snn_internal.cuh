@@ -298,8 +298,9 @@ struct RasterSort {
 cudaError_t raster_sort(RasterSort* w, const RasterList& in, size_t n, cudaStream_t s);
 // Pinned host memory that kernels write small results into (grows, is kept).
 // mu is held from the launch until the result is copied out (of a batch's spikes:
-// out of its host lists): one handle may be read from several threads.
-// read_arrays takes it, callers of raster_read_small hold it.
+// out of its host lists), and while steps are issued: one handle may be read
+// from several threads, and while another thread steps it.  read_arrays takes
+// it, callers of raster_read_small hold it.
 struct HostStage {
     std::mutex mu;
     void* host = nullptr;
