@@ -13,6 +13,9 @@
  *    allocation it makes and frees it in snn_destroy().
  *  - `stream` is a cudaStream_t passed as void*; NULL means the legacy
  *    default stream.  Device work of a network is issued on that stream only.
+ *  - A handle belongs to the device that was current when it was made.  Reads
+ *    (spikes, state, ring, counters, saving and loading) may be called with
+ *    any device current; the other calls need the handle's.
  *  - The library needs an sm_103a GPU; on any other device snn_create()
  *    fails with SNN_ERR_UNSUPPORTED.  There is no CPU fallback.
  *

@@ -610,6 +610,7 @@ size_t batch_smem(int npt, int n_inst) {
 using namespace snn;
 
 struct snn_batch {
+    int device = 0;                      // the one that was current when it was made
     int n_inst = 0;
     int ntot = 0;
     int npt = 0;
@@ -1103,6 +1104,7 @@ int snn_batch_create(const snn_config* cfgs, const uint64_t* seeds, int32_t n_in
     if (prop.major != 10 || prop.minor != 3)
         return set_error(SNN_ERR_UNSUPPORTED, "this library is built for sm_103 (GB300) GPUs only");
     snn_batch* b = new snn_batch();
+    b->device = dev;
     b->stream = reinterpret_cast<cudaStream_t>(stream);
     cudaStream_t s = b->stream;
     b->n_inst = n_inst;
@@ -1363,6 +1365,7 @@ int snn_batch_read_spikes(snn_batch* b, int32_t k, uint32_t* steps_host, uint32_
                           int64_t cap, int64_t* n) {
     if (!b || k < 0 || k >= b->n_inst || !n || cap < 0)
         return set_error(SNN_ERR_INVALID, "bad arguments");
+    const DeviceScope on(b->device);
     std::lock_guard<std::mutex> hold(b->stage.mu);
     const int rc = drain_raster(b);
     auto& st = b->host_steps[k];
@@ -1384,6 +1387,7 @@ int snn_batch_read_spikes(snn_batch* b, int32_t k, uint32_t* steps_host, uint32_
 int snn_batch_read_state(snn_batch* b, int32_t k, float* u_host, float* i_syn_host,
                          int32_t* refr_host) {
     if (!b || k < 0 || k >= b->n_inst) return set_error(SNN_ERR_INVALID, "bad arguments");
+    const DeviceScope on(b->device);
     const InstCold& C = b->cold_h[k];
     if (C.n <= kStageNeurons) {
         const uint32_t* const src[3] = {reinterpret_cast<const uint32_t*>(b->d_u) + C.goff,
@@ -1405,6 +1409,7 @@ int snn_batch_read_state(snn_batch* b, int32_t k, float* u_host, float* i_syn_ho
 
 int snn_batch_counters(snn_batch* b, int32_t k, int64_t* step, uint64_t* spikes, uint64_t* events) {
     if (!b || k < 0 || k >= b->n_inst) return set_error(SNN_ERR_INVALID, "bad arguments");
+    const DeviceScope on(b->device);
     unsigned long long c[2];
     const uint32_t* const src[1] = {reinterpret_cast<const uint32_t*>(b->d_ic + 2 * k)};
     uint32_t* const dst[1] = {reinterpret_cast<uint32_t*>(c)};

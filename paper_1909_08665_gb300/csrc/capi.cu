@@ -250,6 +250,7 @@ int dalloc(T** p, size_t count, const char* what) {
 int plan(snn_net* net, const snn_options* opt) {
     int dev = 0;
     CK(cudaGetDevice(&dev));
+    net->device = dev;
     cudaDeviceProp prop;
     CK(cudaGetDeviceProperties(&prop, dev));
     if (prop.major != 10 || prop.minor != 3)
@@ -761,6 +762,7 @@ int net_update_saturation(snn_net* net) {
 }
 
 int net_ring_to_host(snn_net* net, int32_t* host) {
+    const DeviceScope on(net->device);
     const size_t words = (size_t)kRing * net->n;
     std::lock_guard<std::mutex> hold(net->stage.mu);
     if (!net->d_ring_io) CALL(dalloc(&net->d_ring_io, words, "ring staging"));
@@ -772,6 +774,7 @@ int net_ring_to_host(snn_net* net, int32_t* host) {
 }
 
 int net_ring_from_host(snn_net* net, const int32_t* host) {
+    const DeviceScope on(net->device);
     const size_t words = (size_t)kRing * net->n;
     std::lock_guard<std::mutex> hold(net->stage.mu);
     if (!net->d_ring_io) CALL(dalloc(&net->d_ring_io, words, "ring staging"));
@@ -911,6 +914,7 @@ int snn_sync(snn_net* net) {
 int snn_read_spikes(snn_net* net, uint32_t* steps_host, uint32_t* ids_host, int64_t cap,
                     int64_t* n) {
     if (!net || !n || cap < 0) return fail(SNN_ERR_INVALID, "bad arguments");
+    const DeviceScope on(net->device);
     std::lock_guard<std::mutex> hold(net->stage.mu);
     const RasterList in = {net->d_ras_n, net->d_ras_step, net->d_ras_id, net->ras_cap, net->P, 1, nullptr,
                            (uint32_t)net->ras_lo, net->ras_hi - net->ras_lo, (uint32_t)net->n};
@@ -960,6 +964,7 @@ int snn_read_spikes(snn_net* net, uint32_t* steps_host, uint32_t* ids_host, int6
 
 int snn_raster_size(snn_net* net, int64_t* n) {
     if (!net || !n) return fail(SNN_ERR_INVALID, "bad arguments");
+    const DeviceScope on(net->device);
     uint32_t cnt[kStepThreads];
     const uint32_t* const src[1] = {net->d_ras_n};
     uint32_t* const dst[1] = {cnt};
@@ -972,6 +977,7 @@ int snn_raster_size(snn_net* net, int64_t* n) {
 
 int snn_read_state(snn_net* net, float* u_host, float* i_syn_host, int32_t* refr_host) {
     if (!net) return fail(SNN_ERR_INVALID, "net is NULL");
+    const DeviceScope on(net->device);
     if (net->n <= kStageNeurons) {
         const uint32_t* const src[3] = {reinterpret_cast<const uint32_t*>(net->d_u),
                                         reinterpret_cast<const uint32_t*>(net->d_i),
@@ -995,6 +1001,7 @@ int snn_read_ring(snn_net* net, int32_t* ring_host) {
 
 int snn_counters(snn_net* net, int64_t* step, uint64_t* spikes, uint64_t* events) {
     if (!net) return fail(SNN_ERR_INVALID, "net is NULL");
+    const DeviceScope on(net->device);
     unsigned long long c[2];
     const uint32_t* const src[1] = {reinterpret_cast<const uint32_t*>(net->d_counters)};
     uint32_t* const dst[1] = {reinterpret_cast<uint32_t*>(c)};

@@ -18,6 +18,7 @@ struct snn_net {
     snn_config cfg;
     uint64_t seed;
     cudaStream_t stream;
+    int device = 0;                        // the one that was current when it was made
     int n, n_pop, P, ncmax, npt;
     bool smem_ring;
     int adj_part = 1;                      // partitions of the partition-local adjoint

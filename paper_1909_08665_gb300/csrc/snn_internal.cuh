@@ -251,6 +251,24 @@ inline cudaError_t allow_shared(const void* fn) {
     return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)a.sharedSizeBytes);
 }
 
+// Makes a handle's device the calling thread's current one for the life of the
+// object: the reads launch kernels and allocate staging, wherever the caller is.
+class DeviceScope {
+public:
+    explicit DeviceScope(int dev) {
+        int cur = dev;
+        if (cudaGetDevice(&cur) == cudaSuccess && cur != dev && cudaSetDevice(dev) == cudaSuccess) back_ = cur;
+    }
+    ~DeviceScope() {
+        if (back_ >= 0) cudaSetDevice(back_);
+    }
+    DeviceScope(const DeviceScope&) = delete;
+    DeviceScope& operator=(const DeviceScope&) = delete;
+
+private:
+    int back_ = -1;
+};
+
 // host-side launchers (defined in the .cu files)
 cudaError_t launch_build_count(const BuildParams& bp, uint32_t* rowlen, cudaStream_t s);
 cudaError_t launch_build_scan(const uint32_t* rowlen, int n, unsigned long long* row_start,

@@ -134,3 +134,27 @@ for delay in range(200):                    # at every stage of the other's drai
     got[0] += b.read_spikes_into(0, *bufs[0])
     assert got == [n, 0] and (bufs[0] == delay).all(), (delay, got)
 """)
+
+
+def test_reads_work_from_another_device(run):
+    """A handle's reads launch and allocate on its own device, whichever one is
+    current, and leave that current."""
+    run("""
+net = pkg.Microcircuit(workload.microcircuit(0.02), stream=Stream())
+large = pkg.Microcircuit(workload.microcircuit(0.5), stream=Stream())
+b = pkg.MicrocircuitBatch([workload.microcircuit(0.02)] * 2, stream=Stream())
+many = [np.empty(5000, np.uint32) for _ in range(2)]
+for h, read in ((net, lambda: net.read_spikes_into(*many)), (b, lambda: b.read_spikes_into(1, *many))):
+    h.step(3)
+    read()
+    rt.fake_raster_count()[0] = 5000         # sorted on the device by the next read
+    h.step(3)
+    for call in (read, net.raster_size, net.counters, net.ring, net.state, large.state,
+                 lambda: net.load_state(net.save_state()), lambda: b.state(1), lambda: b.counters(0)):
+        rt.fake_set_device(1)
+        rt.fake_clear()
+        call()
+        assert rt.fake_device() == 1
+        assert not [x for x in calls("launch") + calls("malloc") if " dev 0" not in x], rt.fake_log()
+        rt.fake_set_device(0)
+""")
