@@ -1060,15 +1060,20 @@ int drain_raster(snn_batch* b) {
                            (uint32_t)b->ras_lo, b->step - b->ras_lo, (uint32_t)b->ntot};
     RasterSmall small;
     BCK(raster_read_small(in, b->d_ras_n, &b->stage, b->stream, &small));
-    const uint32_t m = small.n;
+    const uint32_t m = (uint32_t)small.n;       // at most ras_cap
     std::vector<uint32_t> st(m), id(m);
     if (small.done) {
         std::memcpy(st.data(), small.step, sizeof(uint32_t) * m);
         std::memcpy(id.data(), small.id, sizeof(uint32_t) * m);
     } else {
-        BCK(raster_sort(&b->ras_sort, in, m, b->stream));
-        BCK(cudaMemcpyAsync(st.data(), b->ras_sort.step, sizeof(uint32_t) * m, cudaMemcpyDeviceToHost, b->stream));
-        BCK(cudaMemcpyAsync(id.data(), b->ras_sort.id, sizeof(uint32_t) * m, cudaMemcpyDeviceToHost, b->stream));
+        const cudaError_t e = raster_sort(&b->ras_sort, in, m, b->stream);
+        if (e == cudaErrorMemoryAllocation) {
+            BCK(raster_sort_host(in, m, m, b->goff.data(), st.data(), id.data(), b->stream));
+        } else {
+            BCK(e);
+            BCK(cudaMemcpyAsync(st.data(), b->ras_sort.step, sizeof(uint32_t) * m, cudaMemcpyDeviceToHost, b->stream));
+            BCK(cudaMemcpyAsync(id.data(), b->ras_sort.id, sizeof(uint32_t) * m, cudaMemcpyDeviceToHost, b->stream));
+        }
         BCK(cudaMemsetAsync(b->d_ras_n, 0, sizeof(uint32_t), b->stream));
         BCK(cudaStreamSynchronize(b->stream));
     }
@@ -1367,7 +1372,12 @@ int snn_batch_read_spikes(snn_batch* b, int32_t k, uint32_t* steps_host, uint32_
         return set_error(SNN_ERR_INVALID, "bad arguments");
     const DeviceScope on(b->device);
     std::lock_guard<std::mutex> hold(b->stage.mu);
-    const int rc = drain_raster(b);
+    int rc;
+    try {
+        rc = drain_raster(b);
+    } catch (const std::bad_alloc&) {
+        return set_error(SNN_ERR_OOM, "batch raster read: host memory");
+    }
     auto& st = b->host_steps[k];
     auto& id = b->host_ids[k];
     const int64_t m = std::min<int64_t>(cap, (int64_t)st.size());

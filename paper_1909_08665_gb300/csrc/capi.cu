@@ -923,7 +923,7 @@ int snn_read_spikes(snn_net* net, uint32_t* steps_host, uint32_t* ids_host, int6
     if (net->P < kStepThreads) {
         RasterSmall r;
         CK(raster_read_small(in, net->d_ras_n, &net->stage, net->stream, &r));
-        total = r.n;
+        total = (int64_t)r.n;
         lost = r.lost;
         if (r.done) {
             const int64_t got = std::min<int64_t>(total, cap);
@@ -946,7 +946,17 @@ int snn_read_spikes(snn_net* net, uint32_t* steps_host, uint32_t* ids_host, int6
     // sorted on the device, the first `cap` copied back, one transfer per array
     const int64_t got = std::min<int64_t>(total, cap);
     if (got > 0 && (steps_host || ids_host)) {
-        CK(raster_sort(&net->ras_sort, in, (size_t)total, net->stream));
+        const cudaError_t e = raster_sort(&net->ras_sort, in, (size_t)total, net->stream);
+        if (e == cudaErrorMemoryAllocation) {
+            try {
+                CK(raster_sort_host(in, (uint64_t)total, (uint64_t)got, nullptr, steps_host, ids_host, net->stream));
+            } catch (const std::bad_alloc&) {
+                return fail(SNN_ERR_OOM, "raster read: device and host memory");
+            }
+            steps_host = ids_host = nullptr;
+        } else {
+            CK(e);
+        }
         if (steps_host)
             CK(cudaMemcpyAsync(steps_host, net->ras_sort.step, sizeof(uint32_t) * got,
                                cudaMemcpyDeviceToHost, net->stream));

@@ -22,6 +22,7 @@
 // seven launches and the one-CTA scan, not by the 4 MB it moves.
 #include <algorithm>
 #include <cstring>
+#include <vector>
 
 #include "snn_internal.cuh"
 
@@ -216,33 +217,45 @@ __global__ void __launch_bounds__(kBigThreads) k_sort_large(const __grid_constan
 static_assert(kBins == 2 * kBigThreads, "two bins a thread in the scan");
 
 // At most kSmall spikes: one CTA, one launch, all keys in shared memory.  It
-// also counts: head[0] is the number of spikes (clamped counts), head[1] 1 if
-// a list ran out of capacity.  Up to kSmall spikes are sorted out, and the
-// lists are cleared; of more nothing else happens.
+// also counts: head[0], head[1] are the halves of the number of spikes (clamped
+// counts), head[2] is 1 if a list ran out of capacity.  Up to kSmall spikes are
+// sorted out, and the lists are cleared; of more nothing else happens.
 __global__ void __launch_bounds__(kSmall) k_sort_small(const __grid_constant__ SortParams p, uint32_t* counts,
                                                        uint32_t* head) {
     __shared__ unsigned long long s_key[kSmall];
     __shared__ uint32_t s_off[kStepThreads + 1], s_w[32];
+    __shared__ unsigned long long s_sum[32];
     const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
     const uint32_t raw = tid < (uint32_t)p.n_part ? counts[tid] : 0u;
     const uint32_t m = min(raw, p.cap_part);
     const bool lost = __syncthreads_or(raw > p.cap_part) != 0;
-    uint32_t x = m;
+    // the lists' places, exact as far as they are used: a list counts as kSmall
+    // + 1 spikes at most, so the sum tells whether there are more than kSmall
+    const uint32_t few = min(m, kSmall + 1u);
+    uint32_t x = few;
+    unsigned long long sum = m;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
         const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
         if (lane >= (uint32_t)o) x += y;
+        sum += __shfl_xor_sync(0xffffffffu, sum, o);
     }
-    if (lane == 31u) s_w[warp] = x;
+    if (lane == 31u) {
+        s_w[warp] = x;
+        s_sum[warp] = sum;
+    }
     __syncthreads();
-    uint32_t off = x - m;
+    uint32_t off = x - few;
     for (uint32_t w = 0; w < warp; ++w) off += s_w[w];
     if (tid <= (uint32_t)p.n_part) s_off[tid] = off;
     __syncthreads();
     const uint32_t n = s_off[p.n_part];
     if (tid == 0) {
-        head[0] = n;
-        head[1] = lost ? 1u : 0u;
+        sum = 0ull;
+        for (uint32_t w = 0; w * 32u < (uint32_t)p.n_part; ++w) sum += s_sum[w];
+        head[0] = (uint32_t)sum;
+        head[1] = (uint32_t)(sum >> 32);
+        head[2] = lost ? 1u : 0u;
     }
     if (n > kSmall) return;
     if (tid < (uint32_t)p.n_part) counts[tid] = 0u;
@@ -355,41 +368,79 @@ void raster_sort_free(RasterSort* w) {
 
 cudaError_t raster_read_small(const RasterList& in, uint32_t* counts, HostStage* stage, cudaStream_t s,
                               RasterSmall* out) {
+    constexpr size_t kHead = 4;
     uint32_t *host = nullptr, *dev = nullptr;
-    cudaError_t e = host_stage(stage, (2 + 2 * (size_t)kSmall) * sizeof(uint32_t), &host, &dev);
+    cudaError_t e = host_stage(stage, (kHead + 2 * (size_t)kSmall) * sizeof(uint32_t), &host, &dev);
     if (e != cudaSuccess) return e;
     SortParams p = common_params(in);
-    p.step_out = dev + 2;
-    p.id_out = dev + 2 + kSmall;
+    p.step_out = dev + kHead;
+    p.id_out = dev + kHead + kSmall;
     k_sort_small<<<1, kSmall, 0, s>>>(p, counts, dev);
     e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return e;
-    out->n = host[0];
-    out->lost = host[1] != 0u;
-    out->done = host[0] <= kSmall;
-    out->step = host + 2;
-    out->id = host + 2 + kSmall;
+    out->n = (uint64_t)host[1] << 32 | host[0];
+    out->lost = host[2] != 0u;
+    out->done = out->n <= kSmall;
+    out->step = host + kHead;
+    out->id = host + kHead + kSmall;
+    return cudaSuccess;
+}
+
+cudaError_t raster_sort_host(const RasterList& in, uint64_t n, uint64_t limit, const int32_t* goff,
+                             uint32_t* steps, uint32_t* ids, cudaStream_t s) {
+    constexpr size_t kPiece = 1u << 20;
+    std::vector<uint32_t> cnt(in.n_part), st(kPiece), id(kPiece);
+    std::vector<uint64_t> key;                   // step since t_lo, id
+    key.reserve(n);
+    cudaError_t e = cudaMemcpyAsync(cnt.data(), in.counts, sizeof(uint32_t) * in.n_part, cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    for (int c = 0; c < in.n_part && e == cudaSuccess; ++c) {
+        const size_t m = std::min(cnt[c], in.cap_part), base = (size_t)c * in.cap_part;
+        for (size_t at = 0; at < m && e == cudaSuccess; at += kPiece) {
+            const size_t k = std::min(kPiece, m - at);
+            e = cudaMemcpyAsync(st.data(), in.step + base + at, sizeof(uint32_t) * k, cudaMemcpyDeviceToHost, s);
+            if (e == cudaSuccess)
+                e = cudaMemcpyAsync(id.data(), in.id + base + at, sizeof(uint32_t) * k, cudaMemcpyDeviceToHost, s);
+            if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+            for (size_t i = 0; i < k; ++i) key.push_back((uint64_t)(st[i] - in.t_lo) << 32 | id[i]);
+        }
+    }
+    if (e != cudaSuccess) return e;
+    std::sort(key.begin(), key.end());
+    if (in.n_inst > 1) {
+        auto inst = [&](uint64_t x) { return std::upper_bound(goff, goff + in.n_inst + 1, (int32_t)(uint32_t)x) - goff; };
+        std::stable_sort(key.begin(), key.end(), [&](uint64_t a, uint64_t b) { return inst(a) < inst(b); });
+    }
+    limit = std::min<uint64_t>(limit, key.size());
+    for (uint64_t i = 0; i < limit; ++i) {
+        if (steps) steps[i] = in.t_lo + (uint32_t)(key[i] >> 32);
+        if (ids) ids[i] = (uint32_t)key[i];
+    }
     return cudaSuccess;
 }
 
 cudaError_t raster_sort(RasterSort* w, const RasterList& in, size_t n, cudaStream_t s) {
     if (n == 0) return cudaSuccess;
-    cudaError_t e = grow(&w->step, &w->step_cap, n);
-    if (e == cudaSuccess) e = grow(&w->id, &w->id_cap, n);
-    if (e != cudaSuccess) return e;
+    if (n > 0xffffffffull) return cudaErrorMemoryAllocation;     // 32-bit places
     SortParams p = common_params(in);
-    p.step_out = w->step;
-    p.id_out = w->id;
     const long long span = std::max<long long>(1, in.t_span);
     const long long most = std::max<long long>(1, kMaxGroups / in.n_inst);
     while ((((span - 1) >> p.shift) + 1) > most) ++p.shift;
     p.per_inst = (uint32_t)(((span - 1) >> p.shift) + 1);
     p.n_groups = p.per_inst * (uint32_t)in.n_inst;
     p.n = (uint32_t)n;
-    e = grow(&w->group, &w->group_cap, p.n_groups);
+    cudaError_t e = grow(&w->step, &w->step_cap, n);
+    if (e == cudaSuccess) e = grow(&w->id, &w->id_cap, n);
+    if (e == cudaSuccess) e = grow(&w->group, &w->group_cap, p.n_groups);
     if (e == cudaSuccess) e = grow(&w->key, &w->key_cap, 2 * n);
-    if (e != cudaSuccess) return e;
+    if (e != cudaSuccess) {
+        raster_sort_free(w);
+        if (e == cudaErrorMemoryAllocation) cudaGetLastError();      // not sticky: the caller sorts on the host
+        return e;
+    }
+    p.step_out = w->step;
+    p.id_out = w->id;
     p.group = w->group;
     p.key = w->key;
     p.key2 = w->key + n;

@@ -314,6 +314,12 @@ struct RasterSort {
     size_t step_cap = 0, id_cap = 0, group_cap = 0, key_cap = 0;
 };
 cudaError_t raster_sort(RasterSort* w, const RasterList& in, size_t n, cudaStream_t s);
+// The same on the host, the first `limit` of them into steps / ids (each may be
+// null; goff: the instances' id ranges in host memory): for a device without
+// the 24 bytes per spike that raster_sort takes (cudaErrorMemoryAllocation),
+// and for 2^32 spikes or more.  May throw std::bad_alloc.  Waits for the stream.
+cudaError_t raster_sort_host(const RasterList& in, uint64_t n, uint64_t limit, const int32_t* goff,
+                             uint32_t* steps, uint32_t* ids, cudaStream_t s);
 // Pinned host memory that kernels write small results into (grows, is kept).
 // mu is held from the launch until the result is copied out (of a batch's spikes:
 // out of its host lists), and while steps are issued: one handle may be read
@@ -331,7 +337,7 @@ void host_stage_free(HostStage* st);
 // are in step / id (host memory of the stage), sorted, and the lists cleared.
 // n_part must be below kStepThreads.  Waits for the stream.
 struct RasterSmall {
-    uint32_t n;
+    uint64_t n;
     bool lost, done;
     const uint32_t* step;
     const uint32_t* id;

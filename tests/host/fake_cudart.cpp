@@ -24,7 +24,8 @@ std::recursive_mutex g_mu;
 std::string g_text;
 std::map<const void*, std::string> g_name;
 std::map<const void*, std::pair<void*, size_t>> g_var;
-std::map<void*, size_t> g_alloc;
+std::map<long, std::pair<void*, size_t>> g_alloc;    // by number
+long g_allocs = 0;
 size_t g_limit = SIZE_MAX;              // larger allocations fail
 uint32_t* g_count = nullptr;            // the raster count that was read last
 thread_local int g_dev = 0;
@@ -47,7 +48,7 @@ cudaError_t launch(const void* fn, void** args, cudaStream_t s) {
         g_count = *reinterpret_cast<uint32_t**>(args[1]);
         uint32_t* head = *reinterpret_cast<uint32_t**>(args[2]);
         head[0] = *g_count;
-        head[1] = 0u;
+        head[1] = head[2] = 0u;
     }
     return cudaSuccess;
 }
@@ -57,11 +58,11 @@ extern "C" {
 const char* fake_log() { return g_text.c_str(); }
 void fake_clear() { g_text.clear(); }
 uint32_t* fake_raster_count() { return g_count; }
-// the k-th live allocation of n bytes, by address
+// the k-th of the live allocations of n bytes, in the order they were made
 void* fake_alloc(size_t n, int k) {
     std::lock_guard<std::recursive_mutex> hold(g_mu);
     for (const auto& a : g_alloc)
-        if (a.second == n && k-- == 0) return a.first;
+        if (a.second.second == n && k-- == 0) return a.second.first;
     return nullptr;
 }
 void fake_alloc_limit(size_t bytes) { g_limit = bytes; }
@@ -109,12 +110,16 @@ cudaError_t cudaMalloc(void** p, size_t n) {
     if (n > g_limit) return g_last = cudaErrorMemoryAllocation;
     *p = calloc(1, n ? n : 1);
     std::lock_guard<std::recursive_mutex> hold(g_mu);
-    g_alloc[*p] = n;
+    g_alloc[g_allocs++] = {*p, n};
     return *p ? cudaSuccess : (g_last = cudaErrorMemoryAllocation);
 }
 cudaError_t cudaFree(void* p) {
     std::lock_guard<std::recursive_mutex> hold(g_mu);
-    g_alloc.erase(p);
+    for (auto a = g_alloc.begin(); a != g_alloc.end(); ++a)
+        if (a->second.first == p) {
+            g_alloc.erase(a);
+            break;
+        }
     free(p);
     return cudaSuccess;
 }

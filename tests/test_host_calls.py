@@ -158,3 +158,46 @@ for h, read in ((net, lambda: net.read_spikes_into(*many)), (b, lambda: b.read_s
         assert not [x for x in calls("launch") + calls("malloc") if " dev 0" not in x], rt.fake_log()
         rt.fake_set_device(0)
 """)
+
+
+def test_raster_reads_without_device_memory(run):
+    """Where the device has no room for the sort's arrays the spikes come
+    sorted all the same."""
+    run("""
+n, cap = 5000, 77_777
+rng = np.random.default_rng(3)
+net = pkg.Microcircuit(workload.microcircuit(0.02), stream=Stream(), raster_capacity=cap, n_part=1)
+b = pkg.MicrocircuitBatch([workload.microcircuit(0.02)] * 3, stream=Stream(), raster_capacity=cap + 1)
+one = workload.n_neurons(workload.microcircuit(0.02))
+for h, total, entries in ((net, one, cap), (b, 3 * one, cap + 1)):
+    h.step(100)
+    read = h.read_spikes_into if h is net else (lambda s, i: h.read_spikes_into(1, s, i))
+    buf = np.zeros((2, n), np.uint32)
+    read(*buf)
+    h.step(100)
+    rt.fake_raster_count()[0] = n
+    st, ids = words(entries, 0), words(entries, 1)
+    st[:n], ids[:n] = rng.integers(100, 200, n), rng.integers(0, total, n)
+    rt.fake_alloc_limit(1 << 12)
+    got = read(*buf)
+    rt.fake_alloc_limit(1 << 40)
+    st, ids = st[:n], ids[:n]
+    if h is b:
+        mine = (ids >= one) & (ids < 2 * one)
+        st, ids = st[mine], ids[mine] - one
+    order = np.lexsort((ids, st))
+    assert got == st.size > 1000
+    assert (buf[0, :got] == st[order]).all() and (buf[1, :got] == ids[order]).all()
+    h.step(100)
+    rt.fake_raster_count()[0] = n            # a short read keeps the first ones
+    if h is net:
+        st[:] = 100 + st
+        rt.fake_alloc_limit(1 << 12)
+        try:
+            net.read_spikes_into(buf[0, :100], buf[1, :100])
+            assert False
+        except pkg.SnnError as e:
+            assert e.code == pkg.SNN_ERR_OVERFLOW
+        rt.fake_alloc_limit(1 << 40)
+        assert (buf[0, :100] == np.sort(st)[:100]).all()
+""")
