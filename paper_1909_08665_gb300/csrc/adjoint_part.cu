@@ -137,10 +137,6 @@ k_adjoint_part(const __grid_constant__ AdjPartParams p) {
     double* s_gN = reinterpret_cast<double*>(
         (reinterpret_cast<uintptr_t>(s_far + (size_t)p.max_lg * 32) + 7) & ~uintptr_t(7));
     uint8_t* s_mn = reinterpret_cast<uint8_t*>(s_gN + ncmax);
-    // spike flags of the lanes' sources, of two steps: loaded a step ahead, so
-    // that no walk waits for them
-    uint8_t* s_spk = s_mn + ncmax;               // [2][max_lg * 32]
-    const uint32_t spk_row = (uint32_t)p.max_lg * 32u;
 
     if (tid == 0) s_abort = 0u;
     {
@@ -156,8 +152,14 @@ k_adjoint_part(const __grid_constant__ AdjPartParams p) {
     const uint32_t* lenmax_n = ebase + n_lg;         // near columns
     const uint32_t* ebase_n = lenmax_n + n_lg;
     const uint32_t* srcs = ebase_n + n_lg;
-    const uint32_t* lens = srcs + 32 * n_lg;
-    const uint32_t* warp_first = lens + 32 * n_lg;
+    // a word per lane slot: its chunks (m on a source's first lane, else 0) and
+    // the spike flags of its source in the even and the odd steps, loaded a step
+    // ahead, so that no walk waits for them (arrays of their own would take 64
+    // bytes per lane group, 1 % of the shared memory: networks near its limit
+    // would no longer fit)
+    uint8_t* lane_b = reinterpret_cast<uint8_t*>(s_img + kApHeader + 36 * n_lg);
+    auto spk_of = [&](uint32_t slot, int64_t tt) -> uint8_t& { return lane_b[4u * slot + 1u + (uint32_t)(tt & 1)]; };
+    const uint32_t* warp_first = srcs + 64 * n_lg;
     const uint32_t* lg_order = warp_first + kApWarps + 1;
     const uint32_t* ent = s_img + s_img[4];
     const int32_t lo = p.part_lo[c];
@@ -191,15 +193,14 @@ k_adjoint_part(const __grid_constant__ AdjPartParams p) {
     // source's chunks and writes its partial.  Spiking sources' weight
     // partials go to gAc after each walk.
     auto walk = [&](int64_t tt, uint32_t tDt, bool far) {
-        const uint8_t* spk_t = s_spk + (size_t)(tt & 1) * spk_row;
         const uint32_t base_t = tDt * ws;
         for (uint32_t wl = warp_first[warp]; wl < warp_first[warp + 1]; ++wl) {
             const uint32_t L = lg_order[wl];
             const uint32_t j = srcs[L * 32 + lane];
             const uint32_t lm = far ? lenmax[L] : lenmax_n[L];
             const uint32_t eb = far ? ebase[L] : ebase_n[L];
-            const bool spk = (spk_t[L * 32 + lane] & 1u) != 0u;
-            const uint32_t m = lens[L * 32 + lane];
+            const bool spk = (spk_of(L * 32 + lane, tt) & 1u) != 0u;
+            const uint32_t m = lane_b[4u * (L * 32 + lane)];
             const uint32_t* ep = ent + eb + lane;
             float acc = 0.f;
             // entry: weight index << 19 | delay * ws + target; the window
@@ -288,8 +289,8 @@ k_adjoint_part(const __grid_constant__ AdjPartParams p) {
     };
     load_trace(p.len - 1);
     for (uint32_t k = tid; k < 32u * n_lg; k += kApLaunch) {
-        s_spk[(size_t)(t_top & 1) * spk_row + k] = flag_of(k, p.len - 1);
-        if (p.len > 1) s_spk[(size_t)((t_top - 1) & 1) * spk_row + k] = flag_of(k, p.len - 2);
+        spk_of(k, t_top) = flag_of(k, p.len - 1);
+        if (p.len > 1) spk_of(k, t_top - 1) = flag_of(k, p.len - 2);
     }
     __syncthreads();
     uint32_t tD = (uint32_t)(t_top % R);      // window slot of step t
@@ -352,14 +353,13 @@ k_adjoint_part(const __grid_constant__ AdjPartParams p) {
         }
         if (s > 0) walk(t - 1, tD1, true);
         if (s > 1) {
-            uint8_t* row = s_spk + (size_t)(t & 1) * spk_row;
 #pragma unroll
             for (int k = 0; k < kApFlags; ++k) {
                 const uint32_t i = (uint32_t)tid + (uint32_t)k * kApThreads;
-                if (i < 32u * n_lg) row[i] = nf[k];
+                if (i < 32u * n_lg) spk_of(i, t) = nf[k];
             }
             for (uint32_t i = (uint32_t)tid + kApFlags * kApThreads; i < 32u * n_lg; i += kApThreads)
-                row[i] = flag_of(i, s - 2);
+                spk_of(i, t) = flag_of(i, s - 2);
         }
         __syncthreads();                              // the partials of step t are there
         if (s_abort != 0u) break;
@@ -624,8 +624,7 @@ int adjoint_part_plan(int n, int n_pop, const int32_t* pop_start, int n_part, co
     }
     const size_t ws = ((size_t)ncmax + 31) / 32 * 32;
     const size_t smem = img_max * 4 + (size_t)R * ws * 4 + (size_t)2 * (span_max * kMaxPop * kWCodes + 4) * 4 +
-                        (size_t)ncmax * 8 + (size_t)max_lg * 32 * 4 + 8 + (size_t)ncmax * 8 + (size_t)ncmax +
-                        (size_t)max_lg * 64;
+                        (size_t)ncmax * 8 + (size_t)max_lg * 32 * 4 + 8 + (size_t)ncmax * 8 + (size_t)ncmax;
     if (smem > (size_t)optin) return 1;
     plan->grid = n_part * G;
     plan->groups = G;

@@ -201,3 +201,43 @@ for h, total, entries in ((net, one, cap), (b, 3 * one, cap + 1)):
         rt.fake_alloc_limit(1 << 40)
         assert (buf[0, :100] == np.sort(st)[:100]).all()
 """)
+
+
+def test_gradients_near_the_shared_memory_limit_stay_partition_local(run):
+    """The largest network whose rows fit beside the window and the tables: the
+    flags of its spikes take no room of their own."""
+    run("""
+import oracle
+
+
+def adjoint_kernel(scale):
+    # the kernel the backward of a network of this scale launches
+    cfg = workload.microcircuit(scale)
+    rp, tg, dl, code = oracle.Network(cfg).export()
+    n = rp.size - 1
+    parts = -(-n // 512)
+    lo = np.arange(parts + 1) * n // parts
+    ncmax = int(np.diff(lo).max())
+    packed = tg.astype(np.uint32) | dl.astype(np.uint32) << 19 | code.astype(np.uint32) << 25
+    wtab = np.ones((8, 8, 128), np.int32)
+    net = pkg.Microcircuit(cfg, stream=Stream(), n_part=parts, raster_capacity=1 << 16,
+                           rows={"row_ptr": rp, "words": packed, "wtab": wtab})
+    # what the kernels would have made of the rows: every partition's run, and
+    # the entries the step kernel reads
+    src = np.repeat(np.arange(n), np.diff(rp))
+    at = np.searchsorted(src * n + tg, (np.arange(n)[:, None] * n + lo[None]).ravel()).astype(np.uint32)
+    words(n * (parts + 1) + 4)[:at.size] = at
+    pop = np.repeat(np.arange(8), cfg["pop_sizes"])
+    part = np.searchsorted(lo, tg, side="right") - 1
+    index = (pop[tg] * 8 + pop[src]) * 128 + code
+    words(tg.size + 4, 1)[:tg.size] = index.astype(np.uint32) << 19 | (dl.astype(np.uint32) * ncmax + (tg - lo[part]).astype(np.uint32))
+    net.grad_forward(20, 10)
+    rt.fake_clear()
+    net.grad_backward(np.ones(8))
+    names = [x.split()[1] for x in calls("launch") if "k_adjoint" in x and "fold" not in x]
+    net.close()
+    return names[-1]
+
+
+assert "k_adjoint_part" in adjoint_kernel(0.102)
+""")
