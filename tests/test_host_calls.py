@@ -25,7 +25,7 @@ import paper_1909_08665_gb300 as pkg
 import workload
 
 
-def words(n, k):
+def words(n, k=0):
     # the k-th device array of n 32-bit words
     return np.ctypeslib.as_array(ctypes.cast(rt.fake_alloc(4 * n, k), ctypes.POINTER(ctypes.c_uint32)), (n,))
 
