@@ -285,7 +285,7 @@ cudaError_t launch_deliver_stream(const DeliverParams& dp, int w_span, cudaStrea
     if (e != cudaSuccess) return e;
     const size_t smem = stream_smem(dp.ncmax, w_span).total;
     if (smem > (size_t)optin) return cudaErrorInvalidConfiguration;
-    e = cudaFuncSetAttribute(k_deliver_stream, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    e = allow_shared(reinterpret_cast<const void*>(&k_deliver_stream));
     if (e != cudaSuccess) return e;
     k_deliver_stream<<<dp.n_part, kSThreads, smem, s>>>(dp, w_span);
     return cudaGetLastError();

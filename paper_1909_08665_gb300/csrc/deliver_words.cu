@@ -342,7 +342,7 @@ cudaError_t launch_deliver_words(const DeliverParams& dp, cudaStream_t s) {
     if (smem > (size_t)optin) return cudaErrorInvalidConfiguration;
     const void* fn = smem_ring ? reinterpret_cast<const void*>(&k_deliver_words<true>)
                                : reinterpret_cast<const void*>(&k_deliver_words<false>);
-    e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    e = allow_shared(fn);
     if (e != cudaSuccess) return e;
     if (smem_ring)
         k_deliver_words<true><<<dp.n_part, kWThreads, smem, s>>>(dp);

@@ -711,7 +711,7 @@ int snn_grad_backward(snn_net* net, const double* g_rate, double* g_alpha, doubl
                         (n <= kAdjPopTable ? (size_t)n : 0);
     const void* adj_fn = use_pre ? reinterpret_cast<const void*>(&k_adjoint<true>)
                                  : reinterpret_cast<const void*>(&k_adjoint<false>);
-    GCK(cudaFuncSetAttribute(adj_fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    GCK(allow_shared(adj_fn));
 
     StepParams sp;
     fill_step_params(net, &sp);

@@ -173,7 +173,7 @@ cudaError_t launch_deliver_part(const StepParams& sp, const uint32_t* spikes, in
     const size_t smem = part_smem_bytes(sp.ncmax, sp.w_span, smem_ring);
     const void* fn = smem_ring ? reinterpret_cast<const void*>(&k_deliver_part<true>)
                                : reinterpret_cast<const void*>(&k_deliver_part<false>);
-    e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    e = allow_shared(fn);
     if (e != cudaSuccess) return e;
     if (smem_ring)
         k_deliver_part<true><<<sp.n_part, kStepThreads, smem, s>>>(sp, spikes, n, t);

@@ -241,3 +241,24 @@ def adjoint_kernel(scale):
 
 assert "k_adjoint_part" in adjoint_kernel(0.102)
 """)
+
+
+def test_shared_memory_limits_are_never_lowered(run):
+    """A kernel's limit belongs to the whole process: whichever network sets it,
+    it is the most a block may have."""
+    run("""
+nets = [pkg.Microcircuit(workload.microcircuit(s), stream=Stream(), raster_capacity=1 << 16) for s in (0.3, 0.02)]
+spikes = np.zeros(8, np.uint32)
+for net in nets:
+    for tiling in (2, 3, 4, 5):
+        net.deliver(spikes.ctypes.data, 8, 0, tiling)
+    net.grad_forward(4, 2)
+    net.grad_backward(np.ones(8))
+b = pkg.MicrocircuitBatch([workload.microcircuit(0.02)] * 3, stream=Stream(), raster_capacity=1 << 16)
+b.set_tiling(0, 2)
+b.step(5)
+limits = [x.split() for x in calls("attr")]
+for kernel in ("k_deliver_part", "k_deliver_words", "k_deliver_cluster", "k_deliver_stream", "k_adjoint", "k_step", "k_batch"):
+    assert any(kernel in x[1] for x in limits), kernel
+assert {x[2] for x in limits} == {"232448"}, {(x[1], x[2]) for x in limits if x[2] != "232448"}
+""")
