@@ -25,7 +25,7 @@
 #include "snn_internal.cuh"
 
 namespace snn {
-cudaError_t step_max_blocks(int npt, bool smem_ring, bool few, size_t smem, int* blocks_per_sm);
+cudaError_t step_max_blocks(int npt, bool smem_ring, bool few, int threads, size_t smem, int* blocks_per_sm);
 }
 
 using namespace snn;
@@ -259,10 +259,11 @@ int plan(snn_net* net, const snn_options* opt) {
     int P = opt ? opt->n_part : 0;
     // A step of a small network waits on L2 round trips and barriers; with
     // fewer neurons per CTA those come sooner, until reading more partitions'
-    // messages costs as much: us per step at scale 0.05 with 8 / 24 partitions
-    // 1.71 / 1.58, at 0.1 with 16 / 48 1.74 / 1.63, at 0.2 with 31 / 64 1.82 /
-    // 1.69; at 0.37 with 57 / 76 / 152 1.87 / 1.93 / 2.08.  The adjoint keeps
-    // partitions of 512 neurons (adj_part): its sums go over them.
+    // messages costs as much: us per step at scale 0.05 with 8 / 25 partitions
+    // 1.62 / 1.49, at 0.1 with 16 / 49 1.67 / 1.51, at 0.2 with 31 / 64 1.74 /
+    // 1.53, at 0.35 with 53 / 64 1.89 / 1.89; at 0.37 with 57 / 76 / 152 1.87 /
+    // 1.93 / 2.08.  The adjoint keeps partitions of 512 neurons (adj_part): its
+    // sums go over them.
     const int need = std::max(1, (net->n + 511) / 512);
     net->adj_part = P > 0 ? P : std::min(sms, need);
     if (P <= 0) P = std::min(sms, std::max(need, std::min(64, (net->n + 159) / 160)));
@@ -290,9 +291,11 @@ int plan(snn_net* net, const snn_options* opt) {
     const size_t with_ring = step_shared_bytes(ncmax, P, net->w_span, true);
     net->smem_ring = with_ring <= (size_t)smem_max;
     net->smem = step_shared_bytes(ncmax, P, net->w_span, net->smem_ring);
-    CK(step_kernel_configure(npt, net->smem_ring, P <= kFewPartsLimit));
+    const bool few = P <= kFewPartsLimit;
+    net->threads = few && net->smem_ring ? step_threads(ncmax) : kStepThreads;
+    CK(step_kernel_configure(npt, net->smem_ring, few, net->threads));
     int per_sm = 0;
-    CK(step_max_blocks(npt, net->smem_ring, P <= kFewPartsLimit, net->smem, &per_sm));
+    CK(step_max_blocks(npt, net->smem_ring, few, net->threads, net->smem, &per_sm));
     if (per_sm * sms < P)
         return fail(SNN_ERR_UNSUPPORTED, "partitions exceed co-resident CTAs of the step kernel");
     const double tmo = (opt && opt->timeout_s > 0) ? opt->timeout_s : 2.0;
@@ -696,7 +699,7 @@ cudaError_t net_launch(snn_net* net, StepParams& sp, int64_t t0, int64_t n) {
         sp.t0 = t;
         sp.n_steps = (int32_t)chunk;
         cudaError_t e = cudaMemsetAsync(net->d_sync + 5, 0, sizeof(uint32_t), net->stream);
-        if (e == cudaSuccess) e = launch_step(sp, net->npt, net->smem_ring, net->smem, net->stream);
+        if (e == cudaSuccess) e = launch_step(sp, net->npt, net->smem_ring, net->threads, net->smem, net->stream);
         if (e != cudaSuccess) return e;
         t += chunk;
         left -= chunk;
@@ -1027,7 +1030,7 @@ int snn_get_info(snn_net* net, snn_info* info) {
     info->n_neurons = net->n;
     info->n_synapses = (int64_t)net->nnz;
     info->n_part = net->P;
-    info->threads = kStepThreads;
+    info->threads = net->threads;
     info->neurons_per_thread = net->npt;
     info->ring_in_shared = net->smem_ring ? 1 : 0;
     info->max_part_neurons = net->ncmax;

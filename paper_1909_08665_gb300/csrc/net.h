@@ -20,6 +20,7 @@ struct snn_net {
     cudaStream_t stream;
     int device = 0;                        // the one that was current when it was made
     int n, n_pop, P, ncmax, npt;
+    int threads = 0;                       // of a CTA of the step kernel
     bool smem_ring;
     int adj_part = 1;                      // partitions of the partition-local adjoint
     size_t smem;

@@ -13,6 +13,17 @@ constexpr int kDCodes = 256;
 constexpr int kPoisTable = 32;
 constexpr int kRing = 64;                 // delay slots (delays 1..63)
 constexpr int kStepThreads = 512;         // threads per CTA of the step kernel
+// With few partitions (kFewPartsLimit) of few neurons a CTA has fewer threads,
+// as many as it has neurons or a little more, and registers and shared memory
+// let two or three of them share an SM: several such networks, on streams of
+// their own, run beside one another as they do with fewer and larger partitions.
+// us per step of the 10 % network with 512 / 192 threads: alone 1.57 / 1.51, all
+// of 6 networks 3.16 / 1.62, of 9 4.83 / 1.86 (16 partitions of 512 neurons:
+// 1.67, 1.71, 1.74); 20 % with 512 / 256: alone 1.65 / 1.53, 4 networks 3.5 /
+// 1.82; 25 % with 512 / 352: alone 1.67 / 1.64, 4 networks 3.69 / 2.09.  Above
+// 352 neurons the ring slices of two CTAs do not fit an SM.
+constexpr int step_threads(int ncmax) { return ncmax <= 192 ? 192 : ncmax <= 256 ? 256 : ncmax <= 352 ? 352 : kStepThreads; }
+constexpr int step_per_sm(int threads) { return threads == 192 ? 3 : threads <= 352 ? 2 : 1; }
 constexpr int kChunk = 1024;              // spikes per delivery chunk
 constexpr int kBuildThreads = 256;        // threads per CTA of the build kernels
 constexpr uint32_t kTgtBits = 19;
@@ -357,15 +368,15 @@ cudaError_t launch_ring_layout(const int32_t* part_lo, int n_part, int ncmax, in
                                int32_t* abi, bool to_abi, cudaStream_t s);
 cudaError_t launch_init_state(int n, uint32_t key0, uint32_t key1, float lo, float hi,
                               float* u, cudaStream_t s);
-int step_kernel_variant(int npt, bool smem_ring, bool few);
+int step_kernel_variant(int npt, bool smem_ring, bool few, int threads);
 constexpr int kFewPartsLimit = 64;   // kFewParts of the step kernel
 size_t step_shared_bytes(int ncmax, int n_part, int w_span, bool smem_ring);
 // target populations spanned by the widest of the partitions [part_lo[c],
 // part_lo[c+1]) (the rows of the weight table a CTA of the step kernel keeps)
 int partition_pop_span(const int32_t* part_lo, int n_part, const int32_t* pop_start, int n_pop);
 // few: at most kFewParts partitions
-cudaError_t step_kernel_configure(int npt, bool smem_ring, bool few);
-cudaError_t launch_step(const StepParams& sp, int npt, bool smem_ring, size_t smem,
+cudaError_t step_kernel_configure(int npt, bool smem_ring, bool few, int threads);
+cudaError_t launch_step(const StepParams& sp, int npt, bool smem_ring, int threads, size_t smem,
                         cudaStream_t s);
 cudaError_t launch_deliver(const DeliverParams& dp, int tiling, cudaStream_t s);
 // stand-alone delivery of the exact row segments of each partition (one CTA

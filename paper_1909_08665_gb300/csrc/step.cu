@@ -65,23 +65,23 @@ size_t step_shared_bytes(int ncmax, int n_part, int w_span, bool smem_ring) {
     return smem_layout(ncmax, n_part, w_span, smem_ring).total;
 }
 
-static const void* select_step(int npt, bool smem_ring, bool few, int mode) {
+static const void* select_step(int npt, bool smem_ring, bool few, int threads, int mode) {
     switch (mode) {
-        case 0: return step_fn_mode<0>(npt, smem_ring, few);
-        case kModePaced: return step_fn_mode<kModePaced>(npt, smem_ring, few);
-        case kModeSat: return step_fn_mode<kModeSat>(npt, smem_ring, few);
-        case kModeSat | kModePaced: return step_fn_mode<kModeSat | kModePaced>(npt, smem_ring, few);
+        case 0: return step_fn_mode<0>(npt, smem_ring, few, threads);
+        case kModePaced: return step_fn_mode<kModePaced>(npt, smem_ring, few, threads);
+        case kModeSat: return step_fn_mode<kModeSat>(npt, smem_ring, few, threads);
+        case kModeSat | kModePaced: return step_fn_mode<kModeSat | kModePaced>(npt, smem_ring, few, threads);
         default: return nullptr;
     }
 }
 
-int step_kernel_variant(int npt, bool smem_ring, bool few) {
-    return select_step(npt, smem_ring, few, 0) != nullptr;
+int step_kernel_variant(int npt, bool smem_ring, bool few, int threads) {
+    return select_step(npt, smem_ring, few, threads, 0) != nullptr;
 }
 
-cudaError_t step_kernel_configure(int npt, bool smem_ring, bool few) {
+cudaError_t step_kernel_configure(int npt, bool smem_ring, bool few, int threads) {
     for (int mode = 0; mode < 4; ++mode) {
-        const void* fn = select_step(npt, smem_ring, few, mode);
+        const void* fn = select_step(npt, smem_ring, few, threads, mode);
         if (!fn) return cudaErrorInvalidValue;
         const cudaError_t e = allow_shared(fn);
         if (e != cudaSuccess) return e;
@@ -90,13 +90,13 @@ cudaError_t step_kernel_configure(int npt, bool smem_ring, bool few) {
 }
 
 // co-resident CTAs per SM: the smallest of the variants' figures
-cudaError_t step_max_blocks(int npt, bool smem_ring, bool few, size_t smem, int* blocks_per_sm) {
+cudaError_t step_max_blocks(int npt, bool smem_ring, bool few, int threads, size_t smem, int* blocks_per_sm) {
     int best = 1 << 30;
     for (int mode = 0; mode < 4; ++mode) {
-        const void* fn = select_step(npt, smem_ring, few, mode);
+        const void* fn = select_step(npt, smem_ring, few, threads, mode);
         if (!fn) return cudaErrorInvalidValue;
         int b = 0;
-        const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, fn, kStepThreads, smem);
+        const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, fn, threads, smem);
         if (e != cudaSuccess) return e;
         best = std::min(best, b);
     }
@@ -104,13 +104,13 @@ cudaError_t step_max_blocks(int npt, bool smem_ring, bool few, size_t smem, int*
     return cudaSuccess;
 }
 
-cudaError_t launch_step(const StepParams& sp, int npt, bool smem_ring, size_t smem,
+cudaError_t launch_step(const StepParams& sp, int npt, bool smem_ring, int threads, size_t smem,
                         cudaStream_t s) {
     const int mode = (sp.rt_period_ns != 0ull ? kModePaced : 0) | (sp.wrap != nullptr ? kModeSat : 0);
-    const void* fn = select_step(npt, smem_ring, sp.n_part <= kFewParts, mode);
+    const void* fn = select_step(npt, smem_ring, sp.n_part <= kFewParts, threads, mode);
     if (!fn) return cudaErrorInvalidValue;
     void* args[] = {const_cast<StepParams*>(&sp)};
-    return cudaLaunchCooperativeKernel(fn, dim3(sp.n_part), dim3(kStepThreads), args, smem, s);
+    return cudaLaunchCooperativeKernel(fn, dim3(sp.n_part), dim3(threads), args, smem, s);
 }
 
 // Partition tiling of the stand-alone delivery: CTA c takes every spike of
@@ -152,7 +152,7 @@ k_deliver_part(const __grid_constant__ StepParams sp, const uint32_t* __restrict
             s_rl[k] = __ldg(sg + 1) - b;
         }
         __syncthreads();
-        deliver_batches<false>(
+        deliver_batches<false, kStepThreads>(
             sp, s_rb, s_rl, s_w, wbase, (uint32_t)m, t, ring, nullptr, events, nullptr);
         __syncthreads();
     }

@@ -55,7 +55,6 @@
 
 namespace snn {
 
-constexpr int kWarps = kStepThreads / 32;
 constexpr uint32_t kStatusRasterOverflow = 2u;
 // Ids read together with a message header: INL = 7 (64 bytes), or 3 (32 bytes)
 // where there are few partitions (kFewParts) and hardly ever more spikes in
@@ -119,8 +118,9 @@ __device__ __forceinline__ uint32_t warp_incl_scan(uint32_t x) {
     return x;
 }
 
-template <int ITEMS>
+template <int ITEMS, int T>
 __device__ __forceinline__ uint32_t block_scan(uint32_t (&v)[ITEMS], uint32_t* s_warp) {
+    constexpr int kWarps = T / 32;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     uint32_t local = 0;
 #pragma unroll
@@ -204,12 +204,13 @@ __device__ __forceinline__ void add_entry(uint32_t x, const int32_t* s_w, uint32
 
 // s_cnt (non-null while per-step counts are recorded): the list's synaptic
 // events and its non-empty runs are added into s_cnt[0], s_cnt[1]
-template <bool SAT>
+template <bool SAT, int T>
 __device__ __forceinline__ void deliver_batches(const StepParams& sp, const uint32_t* s_rb,
                                                 const uint32_t* s_rl, const int32_t* s_w,
                                                 uint32_t wbase, uint32_t m, int64_t tb,
                                                 int32_t* ring, int32_t* wrap,
                                                 unsigned long long& events, uint32_t* s_cnt) {
+    constexpr int kWarps = T / 32;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int32_t R = kRing * sp.ncmax;                  // ring words of this CTA
     const int32_t base_t = (int32_t)(((uint32_t)tb & (kRing - 1)) * (uint32_t)sp.ncmax);
@@ -335,7 +336,7 @@ __device__ __forceinline__ void early_runs(const StepParams& sp, int c, const ul
 // delivery of the spikes of step tb (message tag tb+1) into this CTA's ring;
 // returns false if a wait timed out or another CTA aborted
 // ---------------------------------------------------------------------------
-template <bool SAT, int INL>
+template <bool SAT, int INL, int T>
 __device__ __forceinline__ bool deliver_list(const StepParams& sp, unsigned char* smem,
                                              const SmemLayout& L, int c, uint32_t wbase,
                                              int64_t tb, int par, int32_t* ring, int32_t* wrap,
@@ -464,14 +465,14 @@ __device__ __forceinline__ bool deliver_list(const StepParams& sp, unsigned char
     const uint32_t S_fast = *s_list;
     if (s_misc[2]) return false;
     if (S_fast <= (uint32_t)kChunk) {
-        deliver_batches<SAT>(sp, s_rb, s_rl, s_w, wbase, S_fast, tb, ring, wrap, events,
+        deliver_batches<SAT, T>(sp, s_rb, s_rl, s_w, wbase, S_fast, tb, ring, wrap, events,
                                           s_cnt);
         __syncthreads();
         flush_counts(S_fast);
         return s_misc[2] == 0u;
     }
     // 2b. more than kChunk spikes: offsets by a block-wide scan, in chunks
-    const uint32_t S = block_scan<1>(cnt, s_warp);   // cnt[0] <- my offset
+    const uint32_t S = block_scan<1, T>(cnt, s_warp);   // cnt[0] <- my offset
     const uint32_t my_off = cnt[0];
 
     for (uint32_t base = 0; base < S; base += kChunk) {
@@ -500,7 +501,7 @@ __device__ __forceinline__ bool deliver_list(const StepParams& sp, unsigned char
             }
         }
         __syncthreads();
-        deliver_batches<SAT>(sp, s_rb, s_rl, s_w, wbase, m, tb, ring, wrap, events,
+        deliver_batches<SAT, T>(sp, s_rb, s_rl, s_w, wbase, m, tb, ring, wrap, events,
                                           s_cnt);
         __syncthreads();
     }
@@ -536,7 +537,6 @@ constexpr int kModeSat = 2;
 
 // local ids of a step's spikes kept in shared memory for the raster (MULTI)
 constexpr int kRecFew = 24;
-constexpr int kPublisher = kStepThreads - 32;   // first thread of the warp that publishes a step's count
 // barrier `id` of the CTA: arrive without waiting, or wait for all n threads
 __device__ __forceinline__ void barrier_arrive(int id, int n) {
     asm volatile("barrier.cta.arrive %0, %1;" ::"r"(id), "r"(n) : "memory");
@@ -545,12 +545,13 @@ __device__ __forceinline__ void barrier_wait(int id, int n) {
     asm volatile("barrier.cta.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
 }
 
-// One CTA's steps: partition c of the network sp describes.  MULTI: one of
+// One CTA's steps, of T threads: partition c of the network sp describes.  MULTI: one of
 // several networks of the launch, whose spikes go to one list (sp.ras_n[0]
 // counts them) with their ids offset.
-template <int NPT, bool SMEM_RING, int MODE, int INL, bool MULTI>
+template <int NPT, bool SMEM_RING, int MODE, int INL, bool MULTI, int T>
 __device__ __forceinline__ void step_body(const StepParams& sp, const int c, unsigned char* smem) {
     constexpr int kHead = (INL + 1) / 2;
+    constexpr int kPublisher = T - 32;               // first thread of the warp that publishes a step's count
     constexpr bool PACED = (MODE & kModePaced) != 0;
     constexpr bool SAT = (MODE & kModeSat) != 0;
     // early run lookups keep 2 x INL more registers live until the delivery:
@@ -578,15 +579,15 @@ __device__ __forceinline__ void step_body(const StepParams& sp, const int c, uns
     int32_t* wrap = SAT ? sp.wrap + (size_t)c * kRing * (size_t)sp.ncmax : nullptr;
     bool saturated = false;
 
-    for (int k = tid; k < kMaxPop * kPoisTable; k += kStepThreads)
+    for (int k = tid; k < kMaxPop * kPoisTable; k += T)
         s_pois[k] = sp.pois_m1[k / kPoisTable][k % kPoisTable];
     // weight-table rows of the target populations of this partition: those
     // from the population of its first neuron on (at most w_span of them)
     const uint32_t wt_base = (uint32_t)pop_index(sp.pop_start, sp.n_pop, lo) * kPopWords;
-    for (uint32_t k = tid; k < (uint32_t)sp.w_span * kPopWords; k += kStepThreads)
+    for (uint32_t k = tid; k < (uint32_t)sp.w_span * kPopWords; k += T)
         s_w[k] = wt_base + k < (uint32_t)(kMaxPop * kPopWords) ? __ldg(&sp.wtab[wt_base + k]) : 0;
     if (SMEM_RING)
-        for (int k = tid; k < kRing * sp.ncmax; k += kStepThreads) ring[k] = ring_g[k];
+        for (int k = tid; k < kRing * sp.ncmax; k += T) ring[k] = ring_g[k];
     if (tid < 32) s_misc[tid] = 0u;
     // pacing to wall-clock time: the first CTA to arrive fixes the anchor of
     // the paced run (the device clock at which step rt_t_anchor starts) in
@@ -606,7 +607,7 @@ __device__ __forceinline__ void step_body(const StepParams& sp, const int c, uns
     uint32_t pf_row_n[NPF], pf_seg_n[NPF];
 #pragma unroll
     for (int k = 0; k < NPT; ++k) {
-        const int li = tid + k * kStepThreads;
+        const int li = tid + k * T;
         u[k] = 0.f; isyn[k] = 0.f; refr[k] = 0; pop[k] = 0; pacc[k] = 0;
         rnd[k] = make_uint4(0u, 0u, 0u, 0u);
         if (k < NPF) { pf_row[k] = pf_seg[k] = 0ull; pf_row_n[k] = pf_seg_n[k] = 0u; }
@@ -650,7 +651,7 @@ __device__ __forceinline__ void step_body(const StepParams& sp, const int c, uns
         // ---- A(t): membrane, threshold, compaction, publication ----
 #pragma unroll
         for (int k = 0; k < NPT; ++k) {
-            const int li = tid + k * kStepThreads;
+            const int li = tid + k * T;
             bool spk = false;
             if (li < nc) {
                 uint8_t upd = 0;
@@ -744,9 +745,9 @@ __device__ __forceinline__ void step_body(const StepParams& sp, const int c, uns
         // publishes the count; the others only arrive and go on
         if (PUB_EARLY) {
             if (tid < kPublisher) {
-                barrier_arrive(1, kStepThreads);
+                barrier_arrive(1, T);
             } else {
-                barrier_wait(1, kStepThreads);
+                barrier_wait(1, T);
                 if (tid == kPublisher) publish();
             }
         }
@@ -763,7 +764,7 @@ __device__ __forceinline__ void step_body(const StepParams& sp, const int c, uns
         if (NPT > 1 && look_up) early_runs(sp, c, pre, (uint32_t)t, early);
 #pragma unroll
         for (int k = 0; k < NPT; ++k) {
-            const int li = tid + k * kStepThreads;
+            const int li = tid + k * T;
             // background count of step t (independent of the network): drawn
             // here, added to the ring input in C(t)
             if (sp.mode == 0 && li < nc) {
@@ -792,7 +793,7 @@ __device__ __forceinline__ void step_body(const StepParams& sp, const int c, uns
         }
         // ---- D: spikes of step t-1 ----
         if (s > 0) {
-            if (!deliver_list<SAT, INL>(
+            if (!deliver_list<SAT, INL, T>(
                     sp, smem, L, c, wt_base, t - 1, s & 1, ring, wrap, events, pre, early)) {
                 record();                        // the list has no gaps
                 aborted = true;
@@ -810,12 +811,12 @@ __device__ __forceinline__ void step_body(const StepParams& sp, const int c, uns
         int32_t cells[NPT];
 #pragma unroll
         for (int k = 0; k < NPT; ++k) {
-            const int li = tid + k * kStepThreads;
+            const int li = tid + k * T;
             if (NPT > 1) cells[k] = li < nc ? ring[slot * (uint32_t)sp.ncmax + (uint32_t)li] : 0;
         }
 #pragma unroll
         for (int k = 0; k < NPT; ++k) {
-            const int li = tid + k * kStepThreads;
+            const int li = tid + k * T;
             if (li < nc) {
                 const uint32_t cell = slot * (uint32_t)sp.ncmax + (uint32_t)li;
                 const int32_t r = NPT > 1 ? cells[k] : ring[cell];
@@ -866,13 +867,13 @@ __device__ __forceinline__ void step_body(const StepParams& sp, const int c, uns
         }
         EarlyRuns<INL> none;
         none.ok = false;
-        deliver_list<SAT, INL>(
+        deliver_list<SAT, INL, T>(
             sp, smem, L, c, wt_base, tl, sp.n_steps & 1, ring, wrap, events, pre, none);
     }
     __syncthreads();
 #pragma unroll
     for (int k = 0; k < NPT; ++k) {
-        const int li = tid + k * kStepThreads;
+        const int li = tid + k * T;
         if (li < nc) {
             sp.u[lo + li] = u[k];
             sp.i_syn[lo + li] = isyn[k];
@@ -880,7 +881,7 @@ __device__ __forceinline__ void step_body(const StepParams& sp, const int c, uns
         }
     }
     if (SMEM_RING)
-        for (int k = tid; k < kRing * sp.ncmax; k += kStepThreads) ring_g[k] = ring[k];
+        for (int k = tid; k < kRing * sp.ncmax; k += T) ring_g[k] = ring[k];
     if (tid == kPublisher) {
         if (!MULTI) sp.ras_n[c] = ras_base;
         atomicAdd(&sp.counters[0], spikes);
@@ -889,18 +890,27 @@ __device__ __forceinline__ void step_body(const StepParams& sp, const int c, uns
     if (lane == 0 && events) atomicAdd(&sp.counters[1], events);   // per-warp counts
 }
 
-template <int NPT, bool SMEM_RING, int MODE, int INL = kInline>
-__global__ void __launch_bounds__(kStepThreads, 1)
+template <int NPT, bool SMEM_RING, int MODE, int INL = kInline, int T = kStepThreads>
+__global__ void __launch_bounds__(T, step_per_sm(T))
 k_step(const __grid_constant__ StepParams sp) {
     extern __shared__ __align__(16) unsigned char smem[];
-    step_body<NPT, SMEM_RING, MODE, INL, false>(sp, (int)blockIdx.x, smem);
+    step_body<NPT, SMEM_RING, MODE, INL, false, T>(sp, (int)blockIdx.x, smem);
 }
 
 // the kernel of one MODE for a launch shape (neurons per thread, ring in
-// shared memory or not, at most kFewParts partitions); nullptr for an unknown
-// shape
+// shared memory or not, at most kFewParts partitions, threads of
+// step_threads); nullptr for an unknown shape
 template <int MODE>
-const void* step_fn_mode(int npt, bool smem_ring, bool few) {
+const void* step_fn_mode(int npt, bool smem_ring, bool few, int threads) {
+    if (threads != kStepThreads) {
+        if (!few || npt != 1 || !smem_ring) return nullptr;
+        switch (threads) {
+            case 192: return reinterpret_cast<const void*>(&k_step<1, true, MODE, kInlineFew, 192>);
+            case 256: return reinterpret_cast<const void*>(&k_step<1, true, MODE, kInlineFew, 256>);
+            case 352: return reinterpret_cast<const void*>(&k_step<1, true, MODE, kInlineFew, 352>);
+            default: return nullptr;
+        }
+    }
     if (few && npt == 1 && smem_ring) return reinterpret_cast<const void*>(&k_step<1, true, MODE, kInlineFew>);
     switch (npt) {
         case 1: return smem_ring ? reinterpret_cast<const void*>(&k_step<1, true, MODE>)
@@ -914,9 +924,9 @@ const void* step_fn_mode(int npt, bool smem_ring, bool few) {
         default: return nullptr;
     }
 }
-extern template const void* step_fn_mode<0>(int, bool, bool);
-extern template const void* step_fn_mode<kModePaced>(int, bool, bool);
-extern template const void* step_fn_mode<kModeSat>(int, bool, bool);
-extern template const void* step_fn_mode<kModeSat | kModePaced>(int, bool, bool);
+extern template const void* step_fn_mode<0>(int, bool, bool, int);
+extern template const void* step_fn_mode<kModePaced>(int, bool, bool, int);
+extern template const void* step_fn_mode<kModeSat>(int, bool, bool, int);
+extern template const void* step_fn_mode<kModeSat | kModePaced>(int, bool, bool, int);
 
 }  // namespace snn

@@ -5,5 +5,5 @@
 #include "step_kernel.cuh"
 
 namespace snn {
-template const void* step_fn_mode<kModePaced>(int, bool, bool);
+template const void* step_fn_mode<kModePaced>(int, bool, bool, int);
 }  // namespace snn

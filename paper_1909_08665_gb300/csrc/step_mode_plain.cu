@@ -4,5 +4,5 @@
 #include "step_kernel.cuh"
 
 namespace snn {
-template const void* step_fn_mode<0>(int, bool, bool);
+template const void* step_fn_mode<0>(int, bool, bool, int);
 }  // namespace snn

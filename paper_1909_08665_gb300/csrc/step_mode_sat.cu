@@ -6,5 +6,5 @@
 #include "step_kernel.cuh"
 
 namespace snn {
-template const void* step_fn_mode<kModeSat>(int, bool, bool);
+template const void* step_fn_mode<kModeSat>(int, bool, bool, int);
 }  // namespace snn

@@ -34,7 +34,7 @@ k_step_multi(const StepParams* __restrict__ params, const int32_t* __restrict__ 
         s_sp.n_steps = n_steps;
     }
     __syncthreads();
-    step_body<NPT, SMEM_RING, 0, INL, true>(s_sp, (int)blockIdx.x - __ldg(&first[a]), smem);
+    step_body<NPT, SMEM_RING, 0, INL, true, kStepThreads>(s_sp, (int)blockIdx.x - __ldg(&first[a]), smem);
 }
 
 // after the launch, when every CTA has read it
