@@ -322,7 +322,8 @@ int snn_deliver(snn_net* net, const uint32_t* spikes_dev, int32_t n_spikes, int6
  *   cfg, seed  model parameters and Philox key, as for snn_create; the
  *              network's row_ptr / words / wtab must be the ones exported
  *              by snn_export_network for the same cfg (any rows in that
- *              format are accepted).
+ *              format are accepted: targets ascending within a row, which a
+ *              call cannot check; words out of order may be left out).
  *   io         device pointers, all required:
  *                row_ptr[n+1] (uint64), words[nnz], wtab[8*8*128]   input
  *                u[n], i_syn[n], refr[n], ring[64*n] slot-major     in/out
@@ -330,7 +331,8 @@ int snn_deliver(snn_net* net, const uint32_t* spikes_dev, int32_t n_spikes, int6
  *                ras_n: spikes recorded; the kernel appends at *ras_n
  *                  and counts past ras_cap (caller zeroes it)     in/out
  *                counters[2]: spikes and synaptic events, added to  in/out
- *                status: ORed with 1 if a grid-barrier wait gave up in/out
+ *                status: ORed with 1 if a wait for the other blocks'
+ *                  spikes gave up                                 in/out
  *   t0         index of the first step (it selects the ring slots and the
  *              background draws, so consecutive calls continue a run).
  * Asynchronous on `stream`.  Results equal snn_step on the same network.

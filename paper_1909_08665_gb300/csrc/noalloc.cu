@@ -24,8 +24,8 @@
 // between the two probes that enclose the run and tests each word's target;
 // the probes touched most of those sectors already.  It walks on in either
 // direction where the outermost probe does not prove the run complete, so any
-// rows give the right result, and rows like the network's own cost one L2
-// round trip.  What bounds a step is that trip, the message's and the run's,
+// rows of ascending targets give the right result, and rows like the network's
+// own cost one L2 round trip.  What bounds a step is that trip, the message's and the run's,
 // and in large networks the SM's own intake: a probe costs a 32-byte sector,
 // 1 KB per (spike, partition).  Measured, us per step at full size: 64 probes
 // over the whole row 6.07; every word of the window loaded and tested 6.34;
@@ -66,8 +66,7 @@ constexpr int kNaPart = 512;            // most partitions, and the neurons of o
 constexpr int kNaMaxDevices = 64;
 constexpr int kNaChunk = 384;           // spikes listed at once
 constexpr int kNaInline = 3;            // spikes read together with a message header (64 B)
-constexpr int kNaSpikes = 1;            // rows a warp probes and loads together
-constexpr int kNaWave = 2;              // words of each per lane before the first add
+constexpr int kNaWave = 2;              // words of a row per lane before the first add
 constexpr uint32_t kNaProbes = 32;      // probes of a window, one per lane
 // half width of the window over the expected run, in standard deviations: one
 // (spike, partition) pair in 4e4 has to walk on, about one step in 6 at full
@@ -230,76 +229,52 @@ __device__ __forceinline__ void na_deliver(const NaParams& p, const NaList& list
         na_add<SMEM_RING>(ring, ring_s, slot * stride + l, wq[s_popo[l] + (word >> 25)], ok);
     };
     constexpr uint32_t kOut = kTgtMask;              // no neuron has this index
-    for (uint32_t g = warp; g < m; g += kNaWarps * kNaSpikes) {
-        // The list is read again in every phase rather than held over the
-        // loads: registers set how many rows a warp has in flight.  The
-        // branches on the list and on lengths are the same for all lanes.
-        uint32_t probe[kNaSpikes];
+    static_assert(kNaProbes == 32u, "one probe per lane");
+    for (uint32_t i = warp; i < m; i += kNaWarps) {
+        // (the branches on the list and on lengths are the same for all lanes)
+        const uint32_t n = list.w[i], gap = na_gap(n);
+        const uint32_t* row = p.words + list.rs[i];  // the window's first word
+        uint32_t probe = kOut;
+        if (lane * gap < n) probe = __ldg(row + lane * gap) & kTgtMask;
+        const uint32_t nl = __popc(__ballot_sync(0xffffffffu, probe < lo));
+        const uint32_t nh = __popc(__ballot_sync(0xffffffffu, probe < hi));
+        // after the last probe below lo; before the first one past hi (a lane
+        // without a probe counts as past, its place is past n)
+        const uint32_t c0 = nl ? (nl - 1u) * gap + 1u : 0u;
+        const uint32_t c1 = min(nh * gap, n);
+        uint32_t e[kNaWave];
 #pragma unroll
-        for (int k = 0; k < kNaSpikes; ++k) {
-            const uint32_t i = g + (uint32_t)k * kNaWarps;
-            probe[k] = kOut;
-            if (i < m) {
-                const uint32_t n = list.w[i], x = lane * na_gap(n);
-                if (lane < kNaProbes && x < n) probe[k] = __ldg(p.words + list.rs[i] + x) & kTgtMask;
-            }
+        for (int h = 0; h < kNaWave; ++h) {
+            const uint32_t x = c0 + lane + 32u * (uint32_t)h;
+            e[h] = kOut;
+            if (x < c1) e[h] = __ldg(row + x);
         }
-        uint32_t e[kNaSpikes][kNaWave], c0[kNaSpikes], c1[kNaSpikes];
+        const int32_t* wq = s_w + (uint32_t)list.q[i] * kWCodes;
+        add(e[0], wq);
 #pragma unroll
-        for (int k = 0; k < kNaSpikes; ++k) {
-            const uint32_t i = g + (uint32_t)k * kNaWarps;
-            c0[k] = c1[k] = 0u;
-            if (i < m) {
-                const uint32_t n = list.w[i], gap = na_gap(n);
-                const uint32_t nl = __popc(__ballot_sync(0xffffffffu, probe[k] < lo));
-                const uint32_t nh = __popc(__ballot_sync(0xffffffffu, probe[k] < hi));
-                // after the last probe below lo; before the first one past hi
-                // (a lane without a probe counts as past, its place is past n)
-                c0[k] = nl ? (nl - 1u) * gap + 1u : 0u;
-                c1[k] = min(nh * gap, n);
+        for (int h = 1; h < kNaWave; ++h)
+            if (c0 + 32u * (uint32_t)h < c1) add(e[h], wq);
+        for (uint32_t x = c0 + 32u * kNaWave; x < c1; x += 32u)
+            add(x + lane < c1 ? __ldg(row + x + lane) : kOut, wq);
+        const bool low = c0 == 0u, high = c1 == n;
+        if (low || high) {
+            const uint32_t a = list.a[i], len = list.len[i];
+            const uint32_t* r = row - a;             // the row's first word
+            // no probe below the partition: 32 words at a time towards the
+            // row's start, until one lies below it
+            for (uint32_t end = low ? a : 0u; end > 0u;) {
+                const uint32_t from = end > 32u ? end - 32u : 0u, x = from + lane;
+                const uint32_t word = x < end ? __ldg(r + x) : kOut;
+                add(word, wq);
+                end = from;
+                if (__any_sync(0xffffffffu, (word & kTgtMask) < lo)) break;
             }
-            const uint32_t* row = p.words + (i < m ? list.rs[i] : 0ull);
-#pragma unroll
-            for (int h = 0; h < kNaWave; ++h) {
-                const uint32_t x = c0[k] + lane + 32u * (uint32_t)h;
-                e[k][h] = kOut;
-                if (x < c1[k]) e[k][h] = __ldg(row + x);
-            }
-        }
-#pragma unroll
-        for (int k = 0; k < kNaSpikes; ++k) {
-            const uint32_t i = g + (uint32_t)k * kNaWarps;
-            if (i < m) {
-                const int32_t* wq = s_w + (uint32_t)list.q[i] * kWCodes;
-                const uint32_t* row = p.words + list.rs[i];   // the window's first word
-                add(e[k][0], wq);
-#pragma unroll
-                for (int h = 1; h < kNaWave; ++h)
-                    if (c0[k] + 32u * (uint32_t)h < c1[k]) add(e[k][h], wq);
-                for (uint32_t x = c0[k] + 32u * kNaWave; x < c1[k]; x += 32u)
-                    add(x + lane < c1[k] ? __ldg(row + x + lane) : kOut, wq);
-                const uint32_t n = list.w[i];
-                const bool low = c0[k] == 0u, high = c1[k] == n;
-                if (low || high) {
-                    const uint32_t a = list.a[i], len = list.len[i];
-                    const uint32_t* r = row - a;     // the row's first word
-                    // no probe below the partition: 32 words at a time towards
-                    // the row's start, until one lies below it
-                    for (uint32_t end = low ? a : 0u; end > 0u;) {
-                        const uint32_t from = end > 32u ? end - 32u : 0u, x = from + lane;
-                        const uint32_t word = x < end ? __ldg(r + x) : kOut;
-                        add(word, wq);
-                        end = from;
-                        if (__any_sync(0xffffffffu, (word & kTgtMask) < lo)) break;
-                    }
-                    // no probe past it: on, until a word lies past it
-                    for (uint32_t from = high ? a + n : len; from < len; from += 32u) {
-                        const uint32_t x = from + lane;
-                        const uint32_t word = x < len ? __ldg(r + x) : 0u;
-                        add(x < len ? word : kOut, wq);
-                        if (__any_sync(0xffffffffu, (word & kTgtMask) >= hi)) break;
-                    }
-                }
+            // no probe past it: on, until a word lies past it
+            for (uint32_t from = high ? a + n : len; from < len; from += 32u) {
+                const uint32_t x = from + lane;
+                const uint32_t word = x < len ? __ldg(r + x) : 0u;
+                add(x < len ? word : kOut, wq);
+                if (__any_sync(0xffffffffu, (word & kTgtMask) >= hi)) break;
             }
         }
     }
@@ -614,10 +589,11 @@ __global__ void __launch_bounds__(THREADS, 1) k_step_noalloc(const __grid_consta
 }
 
 // one neuron per thread covers every network on the full GPU; eight take over
-// where fewer SMs are visible
+// where fewer SMs are visible.  The ring of the few threads' partitions always
+// fits in shared memory.
 template <bool SMEM_RING>
 const void* na_kernel(int threads, int ncmax) {
-    if (threads == kNaFewThreads) return reinterpret_cast<const void*>(&k_step_noalloc<kNaFewThreads, 1, SMEM_RING>);
+    if (threads == kNaFewThreads) return reinterpret_cast<const void*>(&k_step_noalloc<kNaFewThreads, 1, true>);
     if (ncmax <= kNaManyThreads) return reinterpret_cast<const void*>(&k_step_noalloc<kNaManyThreads, 1, SMEM_RING>);
     return reinterpret_cast<const void*>(&k_step_noalloc<kNaManyThreads, 8, SMEM_RING>);
 }
@@ -688,7 +664,7 @@ extern "C" int snn_step_noalloc(const snn_config* cfg, uint64_t seed, const snn_
     if (n > SNN_NOALLOC_MAX_NEURONS)
         return set_error(SNN_ERR_INVALID,
                          "snn_step_noalloc supports at most SNN_NOALLOC_MAX_NEURONS (131072) "
-                         "neurons: its static scratch holds two spike lists of that length");
+                         "neurons: its static scratch holds the spike messages of that many");
     NaParams p;
     std::memset(&p, 0, sizeof(p));
     float pr[4];
@@ -731,7 +707,7 @@ extern "C" int snn_step_noalloc(const snn_config* cfg, uint64_t seed, const snn_
     p.msg_stride = 8 + (ncmax + 7) / 8 * 8;
     const bool smem_ring = na_smem(ncmax, p.w_span, true).total <= (uint32_t)d.optin;
     const size_t smem = na_smem(ncmax, p.w_span, smem_ring).total;
-    const int threads = n > kNaWide || ncmax > kNaFewThreads ? kNaManyThreads : kNaFewThreads;
+    const int threads = n > kNaWide || ncmax > kNaFewThreads || !smem_ring ? kNaManyThreads : kNaFewThreads;
     const void* fn = na_kernel(threads, ncmax, smem_ring);
     if (ncmax > 8 * kNaManyThreads || smem > (size_t)d.optin) return set_error(SNN_ERR_UNSUPPORTED, "step kernel does not fit an SM");
     const size_t msg_words = (size_t)4 * P * p.msg_stride;
