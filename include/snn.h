@@ -96,11 +96,11 @@ typedef struct snn_options {
                                  SNN_ERR_TIMEOUT (tests of the failure path;
                                  every wait is bounded, nothing hangs) */
     int64_t raster_capacity;  /* spikes buffered on the device; 0 auto (64 Mi).
-                                 Of a network each partition holds its share;
-                                 where partitions are smaller than 512 neurons
-                                 (n_part 0, fewer than 32,768 neurons), the share
-                                 of one of 512, so that the memory is up to four
-                                 times 8 bytes per spike of the capacity */
+                                 Of a network each partition holds its share, 8
+                                 bytes per spike; where partitions are smaller
+                                 than 512 neurons (n_part 0, fewer than 32,768
+                                 neurons), the share of one of 512 while all of
+                                 them take at most 0.5 GiB */
     double timeout_s;         /* limit of one grid-barrier wait; 0 = 2 s */
 } snn_options;
 

@@ -300,11 +300,15 @@ int plan(snn_net* net, const snn_options* opt) {
         return fail(SNN_ERR_UNSUPPORTED, "partitions exceed co-resident CTAs of the step kernel");
     const double tmo = (opt && opt->timeout_s > 0) ? opt->timeout_s : 2.0;
     net->timeout_ns = (uint64_t)(tmo * 1e9);
-    const int64_t cap = (opt && opt->raster_capacity > 0) ? opt->raster_capacity : (64ll << 20);
+    constexpr int64_t kDefaultRaster = 64ll << 20;
+    const int64_t cap = (opt && opt->raster_capacity > 0) ? opt->raster_capacity : kDefaultRaster;
     // A partition's list is its share of the capacity.  Small partitions share
     // less evenly than large ones, so each gets the share of one of 512 neurons,
-    // whatever the capacity: a larger one never means a shorter list.
-    net->ras_cap = (uint32_t)std::min<int64_t>(std::max<int64_t>(cap / net->adj_part, 1), 0x7fffffff);
+    // as far as all lists take no more than the default's memory (1.5 GiB for
+    // every small network would make creating one a quarter longer).  A larger
+    // capacity never means a shorter list.
+    const int64_t list = std::min(cap / net->adj_part, std::max(cap, kDefaultRaster) / P);
+    net->ras_cap = (uint32_t)std::min<int64_t>(std::max<int64_t>(list, 1), 0x7fffffff);
     net->inject_fault = opt ? opt->inject_fault : 0;
     return SNN_OK;
 }

@@ -86,17 +86,18 @@ for cap in (0, 4 << 20, 65 << 20):
 
 def test_a_larger_raster_capacity_never_shortens_a_list(run):
     """A partition's list is the share of a partition of 512 neurons (of all
-    neurons in few), at every capacity and by default."""
+    neurons in few), until the lists take the default's memory."""
     run("""
 for scale in (0.005, 0.1, 0.3, 1.0):
     need = -(-workload.n_neurons(workload.microcircuit(scale)) // 512)
     last = 0
-    for cap in (1 << 20, 16 << 20, 0, 65 << 20, 200 << 20):
+    for cap in (1 << 20, 12 << 20, 40 << 20, 64 << 20, 0, 65 << 20, 200 << 20):
         rt.fake_clear()
         net = pkg.Microcircuit(workload.microcircuit(scale), stream=Stream(), raster_capacity=cap)
         sizes = [int(x.split()[-1]) for x in calls("malloc")]
-        entries = (cap or 64 << 20) // min(need, 152)
-        assert sizes.count(4 * entries * net.info()["n_part"]) == 2 and entries > last, (scale, cap, sorted(sizes)[-4:])
+        asked, parts = cap or 64 << 20, net.info()["n_part"]
+        entries = min(asked // min(need, 152), max(asked, 64 << 20) // parts)
+        assert sizes.count(4 * entries * parts) == 2 and entries >= max(last, asked // parts), (scale, cap, sorted(sizes)[-4:])
         last = entries
         net.close()
 """)
