@@ -234,6 +234,7 @@ int dalloc(T** p, size_t count, const char* what) {
     cudaError_t e = cudaMalloc(reinterpret_cast<void**>(p), std::max<size_t>(count, 1) * sizeof(T));
     if (e != cudaSuccess) {
         *p = nullptr;
+        cudaGetLastError();
         g_err = std::string("device allocation of ") + what + " failed: " + cudaGetErrorString(e);
         return SNN_ERR_OOM;
     }
@@ -768,11 +769,44 @@ int net_update_saturation(snn_net* net) {
     return SNN_OK;
 }
 
+namespace {
+
+// The ring copied without staging on the device, where that has no room: by
+// partitions, on the host.
+int ring_by_host(snn_net* net, int32_t* abi, bool to_abi) {
+    std::vector<int32_t> part;
+    try {
+        part.resize((size_t)kRing * net->ncmax);
+    } catch (const std::bad_alloc&) {
+        return fail(SNN_ERR_OOM, "ring copy: host memory");
+    }
+    for (int c = 0; c < net->P; ++c) {
+        const int lo = net->part_lo[c], nc = net->part_lo[c + 1] - lo;
+        int32_t* ring = net->d_ring + (size_t)c * part.size();
+        if (to_abi) {
+            CK(cudaMemcpyAsync(part.data(), ring, sizeof(int32_t) * part.size(), cudaMemcpyDeviceToHost, net->stream));
+            CK(cudaStreamSynchronize(net->stream));
+        }
+        for (int slot = 0; slot < kRing; ++slot) {
+            int32_t *p = part.data() + (size_t)slot * net->ncmax, *a = abi + (size_t)slot * net->n + lo;
+            if (to_abi) std::copy(p, p + nc, a);
+            else std::fill(std::copy(a, a + nc, p), p + net->ncmax, 0);
+        }
+        if (!to_abi) {
+            CK(cudaMemcpyAsync(ring, part.data(), sizeof(int32_t) * part.size(), cudaMemcpyHostToDevice, net->stream));
+            CK(cudaStreamSynchronize(net->stream));
+        }
+    }
+    return SNN_OK;
+}
+
+}  // namespace
+
 int net_ring_to_host(snn_net* net, int32_t* host) {
     const DeviceScope on(net->device);
     const size_t words = (size_t)kRing * net->n;
     std::lock_guard<std::mutex> hold(net->stage.mu);
-    if (!net->d_ring_io) CALL(dalloc(&net->d_ring_io, words, "ring staging"));
+    if (!net->d_ring_io && dalloc(&net->d_ring_io, words, "ring staging") != SNN_OK) return ring_by_host(net, host, true);
     CK(launch_ring_layout(net->d_part_lo, net->P, net->ncmax, net->n, net->d_ring, net->d_ring_io, true,
                           net->stream));
     CK(cudaMemcpyAsync(host, net->d_ring_io, sizeof(int32_t) * words, cudaMemcpyDeviceToHost, net->stream));
@@ -784,7 +818,8 @@ int net_ring_from_host(snn_net* net, const int32_t* host) {
     const DeviceScope on(net->device);
     const size_t words = (size_t)kRing * net->n;
     std::lock_guard<std::mutex> hold(net->stage.mu);
-    if (!net->d_ring_io) CALL(dalloc(&net->d_ring_io, words, "ring staging"));
+    if (!net->d_ring_io && dalloc(&net->d_ring_io, words, "ring staging") != SNN_OK)
+        return ring_by_host(net, const_cast<int32_t*>(host), false);
     CK(cudaMemcpyAsync(net->d_ring_io, host, sizeof(int32_t) * words, cudaMemcpyHostToDevice, net->stream));
     CK(launch_ring_layout(net->d_part_lo, net->P, net->ncmax, net->n, net->d_ring, net->d_ring_io, false,
                           net->stream));

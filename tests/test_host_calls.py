@@ -263,3 +263,23 @@ for kernel in ("k_deliver_part", "k_deliver_words", "k_deliver_cluster", "k_deli
     assert any(kernel in x[1] for x in limits), kernel
 assert {x[2] for x in limits} == {"232448"}, {(x[1], x[2]) for x in limits if x[2] != "232448"}
 """)
+
+
+def test_ring_copies_without_device_memory(run):
+    """Reading, saving and loading the ring where the device has no room for
+    its staging copy."""
+    run("""
+net = pkg.Microcircuit(workload.microcircuit(0.02), stream=Stream(), raster_capacity=1 << 16, n_part=7)
+most, n = net.info()["max_part_neurons"], net.n
+lo = np.arange(8) * n // 7
+ring = words(7 * 64 * most).view(np.int32).reshape(7, 64, most)
+want = np.random.default_rng(1).integers(-9, 9, (64, n)).astype(np.int32)
+for c in range(7):
+    ring[c, :, :lo[c + 1] - lo[c]] = want[:, lo[c]:lo[c + 1]]
+rt.fake_alloc_limit(1 << 12)
+assert (net.ring() == want).all()
+saved = net.save_state()
+ring[:] = -1
+net.load_state(saved)
+assert (net.ring() == want).all() and (ring[:, :, most - 1][np.diff(lo) < most] == 0).all()
+""")
