@@ -1093,15 +1093,9 @@ int drain_raster(snn_batch* b) {
     return small.lost ? set_error(SNN_ERR_OVERFLOW, "batch raster capacity exceeded") : SNN_OK;
 }
 
-}  // namespace
-
-extern "C" {
-
-int snn_batch_create(const snn_config* cfgs, const uint64_t* seeds, int32_t n_inst,
-                     const snn_options* opt, void* stream, snn_batch** out) {
-    if (!cfgs || !seeds || !out || n_inst < 1 || n_inst > kMaxInst)
-        return set_error(SNN_ERR_INVALID, "need 1..1024 configurations, seeds and out");
-    *out = nullptr;
+// side_by_side: in that form where the instances fit
+int create_batch(const snn_config* cfgs, const uint64_t* seeds, int32_t n_inst, const snn_options* opt,
+                 void* stream, bool side_by_side, snn_batch** out) {
     int dev = 0;
     BCK(cudaGetDevice(&dev));
     cudaDeviceProp prop;
@@ -1126,7 +1120,7 @@ int snn_batch_create(const snn_config* cfgs, const uint64_t* seeds, int32_t n_in
     int rc = SNN_OK;
     long long ntot = 0;
     std::vector<int> n_part;
-    const bool parts = plan_parts(cfgs, n_inst, prop.multiProcessorCount, &n_part);
+    const bool parts = side_by_side && plan_parts(cfgs, n_inst, prop.multiProcessorCount, &n_part);
     for (int k = 0; k < n_inst && rc == SNN_OK; ++k) {
         HostTables ht;
         rc = host_tables(&cfgs[k], &ht);
@@ -1338,6 +1332,21 @@ int snn_batch_create(const snn_config* cfgs, const uint64_t* seeds, int32_t n_in
     BCALL(capture_graph(b));
     *out = b;
     return SNN_OK;
+}
+
+}  // namespace
+
+extern "C" {
+
+int snn_batch_create(const snn_config* cfgs, const uint64_t* seeds, int32_t n_inst,
+                     const snn_options* opt, void* stream, snn_batch** out) {
+    if (!cfgs || !seeds || !out || n_inst < 1 || n_inst > kMaxInst)
+        return set_error(SNN_ERR_INVALID, "need 1..1024 configurations, seeds and out");
+    *out = nullptr;
+    // side by side the rows are held twice, packed and decoded: where there is
+    // no room for that the batch kernel takes all of it
+    const int rc = create_batch(cfgs, seeds, n_inst, opt, stream, true, out);
+    return rc == SNN_ERR_OOM ? create_batch(cfgs, seeds, n_inst, opt, stream, false, out) : rc;
 }
 
 int snn_batch_step(snn_batch* b, int64_t n_steps) {

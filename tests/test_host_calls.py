@@ -283,3 +283,18 @@ ring[:] = -1
 net.load_state(saved)
 assert (net.ring() == want).all() and (ring[:, :, most - 1][np.diff(lo) < most] == 0).all()
 """)
+
+
+def test_batches_that_have_no_room_side_by_side(run):
+    """The batch kernel takes a batch whose decoded rows do not fit."""
+    run("""
+cfgs = [workload.microcircuit(0.13)]
+kw = dict(stream=Stream(), raster_capacity=1 << 16)
+assert pkg.MicrocircuitBatch(cfgs, **kw).info(0)["blocks"] < 152
+rt.fake_clear()
+rt.fake_alloc_limit(4 * workload.n_neurons(cfgs[0]) * 60)       # less than the table of the runs of 63 partitions
+b = pkg.MicrocircuitBatch(cfgs, **kw)
+assert b.info(0)["blocks"] == 152
+b.step(3)
+assert any("k_batch" in x for x in calls("launch"))
+""")
