@@ -295,6 +295,7 @@ int plan(snn_net* net, const snn_options* opt) {
     const bool few = P <= kFewPartsLimit;
     net->threads = few && net->smem_ring ? step_threads(ncmax) : kStepThreads;
     CK(step_kernel_configure(npt, net->smem_ring, few, net->threads));
+    CK(deliver_configure());
     int per_sm = 0;
     CK(step_max_blocks(npt, net->smem_ring, few, net->threads, net->smem, &per_sm));
     if (per_sm * sms < P)

@@ -102,13 +102,14 @@ size_t cluster_smem(int ncmax) {
 
 }  // namespace
 
+cudaError_t deliver_cluster_configure() { return allow_shared(reinterpret_cast<const void*>(&k_deliver_cluster)); }
+
 cudaError_t deliver_cluster_check(int ncmax, int n_part, int* max_active_clusters) {
     const size_t smem = cluster_smem(ncmax);
     int dev = 0, optin = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     if (e == cudaSuccess && smem > (size_t)optin) e = cudaErrorInvalidConfiguration;
-    if (e == cudaSuccess) e = allow_shared(reinterpret_cast<const void*>(&k_deliver_cluster));
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)((n_part + kCluster - 1) / kCluster * kCluster));
@@ -120,8 +121,6 @@ cudaError_t deliver_cluster_check(int ncmax, int n_part, int* max_active_cluster
 cudaError_t launch_deliver_cluster(const DeliverParams& dp, cudaStream_t s) {
     if (dp.n_spikes <= 0) return cudaSuccess;
     const size_t smem = cluster_smem(dp.ncmax);
-    const cudaError_t e = allow_shared(reinterpret_cast<const void*>(&k_deliver_cluster));
-    if (e != cudaSuccess) return e;
     const int grid = (dp.n_part + kCluster - 1) / kCluster * kCluster;
     k_deliver_cluster<<<grid, kCThreads, smem, s>>>(dp);
     return cudaGetLastError();

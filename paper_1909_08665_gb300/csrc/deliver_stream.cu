@@ -274,6 +274,8 @@ k_deliver_stream(const __grid_constant__ DeliverParams dp, int w_span) {
 
 size_t deliver_stream_smem(int ncmax, int w_span) { return stream_smem(ncmax, w_span).total; }
 
+cudaError_t deliver_stream_configure() { return allow_shared(reinterpret_cast<const void*>(&k_deliver_stream)); }
+
 cudaError_t launch_deliver_stream(const DeliverParams& dp, int w_span, cudaStream_t s) {
     if (dp.n_spikes <= 0) return cudaSuccess;
     if ((long long)kRing * dp.ncmax >= (long long)kPreOffMask || (uint32_t)dp.ncmax > 0xffffu)
@@ -285,8 +287,6 @@ cudaError_t launch_deliver_stream(const DeliverParams& dp, int w_span, cudaStrea
     if (e != cudaSuccess) return e;
     const size_t smem = stream_smem(dp.ncmax, w_span).total;
     if (smem > (size_t)optin) return cudaErrorInvalidConfiguration;
-    e = allow_shared(reinterpret_cast<const void*>(&k_deliver_stream));
-    if (e != cudaSuccess) return e;
     k_deliver_stream<<<dp.n_part, kSThreads, smem, s>>>(dp, w_span);
     return cudaGetLastError();
 }

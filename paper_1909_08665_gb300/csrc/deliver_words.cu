@@ -329,6 +329,11 @@ cudaError_t launch_predecode(const DeliverParams& dp, const unsigned long long* 
     return cudaGetLastError();
 }
 
+cudaError_t deliver_words_configure() {
+    const cudaError_t e = allow_shared(reinterpret_cast<const void*>(&k_deliver_words<true>));
+    return e != cudaSuccess ? e : allow_shared(reinterpret_cast<const void*>(&k_deliver_words<false>));
+}
+
 cudaError_t launch_deliver_words(const DeliverParams& dp, cudaStream_t s) {
     if (dp.n_spikes <= 0) return cudaSuccess;
     int dev = 0, optin = 0;
@@ -340,10 +345,6 @@ cudaError_t launch_deliver_words(const DeliverParams& dp, cudaStream_t s) {
     const bool smem_ring = words_smem(dp.ncmax, true, dp.max_delay).total <= (size_t)optin;
     const size_t smem = words_smem(dp.ncmax, smem_ring, dp.max_delay).total;
     if (smem > (size_t)optin) return cudaErrorInvalidConfiguration;
-    const void* fn = smem_ring ? reinterpret_cast<const void*>(&k_deliver_words<true>)
-                               : reinterpret_cast<const void*>(&k_deliver_words<false>);
-    e = allow_shared(fn);
-    if (e != cudaSuccess) return e;
     if (smem_ring)
         k_deliver_words<true><<<dp.n_part, kWThreads, smem, s>>>(dp);
     else

@@ -378,6 +378,12 @@ int partition_pop_span(const int32_t* part_lo, int n_part, const int32_t* pop_st
 cudaError_t step_kernel_configure(int npt, bool smem_ring, bool few, int threads);
 cudaError_t launch_step(const StepParams& sp, int npt, bool smem_ring, int threads, size_t smem,
                         cudaStream_t s);
+// the delivery kernels' shared-memory limits, raised when a network is made (a
+// call per launch took 1.4 us of each)
+cudaError_t deliver_configure();
+cudaError_t deliver_words_configure();
+cudaError_t deliver_stream_configure();
+cudaError_t deliver_cluster_configure();
 cudaError_t launch_deliver(const DeliverParams& dp, int tiling, cudaStream_t s);
 // stand-alone delivery of the exact row segments of each partition (one CTA
 // per partition, packed words cut into units of <= 32 words, weight table and,

@@ -161,6 +161,14 @@ k_deliver_part(const __grid_constant__ StepParams sp, const uint32_t* __restrict
     if ((tid & 31) == 0 && events) atomicAdd(&sp.counters[1], events);
 }
 
+cudaError_t deliver_configure() {
+    cudaError_t e = allow_shared(reinterpret_cast<const void*>(&k_deliver_part<true>));
+    if (e == cudaSuccess) e = allow_shared(reinterpret_cast<const void*>(&k_deliver_part<false>));
+    if (e == cudaSuccess) e = deliver_words_configure();
+    if (e == cudaSuccess) e = deliver_stream_configure();
+    return e == cudaSuccess ? deliver_cluster_configure() : e;
+}
+
 cudaError_t launch_deliver_part(const StepParams& sp, const uint32_t* spikes, int n, int64_t t,
                                 bool smem_ring, cudaStream_t s) {
     if (n <= 0) return cudaSuccess;
@@ -171,10 +179,6 @@ cudaError_t launch_deliver_part(const StepParams& sp, const uint32_t* spikes, in
     if (e != cudaSuccess) return e;
     smem_ring = smem_ring && part_smem_bytes(sp.ncmax, sp.w_span, true) <= (size_t)optin;
     const size_t smem = part_smem_bytes(sp.ncmax, sp.w_span, smem_ring);
-    const void* fn = smem_ring ? reinterpret_cast<const void*>(&k_deliver_part<true>)
-                               : reinterpret_cast<const void*>(&k_deliver_part<false>);
-    e = allow_shared(fn);
-    if (e != cudaSuccess) return e;
     if (smem_ring)
         k_deliver_part<true><<<sp.n_part, kStepThreads, smem, s>>>(sp, spikes, n, t);
     else
