@@ -662,7 +662,7 @@ struct snn_batch {
     std::vector<snn_net*> nets;          // empty: does not fit
     bool part_fits = false;              // its kernel's CTAs are co-resident
     bool part = false;                   // steps run in this form
-    int part_npt = 0, part_grid = 0;
+    int part_npt = 0, part_grid = 0, part_threads = 0;
     bool part_smem_ring = false, part_few = true;   // few: no instance above kFewPartsLimit partitions
     size_t part_smem = 0, part_ring_words = 0, part_msg_words = 0;
     std::vector<size_t> part_ring_off;   // of each instance, words
@@ -732,7 +732,7 @@ cudaError_t launch_batch(snn_batch* b, int n_steps) {
     if (e == cudaSuccess) e = cudaMemsetAsync(b->d_sync + 2, 0, sizeof(uint32_t), b->stream);
     if (b->part)
         return e != cudaSuccess ? e
-                                : launch_step_multi(b->part_npt, b->part_smem_ring, b->part_few, b->part_smem, b->part_grid,
+                                : launch_step_multi(b->part_npt, b->part_smem_ring, b->part_few, b->part_threads, b->part_smem, b->part_grid,
                                                     b->d_part, b->d_part_first, b->n_inst, b->d_step, n_steps,
                                                     b->stream);
     if (e == cudaSuccess) e = cudaLaunchKernelExC(&cfg, select_batch(b->npt), args);
@@ -986,6 +986,7 @@ int setup_parts(snn_batch* b) {
     const size_t room = (size_t)optin - sizeof(StepParams) - 64;
     b->part_smem_ring = with_ring <= room && b->part_npt <= 2;
     b->part_smem = b->part_smem_ring ? with_ring : bare;
+    b->part_threads = b->part_few && b->part_npt == 1 && b->part_smem_ring ? step_threads(ncmax) : kStepThreads;
     b->part_ring_words = b->part_ring_off[K];
     b->part_msg_words = msg_off[K];
     BCALL(balloc(&b->d_part, K, "batch partitions"));
@@ -1018,7 +1019,7 @@ int setup_parts(snn_batch* b) {
     BCK(cudaMemcpy(b->d_part, sp.data(), sizeof(StepParams) * K, cudaMemcpyHostToDevice));
     BCK(cudaMemcpy(b->d_part_first, first.data(), sizeof(int32_t) * (K + 1), cudaMemcpyHostToDevice));
     int per_sm = 0;
-    BCK(step_multi_configure(b->part_npt, b->part_smem_ring, b->part_few, b->part_smem, &per_sm));
+    BCK(step_multi_configure(b->part_npt, b->part_smem_ring, b->part_few, b->part_threads, b->part_smem, &per_sm));
     b->part = b->part_fits = per_sm * sms >= b->part_grid;
     BCK(reset_state(b));
     return SNN_OK;
@@ -1451,7 +1452,7 @@ int snn_batch_get_info(snn_batch* b, int32_t k, snn_batch_info* info) {
     info->tune_us_flat = b->tune_us[2][k];
     info->trial_us_per_step = b->trial_us;
     info->blocks = b->part ? b->part_grid : b->blocks;
-    info->threads = kBThreads;
+    info->threads = b->part ? b->part_threads : kBThreads;
     info->neurons_per_thread = b->part ? b->part_npt : b->npt;
     info->graph = b->graph_ok ? 1 : 0;
     info->graph_steps = kGraphChunk;

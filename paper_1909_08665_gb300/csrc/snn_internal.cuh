@@ -454,8 +454,8 @@ cudaError_t launch_adjoint_part_fold(int n, int n_part, int n_pop, const int32_t
 // The step kernel over several networks in one launch (step_multi.cu): CTA b
 // runs partition b - first[k] of network k, first[k] <= b < first[k + 1], from
 // step *step on; *step is advanced afterwards.
-cudaError_t step_multi_configure(int npt, bool smem_ring, bool few, size_t smem, int* blocks_per_sm);
-cudaError_t launch_step_multi(int npt, bool smem_ring, bool few, size_t smem, int grid, const StepParams* params,
+cudaError_t step_multi_configure(int npt, bool smem_ring, bool few, int threads, size_t smem, int* blocks_per_sm);
+cudaError_t launch_step_multi(int npt, bool smem_ring, bool few, int threads, size_t smem, int grid, const StepParams* params,
                               const int32_t* first, int n_net, long long* step, int n_steps, cudaStream_t s);
 // stand-alone delivery through the step kernel's runs (one CTA per partition)
 cudaError_t launch_deliver_part(const StepParams& sp, const uint32_t* spikes, int n, int64_t t,

@@ -1,7 +1,8 @@
-"""Batches side by side whose partitions hold more neurons than a CTA has
-threads: two per thread with the ring in shared and in global memory, four and
-eight.  Three networks of one size take 50 partitions each, 150 CTAs, where the
-batch kernel always takes every SM: the number of CTAs tells the form."""
+"""Batches side by side by the size of their partitions: of fewer neurons than 512
+threads, and of more than a CTA has threads (two per thread with the ring in
+shared and in global memory, four and eight).  Three networks of one size take
+up to 50 partitions each, 150 CTAs, where the batch kernel always takes every
+SM: the number of CTAs tells the form."""
 import numpy as np
 import pytest
 
@@ -19,8 +20,10 @@ import paper_1909_08665_gb300 as pkg  # noqa: E402
 # volley: a fifth of one network's neurons start above threshold, more spikes in
 # a step than a delivery list or a CTA's shared-memory record holds
 @pytest.mark.parametrize("volley", [False, True])
-@pytest.mark.parametrize("scale,npt", [(0.4, 2), (0.6, 2), (0.82, 4), (1.6, 8)])
-def test_wide_partitions_match_single_networks(scale, npt, volley):
+@pytest.mark.parametrize("scale,npt,threads", [
+    (0.1, 1, 192), (0.14, 1, 256), (0.2, 1, 352), (0.25, 1, 512),       # small partitions, of fewer threads
+    (0.4, 2, 512), (0.6, 2, 512), (0.82, 4, 512), (1.6, 8, 512)])
+def test_partitions_match_single_networks(scale, npt, threads, volley):
     cfgs = [workload.microcircuit(scale, seed=60 + k) for k in range(3)]
     cfgs[1] = workload.dc_variant(cfgs[1])
     if volley:
@@ -29,7 +32,8 @@ def test_wide_partitions_match_single_networks(scale, npt, volley):
     stream = torch.cuda.current_stream()
     batch = pkg.MicrocircuitBatch(cfgs, stream=stream)
     info = batch.info(0)
-    assert info["blocks"] == 150 and info["neurons_per_thread"] == npt
+    assert info["blocks"] == (147 if scale == 0.1 else 150)
+    assert info["neurons_per_thread"] == npt and info["threads"] == threads
     got = [[] for _ in cfgs]
     for steps in (1, 2, 47):
         batch.step(steps)
@@ -40,7 +44,7 @@ def test_wide_partitions_match_single_networks(scale, npt, volley):
         net = pkg.Microcircuit(cfg, stream=stream)
         net.step(50)
         st, ids = net.read_spikes()
-        assert st.size > (5000 if volley and k == 2 else 100)
+        assert st.size > (5000 * min(1, scale / 0.4) if volley and k == 2 else 100)
         np.testing.assert_array_equal(np.concatenate([g[0] for g in got[k]]), st)
         np.testing.assert_array_equal(np.concatenate([g[1] for g in got[k]]), ids)
         for a, b in zip(batch.state(k), net.state()):
