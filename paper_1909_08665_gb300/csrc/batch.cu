@@ -1077,6 +1077,7 @@ int drain_raster(snn_batch* b) {
         }
         BCK(cudaMemsetAsync(b->d_ras_n, 0, sizeof(uint32_t), b->stream));
         BCK(cudaStreamSynchronize(b->stream));
+        raster_sort_done(&b->ras_sort);
     }
     for (uint32_t r = 0, k = 0; r < m; ++k) {
         const uint32_t lo = (uint32_t)b->goff[k], hi = (uint32_t)b->goff[k + 1];

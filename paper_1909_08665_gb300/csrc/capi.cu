@@ -1009,6 +1009,7 @@ int snn_read_spikes(snn_net* net, uint32_t* steps_host, uint32_t* ids_host, int6
     }
     CK(cudaMemsetAsync(net->d_ras_n, 0, sizeof(uint32_t) * net->P, net->stream));
     CK(cudaStreamSynchronize(net->stream));
+    raster_sort_done(&net->ras_sort);
     net->ras_lo = INT64_MAX;
     net->ras_hi = 0;
     *n = got;

@@ -366,6 +366,10 @@ void raster_sort_free(RasterSort* w) {
     *w = RasterSort();
 }
 
+void raster_sort_done(RasterSort* w) {
+    if (w->step_cap > kSortKeep) raster_sort_free(w);
+}
+
 cudaError_t raster_read_small(const RasterList& in, uint32_t* counts, HostStage* stage, cudaStream_t s,
                               RasterSmall* out) {
     constexpr size_t kHead = 4;

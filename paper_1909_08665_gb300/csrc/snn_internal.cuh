@@ -305,7 +305,8 @@ cudaError_t launch_max_segment(const uint32_t* seg, int n, int n_part, uint32_t*
 // (instance, step, id); n is the sum of the counts, clamped.  Every step lies
 // in [t_lo, t_lo + t_span) modulo 2^32, every id below n_ids; goff (device,
 // [n_inst + 1]) gives the instances' id ranges when there are several.
-// The arrays of w grow as needed and are kept (raster_sort_free).
+// The arrays of w grow as needed and are kept, up to kSortKeep spikes (100 MB):
+// raster_sort_done, called when the result has been copied, frees larger ones.
 struct RasterList {
     const uint32_t* counts;
     const uint32_t* step;
@@ -325,6 +326,8 @@ struct RasterSort {
     size_t step_cap = 0, id_cap = 0, group_cap = 0, key_cap = 0;
 };
 cudaError_t raster_sort(RasterSort* w, const RasterList& in, size_t n, cudaStream_t s);
+constexpr size_t kSortKeep = 1u << 22;
+void raster_sort_done(RasterSort* w);
 // The same on the host, the first `limit` of them into steps / ids (each may be
 // null; goff: the instances' id ranges in host memory): for a device without
 // the 24 bytes per spike that raster_sort takes (cudaErrorMemoryAllocation),

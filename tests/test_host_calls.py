@@ -298,3 +298,22 @@ assert b.info(0)["blocks"] == 152
 b.step(3)
 assert any("k_batch" in x for x in calls("launch"))
 """)
+
+
+def test_arrays_of_a_large_read_are_given_back(run):
+    """What a read sorts in is kept for the next one, up to 100 MB."""
+    run("""
+for make in (lambda: pkg.Microcircuit(workload.microcircuit(0.02), stream=Stream(), raster_capacity=6 << 20, n_part=1),
+             lambda: pkg.MicrocircuitBatch([workload.microcircuit(0.02)] * 2, stream=Stream(), raster_capacity=6 << 20)):
+    h = make()
+    many = [np.empty(5 << 20, np.uint32) for _ in range(2)]
+    read = (lambda: h.read_spikes_into(*many)) if isinstance(h, pkg.Microcircuit) else (lambda: h.read_spikes_into(0, *many))
+    h.step(3)
+    read()
+    for n, kept in ((2 << 20, True), (5 << 20, False), (1 << 20, True)):
+        h.step(3)
+        rt.fake_raster_count()[0] = n
+        assert read() == n
+        assert bool(rt.fake_alloc(4 * n, 1)) == kept and bool(rt.fake_alloc(16 * n, 0)) == kept, n
+    h.close()
+""")
