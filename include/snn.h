@@ -16,6 +16,12 @@
  *  - A handle belongs to the device that was current when it was made.  Reads
  *    (spikes, state, ring, counters, saving and loading) may be called with
  *    any device current; the other calls need the handle's.
+ *  - One handle may be read from several threads, and while another thread
+ *    steps it: the calls take turns, and a step that is issued while a raster is
+ *    read waits until the read is done.  Handles on streams of their own run
+ *    beside one another as far as the SMs hold their partitions
+ *    (snn_info.n_part blocks of snn_info.threads threads; with n_part 0 three of
+ *    up to 192 threads on an SM, two of up to 352, one of 512).
  *  - The library needs an sm_103a GPU; on any other device snn_create()
  *    fails with SNN_ERR_UNSUPPORTED.  There is no CPU fallback.
  *
@@ -213,6 +219,9 @@ int snn_realtime_stats(snn_net* net, int64_t* missed, int64_t* max_late_ns);
  *       load, the analogue of the paper's per-synapse-core count;
  *   [3] (spike, partition) pairs whose row has no synapse onto the partition:
  *       the paper's spike packets that target no neuron of a core.
+ * [2] and [3] are figures of the network's partitions: compare them between
+ * networks, or with a recording made elsewhere, at one n_part (snn_info.n_part;
+ * n_part 0 gives networks below 32,768 neurons up to 64 partitions).
  * Nothing is flushed here (every spike is delivered), so the paper's flushed
  * count is always 0 and is not recorded.  counts_dev is caller-owned device
  * memory (uint32[4 cap]); this call zeroes it on the network's stream.  NULL

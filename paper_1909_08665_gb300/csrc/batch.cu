@@ -850,7 +850,7 @@ int batch_trials(snn_batch* b) {
             }
     }
     // The partitioned form, where the instances fit, is one more candidate;
-    // with one neuron per thread the only one (it takes 1.7 to 2.6 us per step
+    // with one neuron per thread the only one (it takes 1.5 to 2.6 us per step
     // there, a step of the other form never below 5).
     const size_t n_cand = !b->part_fits ? cand.size() : b->part_npt == 1 ? 1 : cand.size() + 1;
     cudaEvent_t e0 = nullptr, e1 = nullptr;

@@ -27,16 +27,17 @@
 // rows of ascending targets give the right result, and rows like the network's
 // own cost one L2 round trip.  What bounds a step is that trip, the message's and the run's,
 // and in large networks the SM's own intake: a probe costs a 32-byte sector,
-// 1 KB per (spike, partition).  Measured, us per step at full size: 64 probes
-// over the whole row 6.07; every word of the window loaded and tested 6.34;
-// 32 probes of the window, four rows per warp at once 5.15, one row 4.48 (16
-// or 8 probes: 4.80, 4.90); 1024 threads 4.13; the count published by the last
-// warp on a barrier of its own 3.91.
+// 1 KB per (spike, partition).  Measured, us per step at full size, in the
+// versions in which each was decided: 64 probes over the whole row 6.07 and
+// every word of the window loaded and tested 6.34, against 5.15 with 32 probes
+// of the window; four rows per warp at once 5.15, one 4.48; 16 or 8 probes 4.80
+// and 4.90, 32 4.48; 512 threads 4.48, 1024 4.13; the count at the CTA barrier
+// 4.13, published by the last warp on a barrier of its own 3.91 (now 3.87).
 //
 // What it replaced, one warp walking each spike's whole row with an L2 atomic
 // per word between two grid barriers, was bound by the chain of a row's
 // dependent loads: 130 us per step at full size, 48 us at the 10 % scale; now
-// 3.91 and 1.69.
+// 3.87 and 1.69.
 //
 // The paper has no counterpart of this entry point.
 #include <algorithm>
@@ -605,7 +606,7 @@ const void* na_kernel(int threads, int ncmax, bool smem_ring) {
 // each where that is possible; networks too small for that are spread to
 // kNaFew neurons per CTA, where the CTA's own work no longer sets the time of
 // a step (a step waits on L2 round trips and barriers, not on the neurons):
-// scale 0.1 with 48 partitions of 161 neurons 2.45 us per step, with 16 of
+// scale 0.1 with 49 partitions of 158 neurons 2.45 us per step, with 16 of
 // 482 2.60, both in the version with 64 probes a row.
 constexpr int kNaFew = 160;
 int na_partitions(long long n, int sms) {

@@ -23,9 +23,9 @@
 //         neuron ids; the Poisson background count of step t is drawn.
 //         The warps only arrive at the barrier that completes the count, and
 //         go on; the last warp waits at it and publishes the count.  (With a
-//         CTA barrier there, the count waited for the warps that had to have
+//         CTA barrier there, the count waits for the warps that have to have
 //         the other partitions' message heads first: us per step at scale
-//         0.02 1.72, 0.1 1.78, 4 14.6; so 1.64, 1.73 and 12.7.  With one
+//         0.02 1.51, 1.3 3.18, 4 7.93; so 1.45, 3.04 and 7.74.  With one
 //         neuron per thread and more than kFewParts partitions the CTA
 //         barrier is the faster one, see PUB_EARLY.)
 //   D     wait for every partition's message of step t-1 (each word carries
@@ -58,9 +58,8 @@ namespace snn {
 constexpr uint32_t kStatusRasterOverflow = 2u;
 // Ids read together with a message header: INL = 7 (64 bytes), or 3 (32 bytes)
 // where there are few partitions (kFewParts) and hardly ever more spikes in
-// one.  us per step with 7 / 3: scale 0.02 1.54 / 1.49, 0.1 1.63 / 1.59, 0.37
-// (57 partitions) 1.97 / 1.91, 0.6 (91) 2.21 / 2.36, 1 (151) 2.60 / 2.87 (with 7
-// now 2.14 and 2.56, see PUB_EARLY).
+// one.  us per step with 7 / 3: scale 0.02 1.54 / 1.45, 0.1 1.60 / 1.50, 0.37
+// (64 partitions, DC) 1.80 / 1.73, 0.6 (91) 2.13 / 2.29, 1 (151) 2.53 / 2.81.
 constexpr int kInline = 7;
 constexpr int kInlineFew = 3;
 constexpr int kFewParts = kFewPartsLimit;
@@ -68,10 +67,9 @@ constexpr int kFewParts = kFewPartsLimit;
 // entries of each of their runs in one wave (runs: mean 26 entries at scale 1
 // and 4, rarely above 96).  The spikes are dealt round-robin over the warps,
 // and each warp loads its next batch before the adds of the current one.  us
-// per step by shape (spikes x waves), full size: 2 x 3 2.57, 3 x 3 2.62, 2 x 2
-// 2.66, 4 x 3 2.70, 1 x 3 2.75, two batches ahead 2.66; 4x (4 neurons per
-// thread): 2 x 3 8.23, 3 x 3 8.26, and in contiguous batches without the early
-// load 4 x 3 8.53, 6 x 3 8.66, 8 x 3 9.01, 8 x 2 9.74.
+// per step by shape (spikes x waves), full size: 2 x 3 2.53, 3 x 3 2.58, 2 x 2
+// 2.63, 1 x 3 2.73; 1.3x (2 neurons per thread): 3.04, 3.11, 3.14, 3.29; 4x (4
+// neurons): 7.74, 8.34, 7.89, 8.18.
 constexpr int kBatchSpikes = 2;
 constexpr int kRunWave = 3;
 constexpr uint32_t kPopWords = kMaxPop * kWCodes;   // weight-table entries per target population
@@ -555,13 +553,13 @@ __device__ __forceinline__ void step_body(const StepParams& sp, const int c, uns
     constexpr bool PACED = (MODE & kModePaced) != 0;
     constexpr bool SAT = (MODE & kModeSat) != 0;
     // early run lookups keep 2 x INL more registers live until the delivery:
-    // not in the widest variant (us per step without / with: 1.3x 3.44 / 3.12,
-    // 2x 4.78 / 4.46, 4x 8.23 / 8.15)
+    // not in the widest variant (us per step without / with: 1.3x 3.40 / 3.04,
+    // 2x 4.67 / 4.30, 4x 8.09 / 7.74)
     constexpr bool EARLY = NPT <= 4;
     // the count published ahead of the CTA barrier, or at it: with one neuron
     // per thread and many partitions the header warps are the slow ones either
     // way, and they gain from the others' wait (us per step ahead / at it:
-    // scale 0.6 2.16 / 2.14, 1 2.59 / 2.56)
+    // scale 0.6 2.17 / 2.13, 1 2.55 / 2.53)
     constexpr bool PUB_EARLY = NPT > 1 || INL == kInlineFew;
     const int tid = threadIdx.x;
     const int lane = tid & 31;
@@ -707,9 +705,11 @@ __device__ __forceinline__ void step_body(const StepParams& sp, const int c, uns
         // have to be drained by the host between launches).  The publishing
         // thread asks for the spikes' place in it, its warp writes them at the
         // end of the step, when that has arrived.  us per step with lists of
-        // their own / one list: 5 networks of 13,072 neurons 1.57 / 1.63, 12 of
-        // 70,900 1.77 / 1.80, 16 of 187,168 4.96 / 4.76, 32 of 376,261 11.0 /
-        // 10.8; with an atomic per spiking warp 1.78, 1.88, 4.78, 11.0.
+        // their own / one list: 5 networks of 13,072 neurons 1.57 / 1.63 (with
+        // 512 threads; 1.57 with 192), 12 of 70,900 1.77 / 1.80, 16 of 187,168
+        // 4.96 / 4.76, 32 of 376,261 11.0 / 10.8; with an atomic per spiking
+        // warp 1.78, 1.88, 4.78, 11.0.  (Single networks keep a list per
+        // partition: one list costs them 0.04 to 0.5 us.)
         uint32_t rec_at = 0u;
         auto record = [&]() {
             if (!MULTI || tid < kPublisher) return;
@@ -754,10 +754,9 @@ __device__ __forceinline__ void step_body(const StepParams& sp, const int c, uns
         // the run bounds of the step t-1 spikes whose message words this
         // header thread already holds (the head loaded before A(t), arrived
         // by now): with several neurons per thread looked up here, so that
-        // they return during the background draws (4x 7.99 us per step with
-        // the lookups after them, 7.72 before); with one the draw is short and
-        // the heads may still be on their way (scale 0.1 1.57 before it, 1.56
-        // after)
+        // they return during the background draws (4x 0.27 us per step more
+        // with the lookups after them); with one the draw is short and the
+        // heads may still be on their way (scale 0.1 0.01 us more before it)
         EarlyRuns<INL> early;
         early.ok = false;
         const bool look_up = EARLY && s > 0 && tid < P;
@@ -806,8 +805,8 @@ __device__ __forceinline__ void step_body(const StepParams& sp, const int c, uns
         // ---- C(t): ring slot t, Poisson background, synaptic current ----
         const uint32_t slot = (uint32_t)t & (kRing - 1);
         // all of the thread's cells are in flight before the first is cleared
-        // (one after the other, their L2 round trips made C(t) 3 us of the 4x
-        // network's step: 12.7 us per step, now 9.0; 2x 8.4, now 5.3)
+        // (one after the other, their L2 round trips cost 3.7 us of a 4x step,
+        // 3.1 of a 2x step)
         int32_t cells[NPT];
 #pragma unroll
         for (int k = 0; k < NPT; ++k) {

@@ -5,8 +5,8 @@
 // only for one another: there is no barrier over the batch.  A step takes what
 // it takes the largest of the networks alone, where the batch kernel's step
 // costs a grid barrier and four dependent trips to L2 (5 networks of 13,072
-// neurons: 6.59 us per step, here 1.64; 12 of 70,900: 8.6 and 1.83; 16 of
-// 187,168, four neurons per thread: 9.9 and 5.1).
+// neurons: 6.59 us per step, here 1.57; 12 of 70,900: 8.6 and 1.80; 16 of
+// 187,168, four neurons per thread: 9.9 and 4.8).
 #include "step_kernel.cuh"
 
 namespace snn {
