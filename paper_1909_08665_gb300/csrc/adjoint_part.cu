@@ -430,6 +430,17 @@ __global__ void __launch_bounds__(256) k_adjoint_part_fold(int32_t n, int32_t n_
 
 }  // namespace
 
+bool adjoint_part_possible(int n_part, int ncmax, uint64_t nnz) {
+    int dev = 0, sms = 0, optin = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess)
+        return false;
+    const int G = sms / std::max(1, n_part);
+    // each CTA's share of the rows must fit next to the window and the tables
+    return G >= 1 && ncmax <= kApPre * kApThreads && (double)nnz * 4.0 / ((double)n_part * G) <= (double)optin * 0.7;
+}
+
 int adjoint_part_plan(int n, int n_pop, const int32_t* pop_start, int n_part, const int32_t* part_lo,
                       int ncmax, uint64_t nnz, const unsigned long long* d_row_start,
                       const uint32_t* d_pre, const uint32_t* d_seg, AdjPartPlan* plan) {
@@ -439,10 +450,8 @@ int adjoint_part_plan(int n, int n_pop, const int32_t* pop_start, int n_part, co
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess)
         return -1;
-    const int G = sms / std::max(1, n_part);
-    if (G < 1 || ncmax > kApPre * kApThreads || n <= 0) return 1;
-    // each CTA's share of the rows must fit next to the window and the tables
-    if ((double)nnz * 4.0 / ((double)n_part * G) > (double)optin * 0.7) return 1;
+    if (n <= 0 || !adjoint_part_possible(n_part, ncmax, nnz)) return 1;
+    const int G = sms / n_part;
     std::vector<unsigned long long> rs(n + 1);
     std::vector<uint32_t> pre(nnz), seg((size_t)n * (n_part + 1));
     if (cudaMemcpy(rs.data(), d_row_start, sizeof(unsigned long long) * (n + 1), cudaMemcpyDeviceToHost) != cudaSuccess ||

@@ -591,15 +591,16 @@ int snn_grad_backward(snn_net* net, const double* g_rate, double* g_alpha, doubl
 
     if (!g->part_planned) {
         // the partition-local gather when every CTA's share of the rows fits
-        // in shared memory
-        AdjPartPlan plan;
+        // in shared memory, and the device has room for what it takes
         std::vector<int32_t> lo(PA + 1);
+        g->part_ncmax = 0;
         for (int c = 0; c <= PA; ++c) {
             lo[c] = (int32_t)(((long long)c * n) / PA);
             if (c) g->part_ncmax = std::max(g->part_ncmax, lo[c] - lo[c - 1]);
         }
         GCALL(galloc(&g->part_lo, PA + 1, "adjoint partitions"));
         GCK(cudaMemcpy(g->part_lo, lo.data(), sizeof(int32_t) * (PA + 1), cudaMemcpyHostToDevice));
+        int rc = adjoint_part_possible(PA, g->part_ncmax, net->nnz) ? SNN_OK : SNN_ERR_OOM;
         // the rows cut and decoded for these partitions, where they are not
         // the step kernel's
         uint32_t *seg = net->d_seg, *pre = net->d_pre;
@@ -614,30 +615,31 @@ int snn_grad_backward(snn_net* net, const double* g_rate, double* g_alpha, doubl
             for (int p = 0; p <= kMaxPop; ++p) dp.pop_start[p] = net->pop_start[p];
             dp.part_lo = g->part_lo;
             dp.words = net->d_words;
-            int rc = galloc(&seg, (size_t)n * (PA + 1) + 4, "adjoint row segments");
+            if (rc == SNN_OK) rc = galloc(&seg, (size_t)n * (PA + 1) + 4, "adjoint row segments");
             if (rc == SNN_OK) rc = galloc(&pre, (size_t)net->nnz + 4, "adjoint rows");
             cudaError_t e = cudaSuccess;
             if (rc == SNN_OK) e = launch_seg_from_rows(net->d_row_start, net->d_words, n, g->part_lo, PA, seg, s);
             if (rc == SNN_OK && e == cudaSuccess) e = launch_predecode(dp, net->d_row_start, pre, s);
             if (rc == SNN_OK && e == cudaSuccess) e = cudaStreamSynchronize(s);
             if (rc == SNN_OK && e != cudaSuccess) rc = set_cuda_error(e, "adjoint rows");
-            if (rc != SNN_OK) {
-                cudaFree(seg);
-                cudaFree(pre);
-                return rc;
-            }
         }
-        const int rc = adjoint_part_plan(n, net->n_pop, net->pop_start, PA, lo.data(), g->part_ncmax,
-                                         net->nnz, net->d_row_start, pre, seg, &plan);
+        AdjPartPlan plan;
+        int fits = 1;
+        if (rc == SNN_OK)
+            fits = adjoint_part_plan(n, net->n_pop, net->pop_start, PA, lo.data(), g->part_ncmax, net->nnz,
+                                     net->d_row_start, pre, seg, &plan);
         if (PA != P) {
             cudaFree(seg);
             cudaFree(pre);
         }
-        if (rc < 0) return set_error(SNN_ERR_CUDA, "partition-local adjoint plan");
-        if (rc == 0) {
-            g->part = new AdjPartPlan(plan);
-            GCALL(galloc(&g->pds, (size_t)2 * PA * n, "adjoint partials"));
-            GCALL(galloc(&g->gAc, (size_t)PA * n * kMaxPop, "gradient partials"));
+        if (rc != SNN_OK && rc != SNN_ERR_OOM) return rc;
+        if (fits < 0) return set_error(SNN_ERR_CUDA, "partition-local adjoint plan");
+        if (fits == 0) {
+            if (galloc(&g->pds, (size_t)2 * PA * n, "adjoint partials") == SNN_OK &&
+                galloc(&g->gAc, (size_t)PA * n * kMaxPop, "gradient partials") == SNN_OK)
+                g->part = new AdjPartPlan(plan);
+            else
+                adjoint_part_free(&plan);
         }
         g->part_planned = true;
     }

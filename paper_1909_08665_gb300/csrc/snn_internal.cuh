@@ -445,6 +445,8 @@ struct AdjPartPlan {
     uint32_t* d_img = nullptr;
     uint32_t* d_img_off = nullptr;   // [grid + 1]
 };
+// whether a network of so many synapses can fit at all
+bool adjoint_part_possible(int n_part, int ncmax, uint64_t nnz);
 // 0: planned; 1: the network does not fit (use the global gather); < 0: error
 int adjoint_part_plan(int n, int n_pop, const int32_t* pop_start, int n_part, const int32_t* part_lo,
                       int ncmax, uint64_t nnz, const unsigned long long* d_row_start,

@@ -317,3 +317,37 @@ for make in (lambda: pkg.Microcircuit(workload.microcircuit(0.02), stream=Stream
         assert bool(rt.fake_alloc(4 * n, 1)) == kept and bool(rt.fake_alloc(16 * n, 0)) == kept, n
     h.close()
 """)
+
+
+def test_first_gradients_decode_rows_only_where_they_can_fit(run):
+    """The rows are cut and decoded for the adjoint's partitions only where the
+    partition-local form is possible, and it is done without where there is no
+    room for that."""
+    run("""
+rng = np.random.default_rng(2)
+
+
+def backward(per_row, limit=1 << 40):
+    cfg = workload.microcircuit(0.12)
+    n = workload.n_neurons(cfg)
+    rp = np.arange(n + 1) * per_row
+    targets = np.sort(rng.integers(0, n, (n, per_row)), 1).astype(np.uint32).ravel()
+    net = pkg.Microcircuit(cfg, stream=Stream(), raster_capacity=1 << 16,
+                           rows={"row_ptr": rp, "words": targets | np.uint32(1 << 19),
+                                 "wtab": np.ones((8, 8, 128), np.int32)})
+    assert net.info()["n_part"] > -(-n // 512)
+    net.grad_forward(4, 2)
+    rt.fake_clear()
+    rt.fake_alloc_limit(limit)
+    net.grad_backward(np.ones(8))
+    rt.fake_alloc_limit(1 << 40)
+    decoded = [x for x in calls("malloc") if int(x.split()[-1]) == 4 * (n * per_row + 4)]
+    kernel = [x.split()[1] for x in calls("launch") if "k_adjoint" in x and "fold" not in x][-1]
+    net.close()
+    return len(decoded), "k_adjoint_part" in kernel
+
+
+assert backward(300) == (1, True)
+assert backward(1000) == (0, False)             # 246 KB of rows for every CTA
+assert backward(300, 8 << 20) == (1, False)     # tried, no room for 11 MB
+""")
